@@ -1064,6 +1064,25 @@ static RescoreArgs rescore_args(const KernelSpec& sp, const BlockBufs& b, int64_
   return R;
 }
 
+// Scratch of the tensor-core loop's re-score (see RescoreArgs), sized for the
+// largest mini-batch; one loop of a fit runs at a time, so one set serves all.
+static kkm_status alloc_tc_rescore(Workspace& ws, int64_t Nmax, int64_t nLmax, int C, RescoreArgs* t) {
+  t->ldc32 = round_up(nLmax, 32);
+  // one allocation, 256-byte aligned parts
+  const int64_t have = round_up(Nmax * tc_rescore_blocks((int)nLmax) * 32, 64);
+  const int64_t vals = round_up(Nmax * t->ldc32, 64);
+  KKM_TRY(ws.alloc(&t->have, have + vals + ceil_div(Nmax, 128) * tc_rescore_list_words(C, (int)nLmax)));
+  t->C32 = reinterpret_cast<float*>(t->have + have);
+  t->lists = t->have + have + vals;
+  return KKM_OK;
+}
+static void use_tc_rescore(const RescoreArgs& t, RescoreArgs* R) {
+  R->C32 = t.C32;
+  R->ldc32 = t.ldc32;
+  R->have = t.have;
+  R->lists = t.lists;
+}
+
 // Whether the inner iterations of a mini-batch run fused (one cooperative
 // launch each) for this option and block shape.
 // Inner-loop forms (kkm_iteration): the split pair of launches per
@@ -1505,6 +1524,11 @@ static kkm_status fit_impl(const float* X_in, int64_t N, int64_t d, int32_t C, i
   KKM_TRY(alloc_loop(ws, (int)nLmax, C, ldk, trace_cap, &lb, sp.gaussian()));
   Supports& S = lb.S;
   IterState& I = lb.I;
+  RescoreArgs tc_scratch;
+  for (const BatchGeom* g : {&geo.front(), &geo.back()})  // mini-batches come in at most two sizes
+    if (!tc_scratch.lists &&
+        loop_form(opt.iteration, sp, bm, (int)g->Ni, (int)n_landmarks(g->Ni, s), C) == kLoopTc)
+      KKM_TRY(alloc_tc_rescore(ws, Nmax, nLmax, C, &tc_scratch));
   if (from) {
     // the outer loop's state after mini-batch start - 1: medoids, counts, the
     // trace and the displacements so far
@@ -1663,8 +1687,12 @@ static kkm_status fit_impl(const float* X_in, int64_t N, int64_t d, int32_t C, i
     KKM_RUN("build_supports", ms, launch_build_supports(S, ms));
     I.keep_rows = kt_half ? l2_keep_rows(ldk, nL, kL2KeepShareHalf, 2) : l2_keep_rows(ldk, nL, kL2KeepShare, 4);
     I.flag_tau = bm.flag_tau(sp);
-    const RescoreArgs R = rescore_args(sp, bk, ldk);
+    RescoreArgs R = rescore_args(sp, bk, ldk);
     const int form = loop_form(opt.iteration, sp, bm, Ni, nL, C);
+    if (form == kLoopTc) {
+      if (!tc_scratch.lists) return invalid("internal: no re-score scratch");
+      use_tc_rescore(tc_scratch, &R);
+    }
     if (form < 0)
       return invalid(opt.iteration == KKM_ITER_TC
                          ? "KKM_ITER_TC does not apply to this shape (RBF with KKM_BF16 or KKM_FP8, C <= 16, at most "
@@ -2142,9 +2170,14 @@ static kkm_status debug_step_impl(const float* Xb_in, int64_t Ni, int64_t d, con
   const float* kself = sp.kind == KKM_LINEAR ? b.aux_i : nullptr;
   lb.I.keep_rows = 0;
   lb.I.flag_tau = bm.flag_tau(sp);
-  const RescoreArgs R = rescore_args(sp, b, ldk);
+  RescoreArgs R = rescore_args(sp, b, ldk);
   const int form = loop_form(iteration, sp, bm, (int)Ni, nL, C);
   if (form < 0) return invalid("the iteration form asked for does not apply to this shape");
+  if (form == kLoopTc) {
+    RescoreArgs t;
+    KKM_TRY(alloc_tc_rescore(ws, Ni, nL, C, &t));
+    use_tc_rescore(t, &R);
+  }
   KKM_TRY(inner_loop(bm, b, ldk, (int)Ni, lb.S, lb.I, form, 1, kself, u, mg, fh, gh, 0, R, st));
   if (u_out) KKM_CK(cudaMemcpyAsync(u_out, u, (size_t)Ni * 4, cudaMemcpyDeviceToHost, st));
   if (fhat_out) KKM_CK(cudaMemcpyAsync(fhat_out, fh, (size_t)Ni * C * 4, cudaMemcpyDeviceToHost, st));

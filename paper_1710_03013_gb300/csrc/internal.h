@@ -397,7 +397,22 @@ struct RescoreArgs {
   // reads them instead of recomputing them from the rows
   const float* K32 = nullptr;
   int64_t ldk32 = 0;
+  // scratch of the tensor-core loop: the FP32 values it has formed so far
+  // ([sample][ldc32], by the landmark's place), a bit per (sample, landmark)
+  // that says so ([sample][tc_rescore_blocks(nL)][32 words]), and per CTA the
+  // clusters' landmark lists and the landmarks' places
+  float* C32 = nullptr;
+  int64_t ldc32 = 0;
+  uint32_t* have = nullptr;
+  uint32_t* lists = nullptr;
 };
+// Blocks of 1,024 landmarks of the re-score bits, and 4-byte words of a CTA's
+// candidate sets (128), rounds (32), distances (128 x 16), lists, places and
+// cluster bits.
+__host__ __device__ constexpr int tc_rescore_blocks(int nL) { return (nL + 1023) / 1024; }
+__host__ __device__ constexpr int64_t tc_rescore_list_words(int C, int nL) {
+  return 160 + 128 * 16 + (int64_t)(C + 1) * ((nL + 31) / 32) * 32 + (int64_t)C * tc_rescore_blocks(nL) * 32;
+}
 
 // f_hat, distances, argmin, margin, Omega; updates u in place.  With
 // trace == 1 the last CTA also writes the trace entry, the early-stop flag and

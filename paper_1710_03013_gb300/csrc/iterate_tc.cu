@@ -97,9 +97,10 @@ struct TcIterShared {
   double tot_om;
   int tot_ch, tot_lm;
   int ok;
+  int any_flagged;  // a row of the tile is a near tie in this iteration
 };
 
-static_assert(sizeof(TcIterShared) <= 1280, "static shared memory beside the dynamic share");
+static_assert(sizeof(TcIterShared) <= 1024, "static shared memory beside the dynamic share");
 
 // Barrier of the epilogue warps only (named barrier 1), after the warp has
 // reconverged.
@@ -140,10 +141,347 @@ __device__ __forceinline__ uint32_t z_offset(int k, int n) {
                     (kk & 7) * 2);
 }
 
+
+// ------------------------------------------------------ near-tie re-score
+// A flagged row (two or more clusters within the low-precision window) gets
+// f_hat of every candidate cluster from exact FP32 kernel values of its
+// support.  Neither the rows nor the landmarks change between iterations, so
+// a value is formed once per launch and kept: R.C32[i][place of k] beside one
+// bit per (sample, landmark) that says whether it is there.  An iteration
+// then costs a gather and a sum; only rows that were never near this tie
+// before, and landmarks that moved into a candidate cluster, cost dot
+// products.
+//
+// Lists: per cluster, the landmarks of each lane (k = lane mod 32) in index
+// order, [round][lane], a copy per CTA, made from Z when a row is flagged and
+// landmark labels have moved since.  A lane adds its values in that order and
+// the warp adds the lanes in a fixed tree: the sums of a scan over all
+// landmarks, bit for bit.  The place of a landmark in a row of C32 is its
+// rank by cluster when the first list was made, so the values a row needs lie
+// together (in [landmark][sample] order a 32-byte sector held one value of
+// use, and the gathers pushed the block out of L2).
+//
+// The dot products: the CTA's rows with one candidate set are taken kRsRows
+// at a time, the missing landmarks spread over the four warps, one to a lane;
+// they are bound by the latency of their loads from L2 (no shared memory is
+// left for tiles), which the rows of a group share.
+//
+// MNIST-shaped fit with C = 12 (classes split, a quarter of the rows flagged
+// in each of 120 iterations): 1,024 ms when every iteration formed every
+// value again, a row at a time, against 7.6 ms.
+constexpr int kRsRows = 8;          // rows of a group sharing the landmark loads
+constexpr int kRsSumRows = 4;       // rows of a group sharing the list loads
+constexpr uint32_t kRsNone = 0xffffffffu;
+
+// 32 bytes of a row that no one writes during the launch.
+__device__ __forceinline__ void ld_row8(const float* p, float (&v)[8]) {
+  asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+      : "l"(p));
+}
+// The lists of the warp's clusters from the one-hot tiles (an entry is the
+// landmark and its place in a row of C32); `first` also sets the places.
+__device__ __forceinline__ void rescore_lists(const uint8_t* Z, int nL, int C, const int* nj, uint32_t* __restrict__ list,
+                                              uint32_t* place, uint32_t* bits, uint32_t* rounds, bool first, int ew,
+                                              int lane) {
+  const int nS = (nL + 31) >> 5, nblk = tc_rescore_blocks(nL);
+  for (int j = ew; j < C; j += kTcEpiWarps) {
+    uint32_t* const lj = list + (int64_t)j * nS * 32 + lane;
+    int n = 0;
+    uint32_t in_block = 0;
+    for (int s0 = 0; s0 < nS; s0 += 4) {
+      unsigned short z[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int k = (s0 + t) * 32 + lane;
+        z[t] = k < nL ? *reinterpret_cast<const unsigned short*>(Z + z_offset(k, j)) : (unsigned short)0;
+      }
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+        if (z[t]) {
+          lj[32 * n++] = (uint32_t)((s0 + t) * 32 + lane);
+          in_block |= 1u << ((s0 + t) & 31);
+        }
+      if (((s0 + 4) & 31) == 0 || s0 + 4 >= nS) {
+        bits[(j * nblk + (s0 >> 5)) * 32 + lane] = in_block;
+        in_block = 0;
+      }
+    }
+    int at = n;  // inclusive prefix over the lanes
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(kFull, at, o);
+      if (lane >= o) at += y;
+    }
+    at -= n;
+    for (int q = 0; q < j; ++q) at += nj[q];
+    const int most = (int)__reduce_max_sync(kFull, (unsigned)n);
+    for (int m = 0; m < most; ++m) {
+      uint32_t e = kRsNone;
+      if (m < n) {
+        const uint32_t k = lj[32 * m];
+        if (first) place[k] = (uint32_t)(at + m);
+        e = k | (first ? (uint32_t)(at + m) : place[k]) << 16;
+      }
+      lj[32 * m] = e;
+    }
+    if (lane == 0) rounds[j] = (uint32_t)most;
+  }
+}
+
+// FP32 kernel values of N rows and landmark row xl (squared norm nl, sample
+// id own) into out[row * ldo]: dot products in chunks of 32 products, the
+// order of the FP32 block.  Rows are x0 + r * dp for the N bytes r of rows; i0
+// is the sample of row 0.
+template <int N>
+__device__ __forceinline__ void rescore_values(const float* __restrict__ xl, float nl, int own,
+                                            const float* __restrict__ x0, const float* __restrict__ nx0, int i0,
+                                            uint2 rows, int dp, float neg_scale, float* __restrict__ out, int64_t ldo) {
+  const float* xi[N];
+  float dot[N], part[N];
+  auto row = [&](int r) { return (int)(((r < 4 ? rows.x : rows.y) >> (8 * (r & 3))) & 255u); };
+#pragma unroll
+  for (int r = 0; r < N; ++r) {
+    xi[r] = x0 + (int64_t)row(r) * dp;
+    dot[r] = part[r] = 0.0f;
+  }
+  const int n8 = dp >> 3;
+#pragma unroll 2
+  for (int c = 0; c < n8; ++c) {
+    float b[8];
+    ld_row8(xl + c * 8, b);
+#pragma unroll
+    for (int r = 0; r < N; ++r) {
+      float a[8];
+      ld_row8(xi[r] + c * 8, a);
+      part[r] = fmaf(a[0], b[0], fmaf(a[1], b[1], fmaf(a[2], b[2], fmaf(a[3], b[3], part[r]))));
+      part[r] = fmaf(a[4], b[4], fmaf(a[5], b[5], fmaf(a[6], b[6], fmaf(a[7], b[7], part[r]))));
+    }
+    if ((c & 3) == 3) {
+#pragma unroll
+      for (int r = 0; r < N; ++r) {
+        dot[r] += part[r];
+        part[r] = 0.0f;
+      }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < N; ++r) {
+    dot[r] += part[r];
+    out[row(r) * ldo] =
+        own == i0 + row(r) ? 1.0f : exp2f(fmaxf(nx0[row(r)] + nl - 2.0f * dot[r], 0.0f) * neg_scale);
+  }
+}
+
+// Forms the values of the clusters cmask that one of the N rows i[] misses
+// (all four warps; the bits are set after they have all read them).
+template <int N>
+__device__ __forceinline__ void rescore_fill(const RescoreArgs& R, const int32_t* __restrict__ L, int nL,
+                                             const uint32_t* bits, const uint32_t* place, unsigned cmask, int ew,
+                                             int lane, int i0, const int (&i)[kRsRows]) {
+  const int nblk = tc_rescore_blocks(nL);
+  uint2 rows = make_uint2(0u, 0u);  // the rows of the tile, a byte each
+#pragma unroll
+  for (int r = 0; r < N; ++r) (r < 4 ? rows.x : rows.y) |= (uint32_t)(i[r] - i0) << (8 * (r & 3));
+  auto wanted = [&](int b) -> uint32_t {  // the lane's landmarks of the candidate clusters in block b
+    uint32_t want = 0;
+    for (unsigned c = cmask; c; c &= c - 1) want |= bits[((__ffs(c) - 1) * nblk + b) * 32 + lane];
+    return want;
+  };
+  int b = -1, turn = 0;
+  uint32_t miss = 0;
+  bool some = false;
+  while (true) {
+    int k = -1;
+    while (true) {
+      while (miss == 0 && ++b < nblk) {
+        const uint32_t want = wanted(b);
+#pragma unroll
+        for (int r = 0; r < N; ++r) miss |= want & ~R.have[((int64_t)i[r] * nblk + b) * 32 + lane];
+        some |= miss != 0;
+      }
+      if (miss == 0) break;
+      const int p = __ffs(miss) - 1;
+      miss &= miss - 1;
+      if ((turn++ & (kTcEpiWarps - 1)) == ew) {  // the warps take the lane's missing values in turn
+        k = b * 1024 + p * 32 + lane;
+        break;
+      }
+    }
+    if (!__any_sync(kFull, k >= 0)) break;
+    if (k >= 0) {
+      float* const out = R.C32 + (int64_t)i0 * R.ldc32 + place[k];
+      if (R.K32) {  // the block's own FP32 values
+#pragma unroll
+        for (int r = 0; r < N; ++r) out[(i[r] - i0) * R.ldc32] = __ldg(R.K32 + (int64_t)k * R.ldk32 + i[r]);
+      } else {
+        rescore_values<N>(R.XL + (int64_t)k * R.dp, R.nXL[k], L[k], R.Xi + (int64_t)i0 * R.dp, R.nXi + i0, i0, rows,
+                          R.dp, R.neg_scale, out, R.ldc32);
+      }
+    }
+    __syncwarp();
+  }
+  if (!__any_sync(kFull, some)) return;  // nothing is missing (the same in every warp)
+  epi_sync();
+  for (int r = ew; r < N; r += kTcEpiWarps) {
+    int row = i[0];
+#pragma unroll
+    for (int q = 1; q < N; ++q)
+      if (q == r) row = i[q];
+    for (int bb = 0; bb < nblk; ++bb) R.have[((int64_t)row * nblk + bb) * 32 + lane] |= wanted(bb);
+  }
+  epi_sync();
+}
+
+// The first rows of the CTA's tile left in cq (cq[w]: the candidate set of row
+// 32 w + lane, 0 when done) that share one set: up to M of them, taken out of
+// cq; returns how many (0: none left).  The last one is repeated.
+template <int M>
+__device__ __forceinline__ int rescore_group(unsigned (&cq)[kTcEpiWarps], int i0, int lane, unsigned* cmask,
+                                             int (&ri)[M]) {
+  unsigned cm = 0;
+#pragma unroll
+  for (int w = kTcEpiWarps - 1; w >= 0; --w) {
+    const unsigned some = __ballot_sync(kFull, cq[w] != 0);
+    const unsigned c = __shfl_sync(kFull, cq[w], some ? __ffs(some) - 1 : 0);
+    if (some) cm = c;
+  }
+  *cmask = cm;
+  if (!cm) return 0;
+  int n = 0;
+#pragma unroll
+  for (int r = 0; r < M; ++r) ri[r] = i0;
+#pragma unroll
+  for (int w = 0; w < kTcEpiWarps; ++w) {
+    unsigned same = __ballot_sync(kFull, cq[w] == cm);
+    while (same && n < M) {
+      const int l = __ffs(same) - 1;
+      same &= same - 1;
+      if (lane == l) cq[w] = 0;
+#pragma unroll
+      for (int r = 0; r < M; ++r)
+        if (r >= n) ri[r] = i0 + 32 * w + l;
+      ++n;
+    }
+  }
+  return n;
+}
+
+// The re-score of one iteration, by the four epilogue warps (one row of the
+// tile to a thread): the distances of the row's candidate clusters (cand; 0:
+// the row is not flagged) into the CTA's scratch, [128][kTcN].  state: the
+// clusters of the row whose values are all there, kRsFresh when landmark
+// labels have moved since the last call, kRsFirst before the first one; the
+// new state is returned.  Not inlined, so that the loop keeps its registers
+// and its code stays together (inlined, an iteration without a near tie took
+// 0.2 us longer).
+constexpr unsigned kRsFresh = 1u << 16, kRsFirst = 1u << 17;
+
+__device__ __noinline__ unsigned rescore_step(const TcIterShared& sh, const uint8_t* Z, const int32_t* __restrict__ L,
+                                              int nL, int C, const RescoreArgs& R, int i0, int rows, unsigned cand,
+                                              unsigned state) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int ew = warp - 2 * kTcRings, q = warp & 3, et = threadIdx.x - 2 * kTcRings * 32;
+  const int nS = (nL + 31) >> 5, nblk = tc_rescore_blocks(nL);
+  uint32_t* const cands = R.lists + (int64_t)blockIdx.x * tc_rescore_list_words(C, nL);
+  uint32_t* const rounds = cands + 128;
+  float* const dist = reinterpret_cast<float*>(rounds + 32) + q * 32 * kTcN;  // of the warp's rows
+  uint32_t* const list = rounds + 32 + 128 * kTcN;
+  uint32_t* const place = list + (int64_t)C * nS * 32;
+  uint32_t* const bits = place + nS * 32;
+  const float ks = 1.0f;
+  unsigned full = state & 0xffffu;
+  if (state & kRsFresh) {
+    const bool first = (state & kRsFirst) != 0;
+    if (first) {  // no value of the tile's rows is there yet
+      const int quads = rows * nblk * 8;
+      uint4* const h4 = reinterpret_cast<uint4*>(R.have + (int64_t)i0 * nblk * 32);
+      for (int x = et; x < quads; x += kTcEpiWarps * 32) h4[x] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    rescore_lists(Z, nL, C, sh.nj, list, place, bits, rounds, first, ew, lane);
+    full = 0;
+  }
+  // the rows with a candidate cluster whose values may not all be there: the
+  // same groups, in the same order, in every warp
+  cands[q * 32 + lane] = (cand & ~full) ? cand : 0u;
+  full |= cand;
+  epi_sync();
+  {
+    unsigned cq[kTcEpiWarps], cmask;
+#pragma unroll
+    for (int w = 0; w < kTcEpiWarps; ++w) cq[w] = cands[32 * w + lane];
+    int ri[kRsRows];
+    while (const int n = rescore_group(cq, i0, lane, &cmask, ri)) {
+      if (n > 1) rescore_fill<kRsRows>(R, L, nL, bits, place, cmask, ew, lane, i0, ri);
+      else rescore_fill<1>(R, L, nL, bits, place, cmask, ew, lane, i0, ri);
+    }
+  }
+  // sums: up to kRsSumRows rows of the warp with one candidate set, two
+  // clusters at a time, so that 32 gathers are in flight
+  for (unsigned todo = __ballot_sync(kFull, cand != 0); todo;) {
+    const unsigned cmask = __shfl_sync(kFull, cand, __ffs(todo) - 1);
+    unsigned same = __ballot_sync(kFull, cand == cmask) & todo;
+    int rl[kRsSumRows];  // their lanes (the last one repeated)
+    const float* row_c[kRsSumRows];
+#pragma unroll
+    for (int r = 0; r < kRsSumRows; ++r) {
+      rl[r] = same ? __ffs(same) - 1 : rl[r ? r - 1 : 0];
+      same &= same - 1;
+      todo &= ~(1u << rl[r]);
+      row_c[r] = R.C32 + (int64_t)(i0 + q * 32 + rl[r]) * R.ldc32;
+    }
+    for (unsigned c = cmask; c;) {
+      const int j0 = __ffs(c) - 1;
+      c &= c - 1;
+      const int j1 = c ? __ffs(c) - 1 : -1;
+      c &= c - 1;
+      const uint32_t* l0 = list + (int64_t)j0 * nS * 32 + lane;
+      const uint32_t* l1 = list + (int64_t)(j1 < 0 ? 0 : j1) * nS * 32 + lane;
+      const int n0 = (int)rounds[j0], n1 = j1 < 0 ? 0 : (int)rounds[j1];
+      float a0[kRsSumRows], a1[kRsSumRows];
+#pragma unroll
+      for (int r = 0; r < kRsSumRows; ++r) a0[r] = a1[r] = 0.0f;
+      for (int m = 0; m < n0 || m < n1; m += 4) {
+        float v0[4][kRsSumRows], v1[4][kRsSumRows];
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+          const uint32_t e0 = m + x < n0 ? l0[32 * (m + x)] : kRsNone;
+          const uint32_t e1 = m + x < n1 ? l1[32 * (m + x)] : kRsNone;
+#pragma unroll
+          for (int r = 0; r < kRsSumRows; ++r) {
+            v0[x][r] = e0 != kRsNone ? row_c[r][e0 >> 16] : 0.0f;
+            v1[x][r] = e1 != kRsNone ? row_c[r][e1 >> 16] : 0.0f;
+          }
+        }
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+          for (int r = 0; r < kRsSumRows; ++r) {
+            a0[r] += v0[x][r];
+            a1[r] += v1[x][r];
+          }
+      }
+#pragma unroll
+      for (int r = 0; r < kRsSumRows; ++r) {
+        const float f0 = warp_sum_f32(a0[r]), f1 = warp_sum_f32(a1[r]);
+        const float d0 = ks - 2.0f * (f0 / (float)sh.nj[j0]) + sh.ghf[j0];
+        const float d1 = j1 < 0 ? 0.0f : ks - 2.0f * (f1 / (float)sh.nj[j1]) + sh.ghf[j1];
+        if (lane == 0) {
+          dist[rl[r] * kTcN + j0] = d0;
+          if (j1 >= 0) dist[rl[r] * kTcN + j1] = d1;
+        }
+      }
+    }
+  }
+  __syncwarp();
+  return full;
+}
+
 __global__ void __launch_bounds__(kTcThreads, 1)
 iterate_tc_kernel(const __grid_constant__ CUtensorMap map, int Ni, Supports S, IterState I, int iters, int nstages,
                   int32_t* __restrict__ u, float* __restrict__ margin, float* __restrict__ fhat_out,
-                  double* __restrict__ ghat_out, int early_stop, RescoreArgs R, unsigned long long* __restrict__ keys,
+                  double* __restrict__ ghat_out, int early_stop, const __grid_constant__ RescoreArgs R,
+                  unsigned long long* __restrict__ keys,
                   int32_t* __restrict__ kcount, double* __restrict__ ghat_final) {
   extern __shared__ __align__(1024) uint8_t tc_smem_raw[];
   uint8_t* const base =
@@ -175,6 +513,7 @@ iterate_tc_kernel(const __grid_constant__ CUtensorMap map, int Ni, Supports S, I
     sh.verdict = kVerdictSame;
     sh.abort_flag = 0;
     sh.stop = 0;
+    sh.any_flagged = 0;
     sh.never = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -349,6 +688,7 @@ iterate_tc_kernel(const __grid_constant__ CUtensorMap map, int Ni, Supports S, I
     const double gscale = ldexp(1.0, I.gfix_shift), oscale = ldexp(1.0, I.fom_shift);
     const float tau = I.flag_tau;
     const bool rescore = R.Xi != nullptr && tau > 0.0f;
+    unsigned rs_state = kRsFresh | kRsFirst;
 
     // Z and the cluster sizes from the landmark labels: Z zeroed, then a one
     // (0x3C00) at (label, landmark) for every landmark, the labels of eight
@@ -431,13 +771,13 @@ iterate_tc_kernel(const __grid_constant__ CUtensorMap map, int Ni, Supports S, I
       epi_sync();
       if (et == 0) tc_grid_arrive(I.bar);  // grid barrier A: arrive now, wait after the work that needs no g_hat
       target += gridDim.x;
-      // e_ij = K_ii - 2 f_hat_ij (Eq. 15 without g_hat)
-      float e[kTcN];
+      // K_ii - 2 f_hat_ij (Eq. 15 without g_hat)
+      float d[kTcN];
 #pragma unroll
       for (int j = 0; j < kTcN; ++j) {
         const int n = j < C ? sh.nj[j] : 0;
         const float fh = n > 0 ? D[j] / (float)n : __int_as_float(0x7fc00000);
-        e[j] = n > 0 ? ks - 2.0f * fh : inf;
+        d[j] = n > 0 ? ks - 2.0f * fh : inf;
         if (fhat_out && valid && j < C) fhat_out[(int64_t)i * C + j] = fh;
       }
       if (et == 0) sh.ok = tc_grid_wait(I.bar, target, I.err) ? 1 : 0;
@@ -462,12 +802,11 @@ iterate_tc_kernel(const __grid_constant__ CUtensorMap map, int Ni, Supports S, I
       epi_sync();
       if (blockIdx.x == 0 && ghat_out && et < C) ghat_out[et] = sh.gh[et];
       // 4. distances and argmin (lowest j on ties)
-      float d[kTcN];
       float best = inf, second = inf;
       int bj = 0;
 #pragma unroll
       for (int j = 0; j < kTcN; ++j) {
-        d[j] = e[j] < inf ? e[j] + sh.ghf[j < C ? j : 0] : inf;
+        if (d[j] < inf) d[j] += sh.ghf[j < C ? j : 0];
         if (d[j] < best) {
           second = best;
           best = d[j];
@@ -478,92 +817,70 @@ iterate_tc_kernel(const __grid_constant__ CUtensorMap map, int Ni, Supports S, I
       }
       const float scale = ks + sh.ghf[bj];
       const bool flagged = valid && rescore && second < inf && (second - best) < tau * fmaxf(fabsf(second), scale);
-      // 5. near-tie re-score: every candidate cluster of a flagged row gets
-      // f_hat from exact FP32 kernel values of its support (one landmark per
-      // lane in index order, dot products in chunks of 32 products, then a
-      // fixed xor tree); one flagged row at a time per warp
-      unsigned fm = __ballot_sync(kFull, flagged);
-      while (fm) {
-        const int L = __ffs(fm) - 1;
-        fm &= fm - 1;
-        const float bL = __shfl_sync(kFull, best, L), sL = __shfl_sync(kFull, scale, L);
-        const int iL = i0 + q * 32 + L;
-        const float4* xi = reinterpret_cast<const float4*>(R.Xi + (int64_t)iL * R.dp);
-        const float ni = R.nXi[iL];
-        unsigned cmask = 0;  // the row's candidate clusters
-#pragma unroll
-        for (int j = 0; j < kTcN; ++j) {
-          const float dj = __shfl_sync(kFull, d[j], L);
-          if (j < C && sh.nj[j] > 0 && dj - bL < tau * fmaxf(fabsf(dj), sL)) cmask |= 1u << j;
+      // 5. labels, the changed landmarks, cost and counts
+      auto settle = [&]() {
+        const bool ch = valid && bj != cur;
+        if (ch && cord >= 0) {
+          S.lab[cord] = bj;
+          const int idx = (int)atomicAdd(facc + (t & 1) * (C + 3) + C + 2, 1ull);
+          I.lm_list[(size_t)(t & 1) * nL + idx] = (cord << 8) | (cur << 4) | bj;
         }
-        while (cmask) {
-          const int j = __ffs(cmask) - 1;
-          cmask &= cmask - 1;
-          float accr = 0.0f;
-          for (int k = lane; k < nL; k += 32) {
-            if (*reinterpret_cast<const unsigned short*>(Z + z_offset(k, j)) == 0) continue;
-            if (R.K32) {  // the block's own FP32 values
-              accr += __ldg(R.K32 + (int64_t)k * R.ldk32 + iL);
-              continue;
-            }
-            const float4* xl = reinterpret_cast<const float4*>(R.XL + (int64_t)k * R.dp);
-            float dot = 0.0f, part = 0.0f;
-            for (int c = 0; c < (R.dp >> 2); ++c) {
-              const float4 a4 = __ldg(xi + c), b4 = __ldg(xl + c);
-              part = fmaf(a4.x, b4.x, fmaf(a4.y, b4.y, fmaf(a4.z, b4.z, fmaf(a4.w, b4.w, part))));
-              if ((c & 7) == 7) {
-                dot += part;
-                part = 0.0f;
-              }
-            }
-            dot += part;
-            accr += (S.L[k] == iL) ? 1.0f : exp2f(fmaxf(ni + R.nXL[k] - 2.0f * dot, 0.0f) * R.neg_scale);
-          }
-          accr = warp_sum_f32(accr);
-          const float dn = ks - 2.0f * (accr / (float)sh.nj[j]) + sh.ghf[j];
-#pragma unroll
-          for (int jj = 0; jj < kTcN; ++jj)
-            if (jj == j && lane == L) d[jj] = dn;
+        // the cost share as a fixed-point integer (two's complement: a slightly
+        // negative d near 0 adds correctly), summed per warp, then per CTA
+        unsigned long long om = 0ull;
+        if (valid) {
+          cur = bj;
+          if (margin) margin[i] = second - best;
+          if (best < inf) om = (unsigned long long)llrint((double)best * oscale);
         }
-      }
-      if (flagged) {
-        best = inf;
-        second = inf;
-        bj = 0;
 #pragma unroll
-        for (int j = 0; j < kTcN; ++j) {
-          if (d[j] < best) {
-            second = best;
-            best = d[j];
-            bj = j;
-          } else if (d[j] < second) {
-            second = d[j];
-          }
+        for (int o = 16; o > 0; o >>= 1) om += __shfl_xor_sync(kFull, om, o);
+        const int chw = (int)__reduce_add_sync(kFull, ch ? 1u : 0u);
+        if (lane == 0) {
+          sh.osum_w[warp - 2 * kTcRings] = om;
+          sh.chsum_w[warp - 2 * kTcRings] = chw;
         }
-      }
-      // 6. labels, the changed landmarks, cost and counts
-      const bool ch = valid && bj != cur;
-      if (ch && cord >= 0) {
-        S.lab[cord] = bj;
-        const int idx = (int)atomicAdd(facc + (t & 1) * (C + 3) + C + 2, 1ull);
-        I.lm_list[(size_t)(t & 1) * nL + idx] = (cord << 8) | (cur << 4) | bj;
-      }
-      // the cost share as a fixed-point integer (two's complement: a slightly
-      // negative d near 0 adds correctly), summed per warp, then per CTA
-      unsigned long long om = 0ull;
-      if (valid) {
-        cur = bj;
-        if (margin) margin[i] = second - best;
-        if (best < inf) om = (unsigned long long)llrint((double)best * oscale);
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) om += __shfl_xor_sync(kFull, om, o);
-      const int chw = (int)__reduce_add_sync(kFull, ch ? 1u : 0u);
-      if (lane == 0) {
-        sh.osum_w[warp - 2 * kTcRings] = om;
-        sh.chsum_w[warp - 2 * kTcRings] = chw;
-      }
+      };
+      // 6. a warp with a near tie settles after the re-score, which all the
+      // warps do together: every candidate cluster of a flagged row gets
+      // f_hat from exact FP32 kernel values of its support
+      const bool tie = __any_sync(kFull, flagged);
+      if (!tie) settle();
+      else if (lane == 0) sh.any_flagged = 1;
       epi_sync();
+      if (sh.any_flagged) {
+        unsigned cand = 0;  // the row's candidate clusters
+        if (flagged) {
+#pragma unroll
+          for (int j = 0; j < kTcN; ++j)
+            if (j < C && sh.nj[j] > 0 && d[j] - best < tau * fmaxf(fabsf(d[j]), scale)) cand |= 1u << j;
+        }
+        rs_state = rescore_step(sh, Z, S.L, nL, C, R, i0, min(128, Ni - i0), cand, rs_state);
+        if (flagged) {
+          const float* const dn = reinterpret_cast<const float*>(
+                                      R.lists + (int64_t)blockIdx.x * tc_rescore_list_words(C, nL) + 160) +
+                                  row * kTcN;
+#pragma unroll
+          for (int j = 0; j < kTcN; ++j)
+            if (cand >> j & 1u) d[j] = dn[j];
+          best = inf;
+          second = inf;
+          bj = 0;
+#pragma unroll
+          for (int j = 0; j < kTcN; ++j) {
+            if (d[j] < best) {
+              second = best;
+              best = d[j];
+              bj = j;
+            } else if (d[j] < second) {
+              second = d[j];
+            }
+          }
+        }
+        if (tie) settle();
+        epi_sync();
+        if (et == 0) sh.any_flagged = 0;
+      }
       if (et == 0) {  // grid barrier B
         unsigned long long o = 0ull;
         int c = 0;
@@ -608,6 +925,7 @@ iterate_tc_kernel(const __grid_constant__ CUtensorMap map, int Ni, Supports S, I
           atomicSub(&sh.nj[from], 1);
           atomicAdd(&sh.nj[to], 1);
         }
+        rs_state |= kRsFresh;
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       }
       epi_sync();
@@ -635,17 +953,22 @@ iterate_tc_kernel(const __grid_constant__ CUtensorMap map, int Ni, Supports S, I
               failed = true;
               break;
             }
-            tc_fence_after();
-            float Df[kTcN];
+          }
+          // (the last iteration's sums are still in tensor memory: reading them
+          // again costs less than 16 registers throughout the loop)
+          const int par = (final_pass ? t : t - 1) & 1;
+          tc_fence_after();
+          float Df[kTcN];
 #pragma unroll
-            for (int j = 0; j < kTcN; ++j) Df[j] = 0.0f;
-            for (int r = 0; r < active; ++r) {
-              uint32_t v[16];
-              tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(((t & 1) * kTcRings + r) * kTcN), v);
+          for (int j = 0; j < kTcN; ++j) Df[j] = 0.0f;
+          for (int r = 0; r < active; ++r) {
+            uint32_t v[16];
+            tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)((par * kTcRings + r) * kTcN), v);
 #pragma unroll
-              for (int j = 0; j < kTcN; ++j) Df[j] += __uint_as_float(v[j]);
-            }
-            tc_fence_before();
+            for (int j = 0; j < kTcN; ++j) Df[j] += __uint_as_float(v[j]);
+          }
+          tc_fence_before();
+          if (final_pass) {
             epi_sync();
             if (et == 0) *stop_flag = 1;  // the producers may wind down
             if (valid && cord >= 0) {
@@ -664,11 +987,6 @@ iterate_tc_kernel(const __grid_constant__ CUtensorMap map, int Ni, Supports S, I
             epi_sync();
             if (et == 0) tc_grid_arrive(I.bar);
             target += gridDim.x;
-#pragma unroll
-            for (int j = 0; j < kTcN; ++j) {
-              const int n = j < C ? sh.nj[j] : 0;
-              e[j] = n > 0 ? ks - 2.0f * (Df[j] / (float)n) : inf;
-            }
             if (et == 0) sh.ok = tc_grid_wait(I.bar, target, I.err) ? 1 : 0;
             epi_sync();
             if (!sh.ok) {
@@ -685,7 +1003,8 @@ iterate_tc_kernel(const __grid_constant__ CUtensorMap map, int Ni, Supports S, I
           if (valid) {
 #pragma unroll
             for (int j = 0; j < kTcN; ++j)
-              if (j < C && sh.nj[j] > 0) atomicMin(&sh.kbest[j], pack_key(e[j], (uint32_t)i));
+              if (j < C && sh.nj[j] > 0)
+                atomicMin(&sh.kbest[j], pack_key(ks - 2.0f * (Df[j] / (float)sh.nj[j]), (uint32_t)i));
             atomicAdd(&sh.kcnt[cur], 1);
           }
           epi_sync();
@@ -761,6 +1080,8 @@ cudaError_t launch_iterate_tc(const __half* KT, int64_t ldk, int Ni, const Suppo
   int nstages = 0;
   size_t smem = 0;
   if (!tc_iter_shape(Ni, S.nL, S.C, n_sms, &nstages, &smem)) return cudaErrorInvalidValue;
+  if (R.Xi && I.flag_tau > 0.0f && (!R.lists || !R.C32 || !R.have || R.dp % 8 != 0 || S.nL > 0xffff))
+    return cudaErrorInvalidValue;
   if (!I.facc || !I.lm_list || !I.bar || !I.err || (ldk * 2) % 16 != 0 ||
       (reinterpret_cast<uintptr_t>(KT) & 15) != 0)
     return cudaErrorInvalidValue;
