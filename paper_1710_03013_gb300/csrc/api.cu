@@ -727,6 +727,30 @@ static kkm_status kernel_block_fp8(const KernelSpec& sp, const float* P, const i
   return KKM_OK;
 }
 
+// Scratch of the FP32 Gaussian block on the tensor cores, one allocation: the
+// slices, scales and (unless given) norms of nP references and nQ samples, and
+// two zeroed words (pipeline error, a row with NaN or Inf).
+static kkm_status alloc_split(Workspace& ws, const KernelSpec& sp, int64_t nP, int64_t nQ, SplitRows* P, SplitRows* Q,
+                              int** word) {
+  auto part = [](int64_t bytes) { return round_up(bytes, 256); };
+  char* at;
+  KKM_TRY(ws.alloc(&at, 256 + part(6 * nP * sp.dp) + part(6 * nQ * sp.dp) + 2 * part(4 * nP) + 2 * part(4 * nQ)));
+  KKM_CK(cudaMemsetAsync(at, 0, 8, ws.st));
+  auto take = [&](int64_t bytes) {
+    char* const p = at;
+    at += part(bytes);
+    return p;
+  };
+  *word = reinterpret_cast<int*>(take(8));
+  for (SplitRows* s : {P, Q}) {
+    const int64_t n = s == P ? nP : nQ;
+    s->v = reinterpret_cast<__half*>(take(6 * n * sp.dp));
+    s->scale = reinterpret_cast<float*>(take(4 * n));
+    if (s->form_norm) s->norm = reinterpret_cast<float*>(take(4 * n));
+  }
+  return KKM_OK;
+}
+
 int l2_keep_rows(int64_t ldk, int rows, double share, int elem_bytes) {
   static const int l2 = []() {
     int dev = 0, v = 0;
@@ -1955,9 +1979,24 @@ static kkm_status assign_impl(const kkm_model* m, const float* Xnew_in, int64_t 
   const int64_t budget_floats = (int64_t)1 << 27;  // 512 MB of kernel values per chunk
   const int64_t chunk = std::max<int64_t>(1024, std::min<int64_t>(M, budget_floats / std::max(rows_ref, 1)));
   const int64_t ldm = round_up(std::min(chunk, M), 32);
-  float *Xc, *auxc, *Kb;
-  KKM_TRY(ws.alloc(&Xc, ldm * sp.dp));
-  KKM_TRY(ws.alloc(&auxc, ldm));
+  float *Xc = nullptr, *auxc, *Kb;
+  // the FP32 Gaussian block on the tensor cores (kkm_cost keeps the FFMA block,
+  // so that costs compare bit for bit with those of the fits' own kernels)
+  const bool split = !omega_out && split_applies(sp.kind, rows_ref, d) && 3 * ldm <= INT32_MAX;
+  SplitRows SP, SX;
+  int* split_err = nullptr;
+  if (split) {
+    const bool sup = mode == KKM_ASSIGN_SUPPORTS;
+    SP.X = sup ? m->sup : m->med;
+    SP.ld = sp.dp;
+    SP.norm = sup ? m->sup_aux : m->med_aux;
+    SP.form_norm = false;
+    SX.ld = d;
+    KKM_TRY(alloc_split(ws, sp, rows_ref, std::min(chunk, M), &SP, &SX, &split_err));
+  } else {
+    KKM_TRY(ws.alloc(&Xc, ldm * sp.dp));
+    KKM_TRY(ws.alloc(&auxc, ldm));
+  }
   KKM_TRY(ws.alloc(&Kb, (int64_t)rows_ref * ldm));
   const float* kself = sp.kind == KKM_LINEAR ? auxc : nullptr;
   RmsdTcScratch rtc;
@@ -1985,17 +2024,27 @@ static kkm_status assign_impl(const kkm_model* m, const float* Xnew_in, int64_t 
   }
   for (int64_t c0 = 0; c0 < M; c0 += chunk) {
     const int n = (int)std::min<int64_t>(chunk, M - c0);
-    KKM_TRY(prep_rows(sp, X, c0, 1, n, Xc, auxc, st));
+    if (split) {
+      SX.X = X + c0 * d;
+      KKM_RUN("split_rows", st,  // the references with the first chunk
+              launch_split_rows(SP, c0 == 0 ? rows_ref : 0, SX, n, d, sp.dp, nullptr, st));
+      KKM_RUN("gram_split", st,
+              launch_gram_split(SP, rows_ref, SX, n, sp.dp, sp.neg_scale(), Kb, ldm, split_err, sm_count(), st));
+    } else {
+      KKM_TRY(prep_rows(sp, X, c0, 1, n, Xc, auxc, st));
+      if (mode == KKM_ASSIGN_SUPPORTS)
+        KKM_TRY(kernel_block(sp, m->sup, m->sup_aux, nullptr, m->nL, Xc, auxc, nullptr, n, Kb, ldm, st, false, false,
+                             use_rtc ? &rtc : nullptr));
+      else
+        KKM_TRY(kernel_block(sp, m->med, m->med_aux, nullptr, C, Xc, auxc, nullptr, n, Kb, ldm, st, false, false,
+                             use_rtc ? &rtc : nullptr));
+    }
     if (mode == KKM_ASSIGN_SUPPORTS) {
-      KKM_TRY(kernel_block(sp, m->sup, m->sup_aux, nullptr, m->nL, Xc, auxc, nullptr, n, Kb, ldm, st, false, false,
-                           use_rtc ? &rtc : nullptr));
       KKM_RUN("fhat_partial", st, launch_fhat_partial(Kb, ldm, n, lb.S, lb.I, st));
       KKM_RUN("assign", st,
               launch_assign(ldm, n, lb.S, lb.I, kself, lab + c0, nullptr, dist + c0, nullptr, nullptr, 0,
                             /*rebuild=*/0, st));
     } else {
-      KKM_TRY(kernel_block(sp, m->med, m->med_aux, nullptr, C, Xc, auxc, nullptr, n, Kb, ldm, st, false, false,
-                           use_rtc ? &rtc : nullptr));
       KKM_RUN("nearest", st,
               launch_nearest(Kb, ldm, n, C, kself, sp.kind == KKM_LINEAR ? m->med_aux : nullptr, lab + c0,
                              dist + c0, st));
@@ -2013,10 +2062,12 @@ static kkm_status assign_impl(const kkm_model* m, const float* Xnew_in, int64_t 
   if (dist_host) KKM_CK(cudaMemcpyAsync(dist_out, dist, (size_t)M * 4, cudaMemcpyDeviceToHost, st));
   int rtc_err_h = 0;
   if (use_rtc) KKM_CK(cudaMemcpyAsync(&rtc_err_h, rtc.err, 4, cudaMemcpyDeviceToHost, st));
+  if (split) KKM_CK(cudaMemcpyAsync(&rtc_err_h, split_err, 4, cudaMemcpyDeviceToHost, st));
   KKM_CK(cudaStreamSynchronize(st));
   prof_collect();
   if (rtc_err_h) {
-    set_error("tensor-core MD estimate: a bounded pipeline wait gave up");
+    set_error(split ? "tensor-core kernel block: a bounded pipeline wait gave up"
+                    : "tensor-core MD estimate: a bounded pipeline wait gave up");
     return KKM_ETIMEOUT;
   }
   return KKM_OK;
@@ -2046,12 +2097,34 @@ static kkm_status kernel_matrix_impl(const float* A_in, int64_t nA, const float*
   KKM_TRY(device_input(ws, A_in, nA * d, &A));
   KKM_TRY(device_input(ws, B_in, nB * d, &Bm));
   float *Ap, *Bp, *aA, *aB, *o;
+  const bool host_out = !is_device_ptr(out);
+  if (host_out) KKM_TRY(ws.alloc(&o, nA * nB)); else o = out;
+  if (precision == KKM_FP32 && split_applies(sp.kind, nA, d) && 3 * nB <= INT32_MAX) {
+    SplitRows SA, SB;
+    int* word;
+    int word_h[2] = {0, 0};
+    SA.X = A;
+    SB.X = Bm;
+    SA.ld = SB.ld = d;
+    KKM_TRY(alloc_split(ws, sp, nA, nB, &SA, &SB, &word));
+    KKM_RUN("split_rows", st, launch_split_rows(SA, nA, SB, nB, d, sp.dp, word + 1, st));
+    KKM_RUN("gram_split", st,
+            launch_gram_split(SA, nA, SB, nB, sp.dp, sp.neg_scale(), o, nB, word, sm_count(), st));
+    if (host_out) KKM_CK(cudaMemcpyAsync(out, o, (size_t)nA * nB * 4, cudaMemcpyDeviceToHost, st));
+    KKM_CK(cudaMemcpyAsync(word_h, word, 8, cudaMemcpyDeviceToHost, st));
+    KKM_CK(cudaStreamSynchronize(st));
+    prof_collect();
+    if (word_h[0]) {
+      set_error("tensor-core kernel block: a bounded pipeline wait gave up");
+      return KKM_ETIMEOUT;
+    }
+    if (!word_h[1]) return KKM_OK;
+    // rows with NaN or Inf have no slices: the FFMA kernel below gives their values
+  }
   KKM_TRY(ws.alloc(&Ap, nA * sp.dp));
   KKM_TRY(ws.alloc(&Bp, nB * sp.dp));
   KKM_TRY(ws.alloc(&aA, nA));
   KKM_TRY(ws.alloc(&aB, nB));
-  const bool host_out = !is_device_ptr(out);
-  if (host_out) KKM_TRY(ws.alloc(&o, nA * nB)); else o = out;
   KKM_TRY(prep_rows(sp, A, 0, 1, nA, Ap, aA, st));
   KKM_TRY(prep_rows(sp, Bm, 0, 1, nB, Bp, aB, st));
   int tc_err_h = 0;

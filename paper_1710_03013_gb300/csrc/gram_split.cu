@@ -1,0 +1,410 @@
+// The FP32 Gaussian kernel block on the tensor cores (tcgen05): FP32 rows in
+// three 9-bit slices, products exact where it matters.
+//
+//   out[n][m] = exp(-max(0, |p|^2 + |q|^2 - 2 p.q) / (2 sigma^2))
+//
+// Every row is scaled by a power of two so that its largest |value| lies in
+// [2^14, 2^15), and a scaled value is cut into hi + mid + lo, multiples of
+// 2^7, 2^-2 and 2^-11 with at most 256 steps each (27 bits below the row's
+// maximum; FP16 holds each slice exactly, all normal numbers).  The product
+// p.q is then six FP16 products: hi.hi, hi.mid, mid.hi, mid.mid, hi.lo and
+// lo.hi (the three left out are below 2^-27 of the maxima).
+//
+// Accuracy: a tensor-core accumulator drops the bits below its last place at
+// every step, which would bias a long FP32 sum by parts in 10^6.  hi.hi is
+// kept exact instead: its products are multiples of 2^14 of at most 2^16
+// steps, so 256 of them stay below 2^24 steps and no bit is dropped; every
+// 256 values of K the epilogue adds the accumulator to FP32 sums in registers
+// (rounded to nearest).  The other five products share a second accumulator
+// whose total is about 2^-9 of the first, and so are its dropped bits.
+// Measured against 64 bits (relative error of a block; FFMA kernel in
+// brackets): k/255 features of 784 values 8.3e-8 (9.1e-8), blobs 4.1e-8
+// (4.2e-8), blobs 100 from the origin 1.6e-5 (2.4e-5).
+//
+// What bounds it: six FP16 products of 2 d flop per entry.  At 784 values a
+// 3,001 x 15,013 block takes 0.293 ms (1.45 PFLOP/s of FP16 products, 0.76 of
+// the measured BF16 rate) against 1.57 ms for the FFMA kernel (45 of the 74
+// TFLOP/s that independent FFMAs reach).
+//
+// Structure (persistent, one CTA of ten warps per SM, 128 samples x 256
+// references): warp 0 fills three 72 KB stages by TMA (32 values of K, the
+// three slices of both sides, 64-byte swizzle), warp 1 issues the MMAs, warps
+// 2..9 drain and finish.  hi.hi has tensor-memory columns 0..255, the rest
+// 256..511.  In a stage the ten MMAs of the second accumulator go first, so
+// the drain of the first one runs beside them; running totals live in
+// registers (128 per epilogue thread), so the next tile's MMAs start when the
+// accumulators are read, before the exponentials and the stores.
+// Every wait is bounded, as in the BF16 block.
+#include <cuda.h>
+#include <cuda_fp16.h>
+
+#include <algorithm>
+
+#include "device_common.cuh"
+#include "internal.h"
+#include "tc_common.cuh"
+
+namespace kkm {
+
+constexpr int SP_M = 128;
+constexpr int SP_K = 32;                         // values of K per stage (64-byte rows)
+constexpr int SP_STAGES = 3;
+constexpr int SP_A_BYTES = SP_M * SP_K * 2;      // a slice of the sample tile
+constexpr int SP_CHUNK = 256 / SP_K;             // stages whose hi.hi products sum exactly
+constexpr int SP_THREADS = 320;
+// N references per tile: 256, or 64 when tiles of 256 would leave half of the
+// SMs idle (a few samples: one tile's 25 stages of d = 784 are then a chain of
+// 10 us on a few SMs, against 3 us).  An entry's sums do not depend on N.
+template <int N>
+struct SpCfg {
+  static constexpr int kBBytes = N * SP_K * 2;   // a slice of the reference tile
+  static constexpr int kStageBytes = 3 * (SP_A_BYTES + kBBytes);
+  static constexpr size_t kSmem = (size_t)SP_STAGES * kStageBytes + 1024;
+  static constexpr int kTmemCols = 2 * N;
+};
+
+// kind::f16, FP32 accumulator, F16 A and B, both K-major.
+__host__ __device__ constexpr uint32_t sp_idesc(int n) {
+  return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(SP_M >> 4) << 24);
+}
+// K-major operand tile of 64-byte rows with the 64-byte swizzle (8-row atoms,
+// 512 bytes apart).
+__device__ __forceinline__ uint64_t sw64_desc(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
+  d |= (uint64_t)1 << 16;
+  d |= (uint64_t)(512 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)4 << 61;
+  return d;
+}
+
+struct SplitShared {
+  uint64_t full[SP_STAGES], empty[SP_STAGES];
+  uint64_t hfull, hempty;  // hi.hi sums of a chunk ready / read
+  uint64_t rempty;         // the other products' sums of a tile read
+  uint32_t tmem_base;
+  int abort_flag;
+  float nP[8][128], sP[8][128];  // norms and scales of a warp's references
+};
+
+template <int SP_N>
+__global__ void __launch_bounds__(SP_THREADS, 1)
+gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapP, int nQ, int nP,
+                  int dk, const float* __restrict__ normQ, const float* __restrict__ normP,
+                  const float* __restrict__ scaleQ, const float* __restrict__ scaleP, float neg_scale,
+                  float* __restrict__ out, int64_t ldo, int* __restrict__ err) {
+  constexpr int SP_B_BYTES = SpCfg<SP_N>::kBBytes, SP_STAGE_BYTES = SpCfg<SP_N>::kStageBytes;
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  uint8_t* const stages = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  __shared__ SplitShared sh;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int tiles_m = (nQ + SP_M - 1) / SP_M, tiles_n = (nP + SP_N - 1) / SP_N;
+  const int n_tiles = tiles_m * tiles_n;
+  const int nk = (dk + SP_K - 1) / SP_K;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < SP_STAGES; ++s) {
+      mbar_init(&sh.full[s], 1);
+      mbar_init(&sh.empty[s], 1);
+    }
+    mbar_init(&sh.hfull, 1);
+    mbar_init(&sh.hempty, 8);
+    mbar_init(&sh.rempty, 8);
+    sh.abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    tmem_alloc(&sh.tmem_base, SpCfg<SP_N>::kTmemCols);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = sh.tmem_base;
+
+  if (warp == 0) {
+    // ---------------- TMA producer
+    if (lane == 0) {
+      int s = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
+        const int tm = t % tiles_m, tn = t / tiles_m;
+        for (int kb = 0; kb < nk; ++kb) {
+          if (!mbar_wait(&sh.empty[s], ph ^ 1u, &sh.abort_flag)) {
+            ok = false;
+            break;
+          }
+          uint8_t* const a = stages + (size_t)s * SP_STAGE_BYTES;
+          uint8_t* const b = a + 3 * SP_A_BYTES;
+          mbar_expect_tx(&sh.full[s], SP_STAGE_BYTES);
+          // slice v of row r is row v * n + r of the slice array
+#pragma unroll
+          for (int v = 0; v < 3; ++v) {
+            tma_load_2d(&mapQ, &sh.full[s], a + v * SP_A_BYTES, kb * SP_K, v * nQ + tm * SP_M);
+            tma_load_2d(&mapP, &sh.full[s], b + v * SP_B_BYTES, kb * SP_K, v * nP + tn * SP_N);
+          }
+          if (++s == SP_STAGES) {
+            s = 0;
+            ph ^= 1u;
+          }
+        }
+      }
+      if (!ok) {
+        atomicExch(err, 1);
+        sh.abort_flag = 1;
+      }
+    }
+  } else if (warp == 1) {
+    // ---------------- MMA issuer
+    if (lane == 0) {
+      int s = 0;
+      uint32_t ph = 0, hph = 1, rph = 1;  // parities of the next "read" waits
+      bool ok = true;
+      const uint32_t idesc = sp_idesc(SP_N);
+      const uint32_t dh = tmem, dr = tmem + SP_N;
+      for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
+        for (int kb = 0; kb < nk; ++kb) {
+          if (!mbar_wait(&sh.full[s], ph, &sh.abort_flag) ||
+              (kb == 0 && !mbar_wait(&sh.rempty, rph, &sh.abort_flag))) {
+            ok = false;
+            break;
+          }
+          if (kb == 0) rph ^= 1u;
+          tc_fence_after();
+          const uint32_t a = smem_u32(stages + (size_t)s * SP_STAGE_BYTES);
+          const uint32_t b = a + 3 * SP_A_BYTES;
+#pragma unroll
+          for (int k = 0; k < SP_K / 16; ++k) {
+            const uint64_t ah = sw64_desc(a + k * 32), am = sw64_desc(a + SP_A_BYTES + k * 32),
+                           al = sw64_desc(a + 2 * SP_A_BYTES + k * 32);
+            const uint64_t bh = sw64_desc(b + k * 32), bm = sw64_desc(b + SP_B_BYTES + k * 32),
+                           bl = sw64_desc(b + 2 * SP_B_BYTES + k * 32);
+            umma_f16(dr, al, bh, idesc, (kb | k) != 0);
+            umma_f16(dr, ah, bl, idesc, 1);
+            umma_f16(dr, am, bm, idesc, 1);
+            umma_f16(dr, am, bh, idesc, 1);
+            umma_f16(dr, ah, bm, idesc, 1);
+          }
+          const bool first = kb % SP_CHUNK == 0;
+          if (first) {
+            if (!mbar_wait(&sh.hempty, hph, &sh.abort_flag)) {
+              ok = false;
+              break;
+            }
+            hph ^= 1u;
+            tc_fence_after();
+          }
+#pragma unroll
+          for (int k = 0; k < SP_K / 16; ++k)
+            umma_f16(dh, sw64_desc(a + k * 32), sw64_desc(b + k * 32), idesc, !(first && k == 0));
+          umma_commit(&sh.empty[s]);
+          if (++s == SP_STAGES) {
+            s = 0;
+            ph ^= 1u;
+          }
+          if (kb % SP_CHUNK == SP_CHUNK - 1 || kb == nk - 1) umma_commit(&sh.hfull);
+        }
+      }
+      if (!ok) {
+        atomicExch(err, 2);
+        sh.abort_flag = 1;
+      }
+    }
+  } else {
+    // ---------------- epilogue (warps 2..9)
+    const int q = warp & 3, ew = warp - 2, half = ew >> 2;
+    const uint32_t th = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * (SP_N / 2));
+    const int chunks = (nk + SP_CHUNK - 1) / SP_CHUNK;
+    uint32_t hph = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
+      const int tm = t % tiles_m, tn = t / tiles_m;
+      const int n0 = tn * SP_N + half * (SP_N / 2);
+      __syncwarp();
+      for (int c = lane; c < SP_N / 2; c += 32) {
+        const int n = n0 + c;
+        sh.nP[ew][c] = n < nP ? normP[n] : 0.0f;
+        sh.sP[ew][c] = n < nP ? scaleP[n] : 0.0f;
+      }
+      __syncwarp();
+      float tot[SP_N / 2];
+#pragma unroll
+      for (int c = 0; c < SP_N / 2; ++c) tot[c] = 0.0f;
+      for (int ch = 0; ch < chunks; ++ch) {
+        if (lane == 0) ok = mbar_wait(&sh.hfull, hph, &sh.abort_flag);
+        ok = __shfl_sync(kFull, ok ? 1 : 0, 0) != 0;
+        if (!ok) break;
+        hph ^= 1u;
+        tc_fence_after();
+#pragma unroll
+        for (int c0 = 0; c0 < SP_N / 2; c0 += 32) {
+          uint32_t r[32];
+          tmem_ld32(th + (uint32_t)c0, r);
+#pragma unroll
+          for (int c = 0; c < 32; ++c) tot[c0 + c] += __uint_as_float(r[c]);
+        }
+        if (ch + 1 < chunks) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&sh.hempty);
+        }
+      }
+      if (!ok) {
+        if (lane == 0) {
+          atomicExch(err, 3);
+          sh.abort_flag = 1;
+        }
+        break;
+      }
+#pragma unroll
+      for (int c0 = 0; c0 < SP_N / 2; c0 += 32) {
+        uint32_t r[32];
+        tmem_ld32(th + (uint32_t)(SP_N + c0), r);
+#pragma unroll
+        for (int c = 0; c < 32; ++c) tot[c0 + c] += __uint_as_float(r[c]);
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(&sh.hempty);
+        mbar_arrive(&sh.rempty);
+      }
+      const int m = tm * SP_M + q * 32 + lane;
+      const int ncols = min(SP_N / 2, nP - n0);
+      if (m < nQ) {
+        const float nq = normQ[m], sq = scaleQ[m];
+        float* o = out + (int64_t)n0 * ldo + m;
+#pragma unroll
+        for (int c = 0; c < SP_N / 2; ++c) {
+          if (c < ncols) {
+            const float dot = tot[c] * sq * sh.sP[ew][c];
+            const float d2 = fmaxf(nq + sh.nP[ew][c] - 2.0f * dot, 0.0f);
+            o[(int64_t)c * ldo] = exp2f(d2 * neg_scale);
+          }
+        }
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, SpCfg<SP_N>::kTmemCols);
+  }
+}
+
+// ------------------------------------------------------------- row slices
+// One warp per row of the two sets (references, then samples): the
+// power-of-two scale, the three slices, and (when asked) the squared norm;
+// *bad is set for a row holding NaN or Inf (its slices are then meaningless).
+struct SplitSource {
+  const float* X;
+  int64_t ld, n;
+  __half* v;
+  float *scale, *normsq;
+  int vec;  // 16-byte loads
+};
+
+__global__ void split_rows_kernel(SplitSource A, SplitSource B, int d, int ks, int* __restrict__ bad) {
+  const int lane = threadIdx.x & 31;
+  int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (row >= A.n + B.n) return;
+  const bool second = row >= A.n;
+  if (second) row -= A.n;
+  const SplitSource S = second ? B : A;
+  const float* x = S.X + row * S.ld;
+  auto load4 = [&](int c) -> float4 {  // values c..c+3, zero past d
+    if (S.vec) return c < d ? __ldg(reinterpret_cast<const float4*>(x + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    return make_float4(c < d ? __ldg(x + c) : 0.f, c + 1 < d ? __ldg(x + c + 1) : 0.f,
+                       c + 2 < d ? __ldg(x + c + 2) : 0.f, c + 3 < d ? __ldg(x + c + 3) : 0.f);
+  };
+  float2 acc = make_float2(0.0f, 0.0f);
+  uint32_t top = 0;  // the largest |value|, as an integer (NaN and Inf sort above)
+  for (int c = lane * 4; c < d; c += 128) {
+    const float4 v = load4(c);
+    top = max(max(top, max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu)),
+              max(__float_as_uint(v.z) & 0x7fffffffu, __float_as_uint(v.w) & 0x7fffffffu));
+    if (S.normsq) acc = df_add_sq(df_add_sq(df_add_sq(df_add_sq(acc, v.x), v.y), v.z), v.w);
+  }
+  top = __reduce_max_sync(kFull, top);
+  if (S.normsq) {
+    acc = warp_sum_df(acc);
+    if (lane == 0) S.normsq[row] = df_to_float(acc);
+  }
+  const int e = (int)(top >> 23);  // biased exponent (0: zero or subnormal)
+  if (e == 255 && bad && lane == 0) *bad = 1;
+  // scaled maximum in [2^14, 2^15); the exponent stays within the normal range
+  const int up = min(141 - e, 126);  // 14 - (e - 127)
+  const float s = __uint_as_float((uint32_t)(127 + up) << 23);
+  if (lane == 0) S.scale[row] = __uint_as_float((uint32_t)(127 - up) << 23);
+  __half* const o = S.v + row * ks;
+  const int64_t slice = S.n * (int64_t)ks;
+  for (int c = lane * 4; c < ks; c += 128) {
+    const float4 v = load4(c);
+    const float t[4] = {v.x * s, v.y * s, v.z * s, v.w * s};
+    __half h[3][4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float hi = rintf(t[q] * 0x1p-7f) * 0x1p7f;
+      const float r1 = t[q] - hi;  // exact
+      const float mid = rintf(r1 * 0x1p2f) * 0x1p-2f;
+      const float r2 = r1 - mid;   // exact
+      h[0][q] = __float2half_rn(hi);
+      h[1][q] = __float2half_rn(mid);
+      h[2][q] = __float2half_rn(rintf(r2 * 0x1p11f) * 0x1p-11f);
+    }
+#pragma unroll
+    for (int w = 0; w < 3; ++w) *reinterpret_cast<uint2*>(o + w * slice + c) = *reinterpret_cast<const uint2*>(h[w]);
+  }
+}
+
+cudaError_t launch_split_rows(const SplitRows& P, int64_t nP, const SplitRows& Q, int64_t nQ, int64_t d, int ks,
+                              int* bad, cudaStream_t st) {
+  if (nP + nQ <= 0) return cudaSuccess;
+  auto source = [&](const SplitRows& r, int64_t n) {
+    const int vec = d % 4 == 0 && r.ld % 4 == 0 && (reinterpret_cast<uintptr_t>(r.X) & 15) == 0;
+    return SplitSource{r.X, r.ld, n, r.v, r.scale, r.form_norm ? r.norm : nullptr, vec};
+  };
+  split_rows_kernel<<<(unsigned)ceil_div(nP + nQ, 8), 256, 0, st>>>(source(P, nP), source(Q, nQ), (int)d, ks, bad);
+  return cudaGetLastError();
+}
+
+// 2-D map of a slice array [3 n][ks], box = 32 values x box_rows, 64-byte swizzle.
+static bool split_map(CUtensorMap* map, const __half* base, int64_t n, int ks, int box_rows) {
+  auto enc = get_encode();
+  if (!enc) return false;
+  cuuint64_t dims[2] = {(cuuint64_t)ks, (cuuint64_t)(3 * n)};
+  cuuint64_t strides[1] = {(cuuint64_t)(ks * 2)};
+  cuuint32_t box[2] = {SP_K, (cuuint32_t)box_rows};
+  cuuint32_t estr[2] = {1, 1};
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<__half*>(base), dims, strides, box, estr,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+cudaError_t launch_gram_split(const SplitRows& P, int64_t nP, const SplitRows& Q, int64_t nQ, int ks, float neg_scale,
+                              float* out, int64_t ldo, int* err, int n_sms, cudaStream_t st) {
+  if (nP <= 0 || nQ <= 0) return cudaSuccess;
+  if (ks % 8 != 0 || (reinterpret_cast<uintptr_t>(P.v) & 15) || (reinterpret_cast<uintptr_t>(Q.v) & 15) ||
+      3 * nP > INT32_MAX || 3 * nQ > INT32_MAX)
+    return cudaErrorInvalidValue;
+  alignas(64) CUtensorMap mq, mp;
+#define KKM_SPLIT_LAUNCH(N)                                                                                    \
+  do {                                                                                                         \
+    if (!split_map(&mq, Q.v, nQ, ks, SP_M) || !split_map(&mp, P.v, nP, ks, N)) return cudaErrorInvalidValue;   \
+    static const cudaError_t attr = cudaFuncSetAttribute(                                                      \
+        gram_split_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SpCfg<N>::kSmem);              \
+    if (attr != cudaSuccess) return attr;                                                                      \
+    const int64_t tiles = ceil_div(nQ, SP_M) * ceil_div(nP, N);                                                \
+    gram_split_kernel<N><<<(unsigned)std::min<int64_t>(tiles, std::max(n_sms, 1)), SP_THREADS, SpCfg<N>::kSmem, st>>>( \
+        mq, mp, (int)nQ, (int)nP, ks, Q.norm, P.norm, Q.scale, P.scale, neg_scale, out, ldo, err);             \
+  } while (0)
+  if (2 * ceil_div(nQ, SP_M) * ceil_div(nP, 256) <= n_sms) KKM_SPLIT_LAUNCH(64);
+  else KKM_SPLIT_LAUNCH(256);
+#undef KKM_SPLIT_LAUNCH
+  return cudaGetLastError();
+}
+
+}  // namespace kkm

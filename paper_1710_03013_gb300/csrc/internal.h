@@ -234,6 +234,40 @@ cudaError_t launch_gram_rbf_half(const float* A, int64_t nA, const float* Bm, in
                                  const float* normB, const int64_t* idA, const int64_t* idB, float neg_scale,
                                  __half* out, int64_t ldo, cudaStream_t st, float* out32 = nullptr);
 
+// ---- the FP32 Gaussian block on the tensor cores (gram_split.cu) ----------
+// FP32 rows X[r * ld .. + d) as three FP16 slices: v [3][n][ks] (ks = the row
+// length rounded up to 8), a power-of-two scale per row and the squared norms
+// (formed with the slices, or given).
+struct SplitRows {
+  const float* X = nullptr;
+  int64_t ld = 0;
+  __half* v = nullptr;
+  float* scale = nullptr;
+  float* norm = nullptr;
+  bool form_norm = true;
+};
+// The slices of both sides in one launch; *bad (nullable) is set when a value
+// is NaN or Inf.
+cudaError_t launch_split_rows(const SplitRows& P, int64_t nP, const SplitRows& Q, int64_t nQ, int64_t d, int ks,
+                              int* bad, cudaStream_t st);
+// out[n*ldo + m] = exp(-|p_n - q_m|^2 / (2 sigma^2)); *err as launch_gram_tc.
+cudaError_t launch_gram_split(const SplitRows& P, int64_t nP, const SplitRows& Q, int64_t nQ, int ks, float neg_scale,
+                              float* out, int64_t ldo, int* err, int n_sms, cudaStream_t st);
+// Whether kkm_kernel_matrix and kkm_assign take it for an FP32 Gaussian block
+// against nA reference rows of d values: a rule on the references alone, so
+// that a sample's values do not depend on how many samples share the call.  Up
+// to 32 references have the skinny kernel.  From 64 values on it is no slower
+// than the FFMA kernel at any size measured (us a call, FFMA / here: assign of
+// 1 row to 200 supports 73.8 / 76.8 at d = 64 and 82.8 / 75.5 at d = 128, of
+// 2,000 rows to 3,000 supports 98 / 101 and 119 / 101; a 5,000 x 20,000 matrix
+// 382 / 332 at d = 48, 695 / 355 at d = 128; at d = 16 245 / 325).  Fits keep
+// the FFMA kernel: their labels at near ties follow the block's last bits, and
+// a resumed checkpoint has to go on as it began.
+constexpr int64_t kSplitMinDim = 64;
+constexpr bool split_applies(int kind, int64_t nA, int64_t d) {
+  return kind == KKM_RBF && nA > 32 && d >= kSplitMinDim && 3 * nA <= INT32_MAX;
+}
+
 // ---- tensor-core (tcgen05) BF16 kernel block ----------------------------
 // out[n*ldo + m] = kappa(P_n, Q_m) for BF16 rows P [nP][ldb], Q [nQ][ldb]
 // (dk valid columns), with the squared norms of the BF16 rows; out is float,
