@@ -376,11 +376,16 @@ struct Readback {
 struct PendingCheck {
   int* flag = nullptr;  // pinned
   cudaStream_t st = nullptr;
-  ~PendingCheck() { pinned_flag_release(flag); }
+  bool landed = false;
+  ~PendingCheck() {
+    if (flag && !landed) cudaStreamSynchronize(st);  // an error return: the copy into the flag is still on its way
+    pinned_flag_release(flag);
+  }
   kkm_status wait(bool* bad) {
     *bad = false;
     if (!flag) return KKM_OK;
-    KKM_CK(cudaStreamSynchronize(st));
+    if (!landed) KKM_CK(cudaStreamSynchronize(st));
+    landed = true;
     *bad = *flag != 0;
     return KKM_OK;
   }
@@ -392,8 +397,10 @@ struct PendingCheck {
 // prep_rows), pinned host X 16-byte aligned is used in place: *out is its
 // device address, nothing is copied or checked here, and *pull_flag is a
 // zeroed device word for the rows' check.
+// *flag_out gets the check's device flag (nonzero: NaN or Inf).
 static kkm_status device_input_checked(Workspace& ws, const float* p, int64_t n, const float** out, bool* bad,
-                                       PendingCheck* pending = nullptr, int** pull_flag = nullptr) {
+                                       PendingCheck* pending = nullptr, int** pull_flag = nullptr,
+                                       int** flag_out = nullptr) {
   cudaStream_t st = ws.st;
   *bad = false;
   *out = p;
@@ -402,6 +409,7 @@ static kkm_status device_input_checked(Workspace& ws, const float* p, int64_t n,
   int* flag;
   KKM_TRY(ws.alloc(&flag, 1));
   KKM_CK(cudaMemsetAsync(flag, 0, 4, st));
+  if (flag_out) *flag_out = flag;
   cudaPointerAttributes a;
   const bool known = cudaPointerGetAttributes(&a, p) == cudaSuccess;
   if (!known) cudaGetLastError();
@@ -888,26 +896,27 @@ static kkm_status alloc_loop(Workspace& ws, int nLmax, int C, int64_t ldk, int t
   KKM_TRY(ws.alloc(&I.gcta, (int64_t)I.fused_cap * C));
   KKM_TRY(ws.alloc(&I.facc, 2 * (C + 3)));
   if (gaussian) KKM_TRY(ws.alloc(&I.lm_list, 2 * (int64_t)nLmax));
-  KKM_TRY(ws.alloc(&I.bar, 1));
-  KKM_TRY(ws.alloc(&I.err, 1));
-  KKM_CK(cudaMemsetAsync(I.bar, 0, 4, ws.st));
-  KKM_CK(cudaMemsetAsync(I.err, 0, 4, ws.st));
   KKM_TRY(ws.alloc(&I.ghat_cur, C));
-  KKM_TRY(ws.alloc(&I.gtick, C));
-  KKM_CK(cudaMemsetAsync(I.gtick, 0, (size_t)C * 4, ws.st));
-  if (gaussian) {
-    KKM_TRY(ws.alloc(&I.gfix, C));
-    KKM_CK(cudaMemsetAsync(I.gfix, 0, (size_t)C * 8, ws.st));
-    I.gfix_shift = gfix_shift_for(nLmax);
-  }
-  KKM_TRY(ws.alloc(&I.ticket, 1));
-  KKM_TRY(ws.alloc(&I.done, 1));
   KKM_TRY(ws.alloc(&I.trace_omega, std::max(trace_cap, 1)));
   KKM_TRY(ws.alloc(&I.trace_changed, std::max(trace_cap, 1)));
-  KKM_TRY(ws.alloc(&I.trace_count, 1));
-  KKM_CK(cudaMemsetAsync(I.ticket, 0, 4, ws.st));
-  KKM_CK(cudaMemsetAsync(I.done, 0, 4, ws.st));
-  KKM_CK(cudaMemsetAsync(I.trace_count, 0, 4, ws.st));
+  // everything that starts at zero, a 256-byte line or more each, in one block
+  // with one fill (seven fills took longer than a small call's kernels)
+  const int64_t fix = gaussian ? round_up(8 * C, 256) : 0, tick = round_up(4 * C, 256);
+  char* zero;
+  const int64_t bytes = fix + tick + 5 * 256;
+  KKM_TRY(ws.alloc(&zero, bytes));
+  KKM_CK(cudaMemsetAsync(zero, 0, (size_t)bytes, ws.st));
+  if (gaussian) {
+    I.gfix = reinterpret_cast<unsigned long long*>(zero);
+    I.gfix_shift = gfix_shift_for(nLmax);
+  }
+  I.gtick = reinterpret_cast<uint32_t*>(zero + fix);
+  auto word = [&](int k) { return reinterpret_cast<int32_t*>(zero + fix + tick + 256 * k); };
+  I.bar = reinterpret_cast<uint32_t*>(word(0));
+  I.err = word(1);
+  I.ticket = reinterpret_cast<uint32_t*>(word(2));
+  I.done = word(3);
+  I.trace_count = word(4);
   return KKM_OK;
 }
 
@@ -1963,9 +1972,13 @@ static kkm_status assign_impl(const kkm_model* m, const float* Xnew_in, int64_t 
   setup_pool_once(dev);
   Workspace ws(st);
   const float* X = nullptr;
+  // the check is not waited for: its flag keeps the kernels that write labels
+  // and distances from writing any
+  PendingCheck chk;
+  int* bad_d = nullptr;
   {
     bool bad = false;
-    KKM_TRY(device_input_checked(ws, Xnew_in, M * d, &X, &bad));
+    KKM_TRY(device_input_checked(ws, Xnew_in, M * d, &X, &bad, &chk, nullptr, &bad_d));
     if (bad) return invalid("X holds NaN or Inf");
   }
   int32_t* lab = nullptr;
@@ -2020,7 +2033,7 @@ static kkm_status assign_impl(const kkm_model* m, const float* Xnew_in, int64_t 
     S.col_ord = nullptr;
     S.lab = nullptr;
     lb.I.ghat_in = m->ghat;
-    lb.I.done = nullptr;
+    lb.I.done = bad_d;
   }
   for (int64_t c0 = 0; c0 < M; c0 += chunk) {
     const int n = (int)std::min<int64_t>(chunk, M - c0);
@@ -2047,8 +2060,13 @@ static kkm_status assign_impl(const kkm_model* m, const float* Xnew_in, int64_t 
     } else {
       KKM_RUN("nearest", st,
               launch_nearest(Kb, ldm, n, C, kself, sp.kind == KKM_LINEAR ? m->med_aux : nullptr, lab + c0,
-                             dist + c0, st));
+                             dist + c0, st, bad_d));
     }
+  }
+  if (omega_out || lab_host || dist_host) {  // nothing is copied out for bad input
+    bool bad = false;
+    KKM_TRY(chk.wait(&bad));
+    if (bad) return invalid("X holds NaN or Inf");
   }
   double* omega_d = nullptr;
   if (omega_out) {
@@ -2065,6 +2083,11 @@ static kkm_status assign_impl(const kkm_model* m, const float* Xnew_in, int64_t 
   if (split) KKM_CK(cudaMemcpyAsync(&rtc_err_h, split_err, 4, cudaMemcpyDeviceToHost, st));
   KKM_CK(cudaStreamSynchronize(st));
   prof_collect();
+  {
+    bool bad = false;
+    KKM_TRY(chk.wait(&bad));
+    if (bad) return invalid("X holds NaN or Inf");
+  }
   if (rtc_err_h) {
     set_error(split ? "tensor-core kernel block: a bounded pipeline wait gave up"
                     : "tensor-core MD estimate: a bounded pipeline wait gave up");

@@ -562,7 +562,7 @@ cudaError_t launch_iterate_tc(const __half* KT, int64_t ldk, int Ni, const Suppo
 // ---- mini-batch boundary -----------------------------------------------------
 // Eq. 8: u[l] = argmin_j kself[l] - 2 Kt[j][l] + kmm[j]; dmin (nullable).
 cudaError_t launch_nearest(const float* Kt, int64_t ldk, int Ni, int C, const float* kself,
-                           const float* kmm, int32_t* u, float* dmin, cudaStream_t st);
+                           const float* kmm, int32_t* u, float* dmin, cudaStream_t st, const int* skip = nullptr);
 // Eq. 10 keys and member counts c_j (keys/c must be reset by the caller).
 cudaError_t launch_medoid_keys(int64_t ldk, int Ni, const Supports& S, const IterState& I,
                                const float* kself, const int32_t* u, unsigned long long* keys,

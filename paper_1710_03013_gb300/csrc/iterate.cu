@@ -1755,9 +1755,9 @@ cudaError_t launch_iterate(const __half* KT, int64_t ldk, int Ni, const Supports
 // ----------------------------------------------------- Eq. 8 nearest medoid
 __global__ void nearest_kernel(const float* __restrict__ Kt, int64_t ldk, int Ni, int C,
                                const float* __restrict__ kself, const float* __restrict__ kmm,
-                               int32_t* __restrict__ u, float* __restrict__ dmin) {
+                               int32_t* __restrict__ u, float* __restrict__ dmin, const int* __restrict__ skip) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= Ni) return;
+  if (i >= Ni || (skip && *skip)) return;
   const float ks = kself ? kself[i] : 1.0f;
   float best = __int_as_float(0x7f800000);
   int bj = 0;
@@ -1773,9 +1773,10 @@ __global__ void nearest_kernel(const float* __restrict__ Kt, int64_t ldk, int Ni
 }
 
 cudaError_t launch_nearest(const float* Kt, int64_t ldk, int Ni, int C, const float* kself,
-                           const float* kmm, int32_t* u, float* dmin, cudaStream_t st) {
+                           const float* kmm, int32_t* u, float* dmin, cudaStream_t st,
+                           const int* skip) {
   if (Ni <= 0) return cudaSuccess;
-  nearest_kernel<<<(unsigned)ceil_div(Ni, 256), 256, 0, st>>>(Kt, ldk, Ni, C, kself, kmm, u, dmin);
+  nearest_kernel<<<(unsigned)ceil_div(Ni, 256), 256, 0, st>>>(Kt, ldk, Ni, C, kself, kmm, u, dmin, skip);
   return cudaGetLastError();
 }
 
