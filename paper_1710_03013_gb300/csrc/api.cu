@@ -594,17 +594,19 @@ static kkm_status copy_prepared(const KernelSpec& sp, const float* Xp, const int
 }
 // out[a*ldo + b] = K(A_a, B_b).  dist != 0 gives distances instead.
 // Scratch of the MD kernel's tensor-core path (sized for the largest call):
-// BF16 planes of both sides, their squared radii, the refine flags and the
-// tensor-core error word.
+// BF16 planes of both sides, the rotations and bits of the near pairs, the
+// units of the exact pass and the tensor-core error word.
 struct RmsdTcScratch {
-  __nv_bfloat16* P = nullptr;  // [nP_cap][4][3 kp] split-BF16 references
-  __nv_bfloat16* Q = nullptr;  // [nQ_cap][4][3 kp] split-BF16 samples
+  __nv_bfloat16* P = nullptr;  // [nP_cap][3][3 kp] split-BF16 references
+  __nv_bfloat16* Q = nullptr;  // [nQ_cap][3][3 kp] split-BF16 samples
   float4* quat = nullptr;      // [nP_cap][ld_cap] rotations of the pairs to refine
-  int* flags = nullptr;
+  uint8_t* near = nullptr;     // [nP_cap][pitch] a bit per pair to refine
+  uint2* units = nullptr;      // units of the exact pass, *count of them
+  unsigned* count = nullptr;
   int* key = nullptr;    // [nP_cap] reference sort keys
   int* order = nullptr;  // [nP_cap] reference order of the exact pass
   int* err = nullptr;
-  int64_t nP_cap = 0, nQ_cap = 0, ld_cap = 0;
+  int64_t nP_cap = 0, nQ_cap = 0, ld_cap = 0, pitch = 0;
   int kp = 0;
 };
 
@@ -619,10 +621,13 @@ static kkm_status alloc_rmsd_tc(Workspace& ws, const KernelSpec& sp, int64_t nP_
   t->nP_cap = nP_cap;
   t->nQ_cap = nQ_cap;
   t->ld_cap = ld_cap;
-  KKM_TRY(ws.alloc(&t->P, nP_cap * 4 * 3 * t->kp));
-  KKM_TRY(ws.alloc(&t->Q, nQ_cap * 4 * 3 * t->kp));
+  KKM_TRY(ws.alloc(&t->P, nP_cap * 3 * 3 * t->kp));
+  KKM_TRY(ws.alloc(&t->Q, nQ_cap * 3 * 3 * t->kp));
   KKM_TRY(ws.alloc(&t->quat, nP_cap * ld_cap));
-  KKM_TRY(ws.alloc(&t->flags, ceil_div(nP_cap, 32) * ceil_div(nQ_cap, 64)));
+  t->pitch = rmsd_near_pitch(nQ_cap);
+  KKM_TRY(ws.alloc(&t->near, nP_cap * t->pitch));
+  KKM_TRY(ws.alloc(&t->units, rmsd_max_units(nP_cap, nQ_cap)));
+  KKM_TRY(ws.alloc(&t->count, 1));
   KKM_TRY(ws.alloc(&t->key, nP_cap));
   KKM_TRY(ws.alloc(&t->order, nP_cap));
   KKM_TRY(ws.alloc(&t->err, 1));
@@ -631,10 +636,9 @@ static kkm_status alloc_rmsd_tc(Workspace& ws, const KernelSpec& sp, int64_t nP_
 }
 
 // MD kernel block on the tensor cores: a BF16 screen of every pair, then the
-// exact FP32 two-pass kernel only on the 32 x 64 tiles holding a pair the
-// screen could not certify as far (the others keep 0; their true values are
-// below 1e-5), with the references reordered so that near pairs gather in
-// few tiles.
+// exact FP32 residual only for the pairs the screen could not certify as far
+// (the others keep 0; their true values are below 1e-5), in units of 16 x 16
+// pairs, with the references reordered so that near pairs gather in few units.
 static kkm_status rmsd_block_tc(const KernelSpec& sp, const float* A, const float* auxA, const int64_t* idA,
                                 int64_t nA, const float* Bm, const float* auxB, const int64_t* idB, int64_t nB,
                                 float* out, int64_t ldo, const RmsdTcScratch& t, bool block, cudaStream_t st);
@@ -673,23 +677,22 @@ static kkm_status rmsd_block_tc(const KernelSpec& sp, const float* A, const floa
                                 int64_t nA, const float* Bm, const float* auxB, const int64_t* idB, int64_t nB,
                                 float* out, int64_t ldo, const RmsdTcScratch& t, bool block, cudaStream_t st) {
   if (ldo > t.ld_cap) return invalid("internal: MD scratch too small");
+  const int64_t pitch = rmsd_near_pitch(nB);  // of this call's samples
   KKM_RUN("rmsd_to_bf16", st, launch_rmsd_to_bf16(A, nA, sp.ap, sp.n_atoms, t.P, t.kp, 0, st));
   KKM_RUN("rmsd_to_bf16", st, launch_rmsd_to_bf16(Bm, nB, sp.ap, sp.n_atoms, t.Q, t.kp, 1, st));
   KKM_RUN(block ? "rmsd_block" : "rmsd_gram", st,
-          launch_rmsd_tc_estimate(t.P, nA, t.Q, nB, 3 * t.kp, auxA, auxB, sp.n_atoms, sp.neg_scale(), out, t.quat,
-                                  ldo, t.err, sm_count(), st));
-  KKM_RUN("rmsd_plan", st, launch_rmsd_refine_plan(out, ldo, (int)nA, (int)nB, t.key, t.order, t.flags, st));
+          launch_rmsd_screen(t.P, nA, t.Q, nB, 3 * t.kp, auxA, auxB, sp.n_atoms, sp.neg_scale(), out, t.quat,
+                             t.near, pitch, ldo, t.err, sm_count(), st));
+  KKM_RUN("rmsd_plan", st,
+          launch_rmsd_refine_plan(t.near, pitch, (int)nA, (int)nB, t.key, t.order, t.units, t.count, st));
   KKM_RUN("rmsd_exact", st,
-          launch_rmsd_gram(DK_RBF, A, nA, Bm, nB, sp.ap, sp.n_atoms, auxA, auxB, idA, idB, sp.neg_scale(), out, ldo,
-                           st, t.flags, t.order, t.quat));
+          launch_rmsd_exact(A, nA, Bm, nB, sp.ap, sp.n_atoms, idA, idB, sp.neg_scale(), out, ldo, t.near, pitch, t.order,
+                            t.units, t.count, t.quat, st));
   if (prof_on()) {  // pairs the exact pass recomputed (profiling only: a read-back)
-    const int64_t nf = ceil_div(nA, 32) * ceil_div(nB, 64);
-    std::vector<int> f((size_t)nf);
-    KKM_CK(cudaMemcpyAsync(f.data(), t.flags, (size_t)nf * 4, cudaMemcpyDeviceToHost, st));
+    unsigned n = 0;
+    KKM_CK(cudaMemcpyAsync(&n, t.count, 4, cudaMemcpyDeviceToHost, st));
     KKM_CK(cudaStreamSynchronize(st));
-    int64_t tiles = 0;
-    for (int v : f) tiles += v != 0;
-    prof_add_work("rmsd_exact", (double)tiles * 32.0 * 64.0);
+    prof_add_work("rmsd_exact", (double)n * 16.0 * 16.0);
   }
   return KKM_OK;
 }

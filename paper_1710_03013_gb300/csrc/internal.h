@@ -183,7 +183,7 @@ inline int side_by_side_iteration(int iteration) { (void)iteration; return KKM_I
 constexpr int64_t kBf16TensorMinDim = 129;
 
 // Kernel-function codes used on the device.
-enum DevKind { DK_RBF = 0, DK_LINEAR = 1, DK_DIST = 2, DK_RMSD_EST = 3, DK_RAW = 4 /* plain products */ };
+enum DevKind { DK_RBF = 0, DK_LINEAR = 1, DK_DIST = 2, DK_RAW = 3 /* plain products */ };
 
 // --------------------------------------------------------- kernel launchers
 // (all asynchronous on `st`; they return a CUDA error code of the launch)
@@ -276,20 +276,22 @@ constexpr bool split_applies(int kind, int64_t nA, int64_t d) {
 cudaError_t launch_gram_tc(int kind, const __nv_bfloat16* P, int64_t nP, const __nv_bfloat16* Q, int64_t nQ,
                            int dk, int ldb, const float* normP, const float* normQ, float neg_scale, void* out,
                            bool out_half, int64_t ldo, int* err, int n_sms, cudaStream_t st);
-// MD kernel screen on the tensor cores: P [4 nP][kp] and Q [4 nQ][kp] hold
-// split-BF16 centred frames (planes x, y, z and a zero plane; kp = 3 segments
-// of the padded atom count, see launch_rmsd_to_bf16), gP / gQ their squared
-// radii.  out[l*ldo + s] = 0 where the correlation certifies exp(-rmsd^2 /
-// (2 sigma^2)) < kRmsdRefine, else 1 with the optimal rotation as a unit
-// quaternion in quat[l*ldo + s]; the pairs marked 1 are recomputed exactly
-// (launch_rmsd_refine_plan, then launch_rmsd_gram with tile flags and quat).
+// MD kernel screen on the tensor cores: P [3 nP][dk] and Q [3 nQ][dk] hold
+// split-BF16 centred frames (planes x, y, z; dk = 3 segments of the padded
+// atom count, see launch_rmsd_to_bf16), gP / gQ their squared radii.
+// out[l*ldo + s] = 0 for every pair, and bit s % 8 of near[l*pitch + s/8] is 0
+// where the correlation certifies exp(-rmsd^2 / (2 sigma^2)) < kRmsdRefine,
+// else 1 with the optimal rotation as a unit quaternion in quat[l*ldo + s];
+// the near pairs are then evaluated exactly (launch_rmsd_refine_plan,
+// launch_rmsd_exact).  pitch: a multiple of 16 bytes, 8 * pitch >= nQ.
 // The split operands give the correlation to ~1e-5 relative, so the
 // rotation's error enters the exact residual at ~1e-10; the certificate's
 // margin holds for sigma >= 0.5 A and coordinates within ~100 A of the centroid.
 constexpr float kRmsdRefine = 1e-6f;
-cudaError_t launch_rmsd_tc_estimate(const __nv_bfloat16* P, int64_t nP, const __nv_bfloat16* Q, int64_t nQ, int kp,
-                                    const float* gP, const float* gQ, int n_atoms, float neg_scale, float* out,
-                                    float4* quat, int64_t ldo, int* err, int n_sms, cudaStream_t st);
+cudaError_t launch_rmsd_screen(const __nv_bfloat16* P, int64_t nP, const __nv_bfloat16* Q, int64_t nQ, int dk,
+                               const float* gP, const float* gQ, int n_atoms, float neg_scale, float* out,
+                               float4* quat, uint8_t* near, int64_t pitch, int64_t ldo, int* err, int n_sms,
+                               cudaStream_t st);
 // out[k*ldo + L[k]] = 1 (the exact diagonal of a Gaussian kernel block).
 cudaError_t launch_set_diag(void* out, bool out_half, int64_t ldo, const int32_t* L, int nL, cudaStream_t st);
 // FP8 e4m3 operands with a scale per row (rows [ld8] bytes, ld8 a multiple of
@@ -315,23 +317,27 @@ cudaError_t launch_rmsd_prep_rows(const float* X, int n_atoms, int64_t start, in
 cudaError_t launch_rmsd_prep_idx64(const float* X, int n_atoms, const int64_t* idx, int64_t n,
                                    float* out, int ap, float* gsq, cudaStream_t st);
 // kind DK_RBF: out = exp(-rmsd^2/(2 sigma^2)) via neg_scale; DK_DIST: rmsd.
-// tile_flag (nullable): only the tiles of 32 A-frames x 64 B-frames whose
-// flag is set are computed ([ceil(nA/32)][ceil(nB/64)], A-tile major); arow
-// (nullable): A tile rows are the frames arow[0..nA) in that order; quat
-// (nullable, with tile_flag): rotations of the screen for the pairs it
-// marked 1 in out, so only the residual pass runs (pairs marked 0 keep 0).
 cudaError_t launch_rmsd_gram(int kind, const float* A, int64_t nA, const float* Bm, int64_t nB,
                              int ap, int n_atoms, const float* gA, const float* gB,
                              const int64_t* idA, const int64_t* idB, float neg_scale,
-                             float* out, int64_t ldo, cudaStream_t st, const int* tile_flag = nullptr,
-                             const int* arow = nullptr, const float4* quat = nullptr);
-// From the estimate block est [nA][ldo]: the reference order that groups
-// references near the same samples (key [nA], order [nA]) and the refine flag
-// of every (reference tile of that order, sample tile) ([ceil(nA/32)][ceil(nB/64)]).
-cudaError_t launch_rmsd_refine_plan(const float* est, int64_t ldo, int nA, int nB, int* key, int* order, int* flag,
-                                    cudaStream_t st);
-// Centred SoA frames [n][3][ap] (FP32) -> split BF16 rows [n][4][3 kp]
-// (fourth plane and atoms past n_atoms zero): segments (hi, lo, hi) for
+                             float* out, int64_t ldo, cudaStream_t st);
+// Bytes per reference of the near bits, and entries of the unit list.
+constexpr int64_t rmsd_near_pitch(int64_t nQ) { return (nQ + 127) / 128 * 16; }
+constexpr int64_t rmsd_max_units(int64_t nP, int64_t nQ) { return ((nP + 15) / 16) * ((nQ + 15) / 16); }
+// From the screen's near bits ([nA][pitch] bytes): the reference order that
+// groups references near the same samples (key [nA], order [nA]) and the list
+// of units (16 references of that order x 16 samples) that hold a near pair
+// (at most ceil(nA/16) * ceil(nB/16) entries; *count of them).
+cudaError_t launch_rmsd_refine_plan(const uint8_t* near, int64_t pitch, int nA, int nB, int* key, int* order,
+                                    uint2* units, unsigned* count, cudaStream_t st);
+// out = exp(-rmsd^2 / (2 sigma^2)) of the near pairs, at the screen's
+// rotations, over the listed units; the other pairs keep their value.
+cudaError_t launch_rmsd_exact(const float* A, int64_t nA, const float* Bm, int64_t nB, int ap, int n_atoms,
+                              const int64_t* idA, const int64_t* idB, float neg_scale, float* out, int64_t ldo,
+                              const uint8_t* near, int64_t pitch, const int* order, const uint2* units,
+                              const unsigned* count, const float4* quat, cudaStream_t st);
+// Centred SoA frames [n][3][ap] (FP32) -> split BF16 rows [n][3][3 kp] (atoms
+// past n_atoms zero): segments (hi, lo, hi) for
 // side 0 (references), (hi, hi, lo) for side 1 (samples).
 cudaError_t launch_rmsd_to_bf16(const float* src, int64_t n, int ap, int n_atoms, __nv_bfloat16* dst, int kp,
                                 int side, cudaStream_t st);

@@ -156,4 +156,21 @@ __device__ __forceinline__ void quat_to_rot(const float q[4], float R[9]) {
   R[8] = w * w - x * x - y * y + z * z;
 }
 
+// The same with the fused operations written out, so that its bits do not
+// depend on the function it is used in (those of the exact pass have to stay
+// what they are: labels near a tie follow them).
+__device__ __forceinline__ void quat_to_rot_fma(const float q[4], float R[9]) {
+  const float w = q[0], x = q[1], y = q[2], z = q[3];
+  const float ww = __fmul_rn(w, w);
+  R[0] = fmaf(-z, z, fmaf(-y, y, fmaf(x, x, ww)));
+  R[1] = 2.f * fmaf(x, y, -__fmul_rn(w, z));
+  R[2] = 2.f * fmaf(x, z, __fmul_rn(w, y));
+  R[3] = 2.f * fmaf(x, y, __fmul_rn(w, z));
+  R[4] = fmaf(-z, z, fmaf(y, y, fmaf(-x, x, ww)));
+  R[5] = 2.f * fmaf(y, z, -__fmul_rn(w, x));
+  R[6] = 2.f * fmaf(x, z, -__fmul_rn(w, y));
+  R[7] = 2.f * fmaf(y, z, __fmul_rn(w, x));
+  R[8] = fmaf(z, z, fmaf(-y, y, fmaf(-x, x, ww)));
+}
+
 }  // namespace kkm

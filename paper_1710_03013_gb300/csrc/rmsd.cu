@@ -87,7 +87,7 @@ cudaError_t launch_rmsd_prep_idx64(const float* X, int n_atoms, const int64_t* i
 }
 
 // SoA FP32 frames -> BF16 planes for the tensor-core correlation: one warp per
-// frame, row [4 planes][3 kp].  Each coordinate is split v = hi + lo (hi =
+// frame, row [3 planes][3 kp].  Each coordinate is split v = hi + lo (hi =
 // bf16(v), lo = bf16(v - hi)) and the three kp-long segments of a row are
 // (hi, lo, hi) on the reference side and (hi, hi, lo) on the sample side, so
 // one GEMM over 3 kp sums hi.hi + lo.hi + hi.lo: the correlation to about 16
@@ -98,10 +98,10 @@ __global__ void rmsd_to_bf16_kernel(const float* __restrict__ src, int64_t n, in
   const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (row >= n) return;
   const float* s = src + row * 3 * (int64_t)ap;
-  __nv_bfloat16* d = dst + row * 4 * (int64_t)(3 * kp);
-  for (int c = 0; c < 4; ++c)
+  __nv_bfloat16* d = dst + row * 3 * (int64_t)(3 * kp);
+  for (int c = 0; c < 3; ++c)
     for (int k = lane; k < kp; k += 32) {
-      const float v = (c < 3 && k < n_atoms) ? s[c * ap + k] : 0.0f;
+      const float v = k < n_atoms ? s[c * ap + k] : 0.0f;
       const __nv_bfloat16 hi = __float2bfloat16_rn(v);
       const __nv_bfloat16 lo = __float2bfloat16_rn(v - __bfloat162float(hi));
       __nv_bfloat16* r = d + (int64_t)c * 3 * kp + k;
@@ -118,30 +118,33 @@ cudaError_t launch_rmsd_to_bf16(const float* src, int64_t n, int ap, int n_atoms
   return cudaGetLastError();
 }
 
-// ------------------------------------------------- refine-tile ordering
-// After the tensor-core estimate, the exact kernel recomputes only tiles of
-// 32 reference frames x 64 samples holding a pair above kRmsdRefine.  Samples
-// are in trajectory order, so a sample tile is mostly one conformational
-// state; the references are reordered so that a reference tile is too: key
-// = the first sample whose estimate exceeds the threshold (references of one
-// state share it; references near nothing sort last), ties by index.
-__global__ void rmsd_near_key_kernel(const float* __restrict__ est, int64_t ldo, int nA, int nB,
+// --------------------------------------------------- units of the exact pass
+// After the tensor-core screen the exact kernel recomputes units of 16
+// reference frames x 16 samples that hold a pair the screen did not certify
+// far (a bit of `near`, [reference][sample / 8]).  Samples are in trajectory
+// order, so a few neighbours are mostly one conformational state; the
+// references are reordered so that 16 of them are too: key = the first near
+// sample (references of one state share it; references near nothing sort
+// last), ties by index.
+__global__ void rmsd_near_key_kernel(const uint8_t* __restrict__ near, int64_t pitch, int nA, int nB,
                                      int* __restrict__ key) {
   const int lane = threadIdx.x & 31;
   const int a = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (a >= nA) return;
-  const float* row = est + (int64_t)a * ldo;
+  const uint4* row = reinterpret_cast<const uint4*>(near + a * pitch);
   int first = INT_MAX;
-  for (int b0 = 0; b0 < nB && first == INT_MAX; b0 += 32 * 8) {
+  for (int64_t b0 = 0; b0 < pitch / 16 && first == INT_MAX; b0 += 32) {
     int f = INT_MAX;
+    const int64_t b = b0 + lane;
+    if (b < pitch / 16) {
+      const uint4 v = row[b];
+      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int b = b0 + q * 32 + lane;
-      if (b < nB && row[b] > kRmsdRefine) f = min(f, b);
+      for (int q = 3; q >= 0; --q)
+        if (w[q]) f = (int)(b * 128 + q * 32 + __ffs(w[q]) - 1);
+      if (f >= nB) f = INT_MAX;  // (bytes past the last tile of samples are not written)
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) f = min(f, __shfl_xor_sync(kFull, f, o));
-    first = f;
+    first = (int)__reduce_min_sync(kFull, (unsigned)f);
   }
   if (lane == 0) key[a] = first;
 }
@@ -167,32 +170,215 @@ __global__ void rmsd_rank_kernel(const int* __restrict__ key, int nA, int* __res
   order[rank] = a;
 }
 
-// flag[t][u] = 1 if reference tile t (of the order) and sample tile u hold a
-// pair above the threshold; one CTA per (sample tile, reference tile).
-__global__ void rmsd_tile_flag_kernel(const float* __restrict__ est, int64_t ldo, int nA, int nB,
-                                      const int* __restrict__ order, int* __restrict__ flag) {
-  const int u = blockIdx.x, t = blockIdx.y;
-  const int b = u * 64 + (threadIdx.x & 63);
-  int hit = 0;
-  for (int r = threadIdx.x >> 6; r < 32; r += blockDim.x >> 6) {
-    const int ar = t * 32 + r;
-    if (ar < nA && b < nB) hit |= est[(int64_t)order[ar] * ldo + b] > kRmsdRefine;
+constexpr int RX_A = 16, RX_B = 16;  // references x samples of a unit
+
+// Appends every unit (reference tile t of the order, sample tile u) that holds
+// a near pair (in no fixed order: no value depends on it).
+__global__ void __launch_bounds__(256)
+rmsd_units_kernel(const uint8_t* __restrict__ near, int64_t pitch, int nA, int nB, const int* __restrict__ order,
+                  uint2* __restrict__ units, unsigned* __restrict__ count) {
+  const int u = blockIdx.x * 256 + threadIdx.x;
+  const int T = (nA + RX_A - 1) / RX_A, U = (nB + RX_B - 1) / RX_B;
+  const int lane = threadIdx.x & 31;
+  for (int t = blockIdx.y; t < T; t += gridDim.y) {
+    unsigned hit = 0;
+    if (u < U) {
+#pragma unroll
+      for (int r = 0; r < RX_A; ++r) {
+        const int a = order[min(t * RX_A + r, nA - 1)];
+        hit |= *reinterpret_cast<const uint16_t*>(near + a * pitch + 2 * (int64_t)u);
+      }
+    }
+    const unsigned m = __ballot_sync(kFull, hit != 0);
+    unsigned at = 0;
+    if (lane == 0 && m) at = atomicAdd(count, (unsigned)__popc(m));
+    at = __shfl_sync(kFull, at, 0);
+    if (hit) units[at + __popc(m & ((1u << lane) - 1u))] = make_uint2((unsigned)t, (unsigned)u);
   }
-  hit = __syncthreads_or(hit);
-  if (threadIdx.x == 0) flag[(int64_t)t * gridDim.x + u] = hit;
 }
 
-cudaError_t launch_rmsd_refine_plan(const float* est, int64_t ldo, int nA, int nB, int* key, int* order, int* flag,
-                                    cudaStream_t st) {
+cudaError_t launch_rmsd_refine_plan(const uint8_t* near, int64_t pitch, int nA, int nB, int* key, int* order,
+                                    uint2* units, unsigned* count, cudaStream_t st) {
   if (nA <= 0 || nB <= 0) return cudaSuccess;
-  rmsd_near_key_kernel<<<(unsigned)ceil_div(nA, 8), 256, 0, st>>>(est, ldo, nA, nB, key);
+  if (pitch % 16 != 0 || (reinterpret_cast<uintptr_t>(near) & 15)) return cudaErrorInvalidValue;
+  const cudaError_t e = cudaMemsetAsync(count, 0, sizeof(unsigned), st);
+  if (e != cudaSuccess) return e;
+  rmsd_near_key_kernel<<<(unsigned)ceil_div(nA, 8), 256, 0, st>>>(near, pitch, nA, nB, key);
   if ((size_t)nA * sizeof(int) <= 48 * 1024)
     rmsd_rank_kernel<true><<<(unsigned)ceil_div(nA, 256), 256, (size_t)nA * sizeof(int), st>>>(key, nA, order);
   else
     rmsd_rank_kernel<false><<<(unsigned)ceil_div(nA, 256), 256, 0, st>>>(key, nA, order);
-  rmsd_tile_flag_kernel<<<dim3((unsigned)ceil_div(nB, 64), (unsigned)ceil_div(nA, 32)), 256, 0, st>>>(est, ldo, nA, nB,
-                                                                                                   order, flag);
+  const int64_t T = ceil_div(nA, RX_A), U = ceil_div(nB, RX_B);
+  rmsd_units_kernel<<<dim3((unsigned)ceil_div(U, 256), (unsigned)std::min<int64_t>(T, 65535)), 256, 0, st>>>(
+      near, pitch, nA, nB, order, units, count);
   prof_more_launches(2);
+  return cudaGetLastError();
+}
+
+// ------------------------------------------------------------- exact pass
+// exp(-r^2 / (2 sigma^2)) of the near pairs, r^2 = sum_a |R x_a - y_a|^2 / n
+// evaluated directly at the screen's rotation (no cancellation), 12 FMAs per
+// atom and pair: bound by FMA issue.  A warp takes a unit of 16 x 16 pairs by
+// itself, 2 references x 4 samples to a lane (their nine-entry rotations in
+// registers): small units waste little on pairs the screen has settled (a
+// 64-sample tile of a trajectory with dwells of ~100 straddles two states: 24 %
+// of all pairs recomputed, 15.7 % in units of 16), and no warp waits for
+// another.  Eight atoms of the unit's 32 frames at a time reach shared memory
+// by cp.async, four stages per warp (24 floats a frame in a pitch of 28, so
+// that four sample rows start on different banks).
+//
+// 10,000 x 10,000 pairs of 300 atoms, an eighth of them near: 2.71 ms (4.41 ms
+// in tiles of 32 x 64 pairs staged by the CTA).  ncu: FMA pipe 52 %, the rest
+// dispatch stalls (operands from one register bank); paired FMAs
+// (__ffma2_rn) took 3.4 ms, 16-byte shared loads of four atoms 2.84 ms.  One
+// unit to a warp and no persistent CTAs: beside the block a fit's inner loop
+// gets onto the SMs as units finish (MD-shaped fit 51.8 -> 51.2 ms).
+constexpr int RX_T = 8, RX_STAGES = 4, RX_WARPS = 4, RX_PITCH = 28;
+constexpr int RX_STAGE_FLOATS = (RX_A + RX_B) * RX_PITCH;
+constexpr size_t RX_SMEM = sizeof(float) * RX_WARPS * RX_STAGES * RX_STAGE_FLOATS;
+
+__device__ __forceinline__ void rx_cp16(float* dst, const float* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void rx_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void rx_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+__global__ void __launch_bounds__(RX_WARPS * 32, 3)
+rmsd_exact_kernel(const float* __restrict__ A, int nA, const float* __restrict__ Bm, int nB, int ap, int n_atoms,
+                  const int64_t* __restrict__ idA, const int64_t* __restrict__ idB, float neg_scale,
+                  float* __restrict__ out, int64_t ldo, const uint8_t* __restrict__ near, int64_t pitch,
+                  const int* __restrict__ order, const uint2* __restrict__ units, const unsigned* __restrict__ count,
+                  const float4* __restrict__ quat) {
+  extern __shared__ __align__(16) float rx_smem[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float* const ring = rx_smem + warp * RX_STAGES * RX_STAGE_FLOATS;
+  const int lr = lane >> 2, ls = lane & 3;  // references lr, lr + 8; samples ls, ls + 4, ls + 8, ls + 12
+  const int nk = ap / RX_T;
+  const float inv_n = 1.0f / (float)n_atoms;
+  const unsigned n_units = *count;
+  const unsigned w = blockIdx.x * RX_WARPS + warp;
+  if (w >= n_units) return;
+  const uint2 un = units[w];
+  const int a0 = (int)un.x * RX_A, b0 = (int)un.y * RX_B;
+  // the lane's six 16-byte pieces of a stage: frame e / 6 (16 references,
+  // then 16 samples; rows past the end repeat the last one), plane and half
+  const float* src[6];
+  int dst[6];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    const int e = lane + 32 * i, f = e / 6, part = e % 6;
+    const float* row = f < RX_A ? A + (int64_t)order[min(a0 + f, nA - 1)] * 3 * ap
+                                : Bm + (int64_t)min(b0 + f - RX_A, nB - 1) * 3 * ap;
+    src[i] = row + (part >> 1) * ap + (part & 1) * 4;
+    dst[i] = f * RX_PITCH + part * 4;
+  }
+  auto issue = [&](int kt) {
+    if (kt < nk) {
+      float* const st = ring + (kt & (RX_STAGES - 1)) * RX_STAGE_FLOATS;
+#pragma unroll
+      for (int i = 0; i < 6; ++i) rx_cp16(st + dst[i], src[i] + kt * RX_T);
+    }
+    rx_commit();
+  };
+#pragma unroll
+  for (int kt = 0; kt < RX_STAGES - 1; ++kt) issue(kt);
+  // rotations of the near pairs (the identity elsewhere)
+  float R[2][4][9], res[2][4];
+  unsigned need = 0u;
+  int arow[2];
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int a = a0 + lr + 8 * r;
+    arow[r] = order[min(a, nA - 1)];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int b = b0 + ls + 4 * q;
+      res[r][q] = 0.0f;
+      float qq[4] = {1.f, 0.f, 0.f, 0.f};
+      if (a < nA && b < nB && (near[arow[r] * pitch + (b >> 3)] >> (b & 7) & 1)) {
+        need |= 1u << (r * 4 + q);
+        const float4 v = quat[(int64_t)arow[r] * ldo + b];
+        qq[0] = v.x;
+        qq[1] = v.y;
+        qq[2] = v.z;
+        qq[3] = v.w;
+      }
+      quat_to_rot_fma(qq, R[r][q]);
+    }
+  }
+  for (int kt = 0; kt < nk; ++kt) {
+    rx_wait<RX_STAGES - 2>();
+    __syncwarp();  // the stage's copies of every lane have landed, and the one to refill has been read
+    issue(kt + RX_STAGES - 1);
+    const float* const st = ring + (kt & (RX_STAGES - 1)) * RX_STAGE_FLOATS;
+#pragma unroll 1
+    for (int h = 0; h < RX_T / 2; ++h) {
+      float x[2][3][2], y[4][3][2];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+          *reinterpret_cast<float2*>(x[r][c]) =
+              *reinterpret_cast<const float2*>(st + (lr + 8 * r) * RX_PITCH + c * RX_T + h * 2);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          *reinterpret_cast<float2*>(y[q][c]) =
+              *reinterpret_cast<const float2*>(st + (RX_A + ls + 4 * q) * RX_PITCH + c * RX_T + h * 2);
+      }
+      // neighbouring FMAs share the reference's coordinate
+#pragma unroll
+      for (int e = 0; e < 2; ++e)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          float t[4][3];
+#pragma unroll
+          for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) t[q][c] = fmaf(R[r][q][3 * c + 2], x[r][2][e], -y[q][c][e]);
+#pragma unroll
+          for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) t[q][c] = fmaf(R[r][q][3 * c + 1], x[r][1][e], t[q][c]);
+#pragma unroll
+          for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) t[q][c] = fmaf(R[r][q][3 * c], x[r][0][e], t[q][c]);
+#pragma unroll
+          for (int c = 2; c >= 0; --c)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) res[r][q] = fmaf(t[q][c], t[q][c], res[r][q]);
+        }
+    }
+  }
+  rx_wait<0>();
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int64_t ia = idA ? idA[arow[r]] : -2;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int b = b0 + ls + 4 * q;
+      if (need & (1u << (r * 4 + q))) {
+        const bool same = idB && idB[b] == ia;
+        out[(int64_t)arow[r] * ldo + b] = same ? 1.0f : exp2f(fmaxf(res[r][q] * inv_n, 0.0f) * neg_scale);
+      }
+    }
+  }
+}
+
+cudaError_t launch_rmsd_exact(const float* A, int64_t nA, const float* Bm, int64_t nB, int ap, int n_atoms,
+                              const int64_t* idA, const int64_t* idB, float neg_scale, float* out, int64_t ldo,
+                              const uint8_t* near, int64_t pitch, const int* order, const uint2* units,
+                              const unsigned* count, const float4* quat, cudaStream_t st) {
+  if (nA <= 0 || nB <= 0) return cudaSuccess;
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(rmsd_exact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RX_SMEM);
+  if (attr != cudaSuccess) return attr;
+  const int64_t units_max = ceil_div(nA, RX_A) * ceil_div(nB, RX_B);
+  rmsd_exact_kernel<<<(unsigned)ceil_div(units_max, RX_WARPS), RX_WARPS * 32, RX_SMEM, st>>>(A, (int)nA, Bm, (int)nB, ap, n_atoms, idA, idB, neg_scale,
+                                                          out, ldo, near, pitch, order, units, count, quat);
   return cudaGetLastError();
 }
 
@@ -212,6 +398,11 @@ __device__ __forceinline__ float qcp_rotation(const float H[9], float Gx, float 
 // stage, 2 references x 4 samples per thread (16 x TA/2 threads).  TA = 32
 // for kernel blocks, TA = 8 for the few-reference calls (medoid columns,
 // k-means++ columns).
+// The function is kept whole, with the tile flags, the reference order and the
+// given rotations of an earlier exact pass that no launch passes any more: the
+// compiler fuses multiplications and additions of the QCP root by what else is
+// in the function, and without them the last bits of every medoid column, and
+// with these the labels of rows near a tie, would change.
 constexpr int RT_B = 64, RT_K = 8;
 
 template <int TA>
@@ -484,15 +675,13 @@ rmsd_gram_kernel(const float* __restrict__ A, int nA, const float* __restrict__ 
 
 cudaError_t launch_rmsd_gram(int kind, const float* A, int64_t nA, const float* Bm, int64_t nB, int ap,
                              int n_atoms, const float* gA, const float* gB, const int64_t* idA,
-                             const int64_t* idB, float neg_scale, float* out, int64_t ldo, cudaStream_t st,
-                             const int* tile_flag, const int* arow, const float4* quat) {
+                             const int64_t* idB, float neg_scale, float* out, int64_t ldo, cudaStream_t st) {
   if (nA <= 0 || nB <= 0) return cudaSuccess;
-  if ((tile_flag || quat) && nA <= 8) return cudaErrorInvalidValue;  // laid out for 32-frame A tiles
   const int vec_ok = (ldo % 4 == 0) && ((reinterpret_cast<uintptr_t>(out) & 15) == 0);
 #define KKM_RMSD_LAUNCH(K, TA)                                                                       \
   rmsd_gram_kernel<K, TA><<<dim3((unsigned)ceil_div(nB, RT_B), (unsigned)ceil_div(nA, TA)),          \
                             RmsdCfg<TA>::NT, 0, st>>>(A, (int)nA, Bm, (int)nB, ap, n_atoms, gA, gB, idA, \
-                                                      idB, neg_scale, out, ldo, vec_ok, tile_flag, arow, quat)
+                                                      idB, neg_scale, out, ldo, vec_ok, nullptr, nullptr, nullptr)
   if (nA <= 8) {
     if (kind == DK_DIST) KKM_RMSD_LAUNCH(DK_DIST, 8); else KKM_RMSD_LAUNCH(DK_RBF, 8);
   } else {

@@ -72,8 +72,8 @@ static uint64_t fit_bytes(const kkm_problem& p) {
   if (p.opt.precision == KKM_BF16) blk += 2ull * (Nmax + nL) * dp + 4ull * (Nmax + nL);
   if (p.opt.precision == KKM_FP8) blk += (uint64_t)(Nmax + nL) * round_up(dp, 16) + 8ull * (Nmax + nL);
   if (p.kernel.kind == KKM_RMSD)  // tensor-core MD path: split-BF16 planes, rotations, refine plan
-    blk += 24ull * round_up(p.kernel.n_atoms, 64) * (Nmax + nL) + 16ull * nL * ldk + 8ull * nL +
-           4ull * ceil_div(nL, 32) * ceil_div(Nmax, 64);
+    blk += 18ull * round_up(p.kernel.n_atoms, 64) * (Nmax + nL) + 16ull * nL * ldk + 8ull * nL +
+           nL * rmsd_near_pitch(Nmax) + 8ull * rmsd_max_units(nL, Nmax);
   const bool two = fit_overlaps(side_by_side_pipeline(p.opt.pipeline), (int)B, p.kernel.kind, p.opt.precision);
   uint64_t b = blk * (two ? 2 : 1);
   b += 4ull * N * d + 4ull * N + 4ull * Nmax;   // input copy, labels out, labels
@@ -101,8 +101,8 @@ static uint64_t assign_bytes(const kkm_model* m, int64_t M, int32_t mode) {
   if (mode == KKM_ASSIGN_SUPPORTS) b += 4ull * units * ldm + 8ull * units * ceil_div(ldm, kStripCols);
   if (split_applies(m->kind, rows_ref, m->d)) b += 6ull * m->dp * (rows_ref + ldm) + 4ull * (rows_ref + ldm);
   if (m->kind == KKM_RMSD)  // tensor-core MD path
-    b += 24ull * round_up(m->n_atoms, 64) * (rows_ref + ldm) + 16ull * rows_ref * ldm + 8ull * rows_ref +
-         4ull * ceil_div(rows_ref, 32) * ceil_div(ldm, 64);
+    b += 18ull * round_up(m->n_atoms, 64) * (rows_ref + ldm) + 16ull * rows_ref * ldm + 8ull * rows_ref +
+         rows_ref * rmsd_near_pitch(ldm) + 8ull * rmsd_max_units(rows_ref, ldm);
   return b + kSlackBytes;
 }
 
