@@ -2147,12 +2147,6 @@ static kkm_status kernel_matrix_impl(const float* A_in, int64_t nA, const float*
     if (!word_h[1]) return KKM_OK;
     // rows with NaN or Inf have no slices: the FFMA kernel below gives their values
   }
-  KKM_TRY(ws.alloc(&Ap, nA * sp.dp));
-  KKM_TRY(ws.alloc(&Bp, nB * sp.dp));
-  KKM_TRY(ws.alloc(&aA, nA));
-  KKM_TRY(ws.alloc(&aB, nB));
-  KKM_TRY(prep_rows(sp, A, 0, 1, nA, Ap, aA, st));
-  KKM_TRY(prep_rows(sp, Bm, 0, 1, nB, Bp, aB, st));
   int tc_err_h = 0;
   if (precision == KKM_BF16) {
     __nv_bfloat16 *Ab, *Bb;
@@ -2164,31 +2158,41 @@ static kkm_status kernel_matrix_impl(const float* A_in, int64_t nA, const float*
     KKM_TRY(ws.alloc(&nBb, nB));
     KKM_TRY(ws.alloc(&err, 1));
     KKM_CK(cudaMemsetAsync(err, 0, 4, st));
-    KKM_TRY(kernel_block_bf16(sp, Ap, nullptr, nA, Bp, nB, o, false, nB, Ab, nAb, Bb, nBb, err, st));
+    KKM_RUN("to_bf16", st, launch_rows_to_bf16(A, nA, Ab, nAb, Bm, nB, Bb, nBb, d, sp.dp, st));
+    KKM_TRY(kernel_block_bf16(sp, nullptr, nullptr, nA, nullptr, nB, o, false, nB, Ab, nAb, Bb, nBb, err, st, 0,
+                              /*converted=*/true));
     KKM_CK(cudaMemcpyAsync(&tc_err_h, err, 4, cudaMemcpyDeviceToHost, st));
-  } else if (precision == KKM_FP8) {
-    const int64_t ld8 = round_up(sp.dp, 16);
-    uint8_t *A8, *B8;
-    float *sA, *sB, *nA8, *nB8;
-    int* err;
-    KKM_TRY(ws.alloc(&A8, nA * ld8));
-    KKM_TRY(ws.alloc(&B8, nB * ld8));
-    KKM_TRY(ws.alloc(&sA, nA));
-    KKM_TRY(ws.alloc(&sB, nB));
-    KKM_TRY(ws.alloc(&nA8, nA));
-    KKM_TRY(ws.alloc(&nB8, nB));
-    KKM_TRY(ws.alloc(&err, 1));
-    KKM_CK(cudaMemsetAsync(err, 0, 4, st));
-    KKM_TRY(kernel_block_fp8(sp, Ap, nullptr, nA, Bp, nB, o, false, nB, A8, sA, nA8, B8, sB, nB8, err, st));
-    KKM_CK(cudaMemcpyAsync(&tc_err_h, err, 4, cudaMemcpyDeviceToHost, st));
-  } else if (sp.kind == KKM_RMSD && nA >= kRmsdTcMinRefs) {
-    // the MD kernel takes the same tensor-core estimate + exact-refine path as a fit
-    RmsdTcScratch rtc;
-    KKM_TRY(alloc_rmsd_tc(ws, sp, nA, nB, nB, &rtc));
-    KKM_TRY(kernel_block(sp, Ap, aA, nullptr, nA, Bp, aB, nullptr, nB, o, nB, st, false, false, &rtc));
-    KKM_CK(cudaMemcpyAsync(&tc_err_h, rtc.err, 4, cudaMemcpyDeviceToHost, st));
   } else {
-    KKM_TRY(kernel_block(sp, Ap, aA, nullptr, nA, Bp, aB, nullptr, nB, o, nB, st));
+    KKM_TRY(ws.alloc(&Ap, nA * sp.dp));
+    KKM_TRY(ws.alloc(&Bp, nB * sp.dp));
+    KKM_TRY(ws.alloc(&aA, nA));
+    KKM_TRY(ws.alloc(&aB, nB));
+    KKM_TRY(prep_rows(sp, A, 0, 1, nA, Ap, aA, st));
+    KKM_TRY(prep_rows(sp, Bm, 0, 1, nB, Bp, aB, st));
+    if (precision == KKM_FP8) {
+      const int64_t ld8 = round_up(sp.dp, 16);
+      uint8_t *A8, *B8;
+      float *sA, *sB, *nA8, *nB8;
+      int* err;
+      KKM_TRY(ws.alloc(&A8, nA * ld8));
+      KKM_TRY(ws.alloc(&B8, nB * ld8));
+      KKM_TRY(ws.alloc(&sA, nA));
+      KKM_TRY(ws.alloc(&sB, nB));
+      KKM_TRY(ws.alloc(&nA8, nA));
+      KKM_TRY(ws.alloc(&nB8, nB));
+      KKM_TRY(ws.alloc(&err, 1));
+      KKM_CK(cudaMemsetAsync(err, 0, 4, st));
+      KKM_TRY(kernel_block_fp8(sp, Ap, nullptr, nA, Bp, nB, o, false, nB, A8, sA, nA8, B8, sB, nB8, err, st));
+      KKM_CK(cudaMemcpyAsync(&tc_err_h, err, 4, cudaMemcpyDeviceToHost, st));
+    } else if (sp.kind == KKM_RMSD && nA >= kRmsdTcMinRefs) {
+      // the MD kernel takes the same tensor-core estimate + exact-refine path as a fit
+      RmsdTcScratch rtc;
+      KKM_TRY(alloc_rmsd_tc(ws, sp, nA, nB, nB, &rtc));
+      KKM_TRY(kernel_block(sp, Ap, aA, nullptr, nA, Bp, aB, nullptr, nB, o, nB, st, false, false, &rtc));
+      KKM_CK(cudaMemcpyAsync(&tc_err_h, rtc.err, 4, cudaMemcpyDeviceToHost, st));
+    } else {
+      KKM_TRY(kernel_block(sp, Ap, aA, nullptr, nA, Bp, aB, nullptr, nB, o, nB, st));
+    }
   }
   if (host_out) KKM_CK(cudaMemcpyAsync(out, o, (size_t)nA * nB * 4, cudaMemcpyDeviceToHost, st));
   KKM_CK(cudaStreamSynchronize(st));

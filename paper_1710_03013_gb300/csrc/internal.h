@@ -308,6 +308,9 @@ cudaError_t launch_to_fp8(const float* src, int64_t n, int dp, int ld8, uint8_t*
 // BF16 copy of FP32 rows [n][dp] with the squared norms of the rounded rows.
 cudaError_t launch_to_bf16(const float* src, int64_t n, int dp, __nv_bfloat16* dst, float* normsq,
                            cudaStream_t st);
+// The same for two sets of unpadded rows [n][d] in one launch (padded to dp).
+cudaError_t launch_rows_to_bf16(const float* XA, int64_t nA, __nv_bfloat16* A, float* nrmA, const float* XB, int64_t nB,
+                                __nv_bfloat16* B, float* nrmB, int64_t d, int dp, cudaStream_t st);
 
 // ---- MD kernel (RMSD) -----------------------------------------------------
 // Frames [n][n_atoms][3] (rows start + l*step of X) -> centred SoA [n][3][ap]
