@@ -22,9 +22,13 @@
 // (4.2e-8), blobs 100 from the origin 1.6e-5 (2.4e-5).
 //
 // What bounds it: six FP16 products of 2 d flop per entry.  At 784 values a
-// 3,001 x 15,013 block takes 0.293 ms (1.45 PFLOP/s of FP16 products, 0.76 of
+// 3,001 x 15,013 block takes 0.27 ms (1.57 PFLOP/s of FP16 products, 0.82 of
 // the measured BF16 rate) against 1.57 ms for the FFMA kernel (45 of the 74
-// TFLOP/s that independent FFMAs reach).
+// TFLOP/s that independent FFMAs reach).  A tile's exponentials and stores took
+// 20,000 clocks as one chain behind a column test each, longer than the 8
+// stages of MMAs that cover them, so the next chunk waited 4,300: computed in
+// eights without the test (full tiles) and with an elected issuer it is 0.27
+// instead of 0.29 ms.  Pairs of SMs (cta_group::2) measured 0.29-0.31 ms.
 //
 // Structure (persistent, one CTA of ten warps per SM, 128 samples x 256
 // references): warp 0 fills three 72 KB stages by TMA (32 values of K, the
@@ -85,7 +89,7 @@ struct SplitShared {
   uint64_t rempty;         // the other products' sums of a tile read
   uint32_t tmem_base;
   int abort_flag;
-  float nP[8][128], sP[8][128];  // norms and scales of a warp's references
+  float2 ns[8][128];  // norm and scale of a warp's references
 };
 
 template <int SP_N>
@@ -158,7 +162,8 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer
-    if (lane == 0) {
+    {
+      const bool issuer = elect_one();
       int s = 0;
       uint32_t ph = 0, hph = 1, rph = 1;  // parities of the next "read" waits
       bool ok = true;
@@ -175,18 +180,21 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
           tc_fence_after();
           const uint32_t a = smem_u32(stages + (size_t)s * SP_STAGE_BYTES);
           const uint32_t b = a + 3 * SP_A_BYTES;
+          if (issuer) {
 #pragma unroll
-          for (int k = 0; k < SP_K / 16; ++k) {
-            const uint64_t ah = sw64_desc(a + k * 32), am = sw64_desc(a + SP_A_BYTES + k * 32),
-                           al = sw64_desc(a + 2 * SP_A_BYTES + k * 32);
-            const uint64_t bh = sw64_desc(b + k * 32), bm = sw64_desc(b + SP_B_BYTES + k * 32),
-                           bl = sw64_desc(b + 2 * SP_B_BYTES + k * 32);
-            umma_f16(dr, al, bh, idesc, (kb | k) != 0);
-            umma_f16(dr, ah, bl, idesc, 1);
-            umma_f16(dr, am, bm, idesc, 1);
-            umma_f16(dr, am, bh, idesc, 1);
-            umma_f16(dr, ah, bm, idesc, 1);
+            for (int k = 0; k < SP_K / 16; ++k) {
+              const uint64_t ah = sw64_desc(a + k * 32), am = sw64_desc(a + SP_A_BYTES + k * 32),
+                             al = sw64_desc(a + 2 * SP_A_BYTES + k * 32);
+              const uint64_t bh = sw64_desc(b + k * 32), bm = sw64_desc(b + SP_B_BYTES + k * 32),
+                             bl = sw64_desc(b + 2 * SP_B_BYTES + k * 32);
+              umma_f16(dr, al, bh, idesc, (kb | k) != 0);
+              umma_f16(dr, ah, bl, idesc, 1);
+              umma_f16(dr, am, bm, idesc, 1);
+              umma_f16(dr, am, bh, idesc, 1);
+              umma_f16(dr, ah, bm, idesc, 1);
+            }
           }
+          __syncwarp();
           const bool first = kb % SP_CHUNK == 0;
           if (first) {
             if (!mbar_wait(&sh.hempty, hph, &sh.abort_flag)) {
@@ -196,19 +204,22 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
             hph ^= 1u;
             tc_fence_after();
           }
+          if (issuer) {
 #pragma unroll
-          for (int k = 0; k < SP_K / 16; ++k)
-            umma_f16(dh, sw64_desc(a + k * 32), sw64_desc(b + k * 32), idesc, !(first && k == 0));
-          umma_commit(&sh.empty[s]);
+            for (int k = 0; k < SP_K / 16; ++k)
+              umma_f16(dh, sw64_desc(a + k * 32), sw64_desc(b + k * 32), idesc, !(first && k == 0));
+            umma_commit(&sh.empty[s]);
+            if (kb % SP_CHUNK == SP_CHUNK - 1 || kb == nk - 1) umma_commit(&sh.hfull);
+          }
+          __syncwarp();
           if (++s == SP_STAGES) {
             s = 0;
             ph ^= 1u;
           }
-          if (kb % SP_CHUNK == SP_CHUNK - 1 || kb == nk - 1) umma_commit(&sh.hfull);
         }
       }
       if (!ok) {
-        atomicExch(err, 2);
+        if (issuer) atomicExch(err, 2);
         sh.abort_flag = 1;
       }
     }
@@ -225,8 +236,7 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
       __syncwarp();
       for (int c = lane; c < SP_N / 2; c += 32) {
         const int n = n0 + c;
-        sh.nP[ew][c] = n < nP ? normP[n] : 0.0f;
-        sh.sP[ew][c] = n < nP ? scaleP[n] : 0.0f;
+        sh.ns[ew][c] = n < nP ? make_float2(normP[n], scaleP[n]) : make_float2(0.0f, 0.0f);
       }
       __syncwarp();
       float tot[SP_N / 2];
@@ -276,13 +286,24 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
       if (m < nQ) {
         const float nq = normQ[m], sq = scaleQ[m];
         float* o = out + (int64_t)n0 * ldo + m;
+        auto value = [&](int c) {
+          const float2 ns = sh.ns[ew][c];
+          const float dot = tot[c] * sq * ns.y;
+          return exp2f(fmaxf(nq + ns.x - 2.0f * dot, 0.0f) * neg_scale);
+        };
+        if (ncols >= SP_N / 2) {
 #pragma unroll
-        for (int c = 0; c < SP_N / 2; ++c) {
-          if (c < ncols) {
-            const float dot = tot[c] * sq * sh.sP[ew][c];
-            const float d2 = fmaxf(nq + sh.nP[ew][c] - 2.0f * dot, 0.0f);
-            o[(int64_t)c * ldo] = exp2f(d2 * neg_scale);
+          for (int c = 0; c < SP_N / 2; c += 8) {  // eight chains of exponentials at a time, then their stores
+            float v[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] = value(c + e);
+#pragma unroll
+            for (int e = 0; e < 8; ++e, o += ldo) st_global(o, v[e]);
           }
+        } else {
+#pragma unroll
+          for (int c = 0; c < SP_N / 2; ++c, o += ldo)
+            if (c < ncols) *o = value(c);
         }
       }
     }
