@@ -50,7 +50,9 @@ typedef enum kkm_status {
 typedef enum kkm_kernel_kind { KKM_RBF = 0, KKM_RMSD = 1, KKM_LINEAR = 2 } kkm_kernel_kind;
 
 /* Arithmetic of the kernel-block evaluation K(X^i, L).  KKM_FP32 is the
- * plain FFMA path.  KKM_BF16 (RBF and linear kernels) runs the Gram product
+ * FP32 path: FFMA, or for the Gaussian blocks of kkm_kernel_matrix and
+ * kkm_assign (more than 32 reference rows, d >= 64) FP16 products of three
+ * slices of each row on the tensor cores, as accurate as FFMA.  KKM_BF16 (RBF and linear kernels) runs the Gram product
  * on the tensor cores from BF16-rounded rows with FP32 accumulation; the
  * C-column blocks (Eq. 8, 12, k-means++) and all sums stay FP32/FP64.
  * KKM_FP8 (RBF and linear kernels) runs it on e4m3 rows, each scaled by
