@@ -935,13 +935,6 @@ static kkm_status kmeanspp_dev(const KernelSpec& sp, const float* Xi, const floa
   double* P = D2 + Ni;
   double* bsum = P + Ni;
   if (sp.kind != KKM_RMSD) {
-    if (kpp_cluster_applies(Ni, sp.dp) && sp.dp <= 10240) {
-      if (C > 1)
-        KKM_RUN("kpp_round", st,
-                launch_kpp_cluster(Xi, sp.dp, Ni, sp.kind == KKM_LINEAR, sp.neg_scale(), kself, D2, P, bsum, picks,
-                                   draws_d, C, st));
-      return KKM_OK;
-    }
     for (int r = 1; r < C; ++r)
       KKM_RUN("kpp_round", st,
               launch_kpp_fused_round(Xi, sp.dp, Ni, sp.kind == KKM_LINEAR, sp.neg_scale(), kself, D2, P, bsum, picks,

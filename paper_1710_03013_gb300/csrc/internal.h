@@ -619,13 +619,6 @@ cudaError_t launch_kpp_round(const float* Kc, int N0, const float* kself, double
 // One whole k-means++ round on prepared rows (RBF or linear kernel), the next
 // pick drawn by the last CTA; *ticket is zero between launches.  D2 holds
 // N0 + N0 + ceil(N0 / 32) doubles (D^2, running sums, CTA totals).
-// All rounds r = 1 .. C - 1 in one launch (draws[1 .. C), picks[0] given), for
-// mini-batches of at most a few MB (kpp_cluster_applies) and rows of at most
-// 10,240 values.
-bool kpp_cluster_applies(int N0, int dp);
-cudaError_t launch_kpp_cluster(const float* X, int dp, int N0, bool linear, float neg_scale, const float* kself,
-                               double* D2, double* P, double* bsum, int32_t* picks, const double* draws, int C,
-                               cudaStream_t st);
 cudaError_t launch_kpp_fused_round(const float* X, int dp, int N0, bool linear, float neg_scale, const float* kself,
                                    double* D2, double* P, double* bsum, int32_t* picks, const double* draws, int r,
                                    uint32_t* ticket, cudaStream_t st);

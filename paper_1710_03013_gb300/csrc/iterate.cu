@@ -2244,31 +2244,18 @@ kpp_pick_kernel(const double* __restrict__ D2, const double* __restrict__ P,
 // is 0, the lowest sample not picked yet.
 constexpr int kKppSamples = 32;  // samples per CTA of the one-launch round
 
-// The barrier of the kKppThreads threads that draw a pick: the CTA, or the
-// first eight warps of a larger one (named barrier 1).
-struct KppCtaSync {
-  __device__ __forceinline__ void operator()() const { __syncthreads(); }
-};
-struct KppPartSync {
-  __device__ __forceinline__ void operator()() const {
-    __syncwarp();
-    asm volatile("barrier.sync 1, %0;" ::"n"(kKppThreads) : "memory");
-  }
-};
-
-// inclusive scan of one double per thread over kKppThreads threads; sh holds
-// kKppThreads / 32 slots
-template <typename Sync>
-__device__ __forceinline__ double kpp_block_scan(double v, double* sh, Sync sync) {
+// inclusive scan of one double per thread over the CTA (kKppThreads); sh
+// holds kKppThreads / 32 slots
+__device__ __forceinline__ double kpp_block_scan(double v, double* sh) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const double y = __shfl_up_sync(kFull, v, o);
     if (lane >= o) v += y;
   }
-  sync();
+  __syncthreads();
   if (lane == 31) sh[w] = v;
-  sync();
+  __syncthreads();
   double off = 0.0;
   for (int q = 0; q < w; ++q) off += sh[q];
   return off + v;
@@ -2358,42 +2345,40 @@ __device__ __forceinline__ void kpp_group(const float* __restrict__ X, int dp, i
 // after) contains it; if rounding put the target at the very end, the last
 // sample with D^2 > 0; if every D^2 is 0, the lowest sample not picked yet
 // (picks[0..r) in global memory).
-template <typename Sync>
 __device__ int kpp_pick(int N0, int nb, const double* P, const double* bsum, const double* D2, const int32_t* picks,
-                        double u, int r, double* wsh, double* base_sh, double* total_sh, int* blk_sh, int* pick_sh,
-                        Sync sync) {
+                        double u, int r, double* wsh, double* base_sh, double* total_sh, int* blk_sh, int* pick_sh) {
   const int tid = threadIdx.x;
   double run = 0.0;
   for (int b0 = 0; b0 < nb; b0 += kKppThreads) {
     const double v = b0 + tid < nb ? __ldcg(bsum + b0 + tid) : 0.0;
-    const double incl = kpp_block_scan(v, wsh, sync);
+    const double incl = kpp_block_scan(v, wsh);
     if (tid == kKppThreads - 1) *total_sh = incl;
-    sync();
+    __syncthreads();
     run += *total_sh;
-    sync();
+    __syncthreads();
   }
   if (tid == 0) {
     *blk_sh = -1;
     *pick_sh = -1;
   }
-  sync();
+  __syncthreads();
   const double total = run;
   if (total > 0.0) {
     const double target = u * total;
     double before = 0.0;  // running sum of the earlier chunks
     for (int b0 = 0; b0 < nb; b0 += kKppThreads) {
       const double v = b0 + tid < nb ? __ldcg(bsum + b0 + tid) : 0.0;
-      const double incl = before + kpp_block_scan(v, wsh, sync);
+      const double incl = before + kpp_block_scan(v, wsh);
       const double excl = incl - v;
       if (b0 + tid < nb && excl <= target && incl > target) {
         *blk_sh = b0 + tid;
         *base_sh = excl;
       }
       if (tid == kKppThreads - 1) *total_sh = incl;
-      sync();
+      __syncthreads();
       before = *total_sh;
       const bool found = *blk_sh >= 0;
-      sync();
+      __syncthreads();
       if (found) break;
     }
     const int blk = *blk_sh;
@@ -2408,7 +2393,7 @@ __device__ int kpp_pick(int N0, int nb, const double* P, const double* bsum, con
       }
     }
   }
-  sync();
+  __syncthreads();
   if (tid == 0 && *pick_sh < 0) {
     if (total > 0.0) {  // rounding put the target at the very end
       int l = N0 - 1;
@@ -2425,122 +2410,8 @@ __device__ int kpp_pick(int N0, int nb, const double* P, const double* bsum, con
       }
     }
   }
-  sync();
+  __syncthreads();
   return *pick_sh;
-}
-
-// All rounds of kernel k-means++ in one launch by one cluster of eight CTAs, for
-// mini-batches small enough that a round is latency, not bandwidth.  A warp
-// takes whole groups of 32 samples (the same ones every round): the kernel
-// column of the last pick with as many lanes to a row as it has 16-byte
-// vectors (idle lanes of a full warp would only add zeros to the same tree),
-// the D^2 update and the group's running sums; the cluster meets, every CTA
-// draws the same pick from the groups' sums, and meets again.  The values,
-// their order and the picks are those of the one-launch-per-round kernel.
-//
-// What it is for: a fit of C clusters made C - 1 launches here, a third of all
-// launches of a batch of small problems, and the host queues those for 32 fits
-// at once.  Four rounds over 2,000 x 16 values 47 -> 36 us; 64 small problems
-// make 3,727 launches instead of 6,092, 33.1 -> 28.7 ms of fits without
-// iterations.  Beyond about 6 MB a round wants more SMs than a cluster has.
-constexpr int kKppCluster = 8;
-constexpr int kKppClusterWarps = 16;
-constexpr int64_t kKppClusterBytes = (int64_t)6 << 20;
-
-__device__ __forceinline__ void kpp_cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-// W lanes to a row (a power of two, at least its 16-byte vectors, or 32).
-template <int W>
-__global__ void __cluster_dims__(kKppCluster, 1, 1) __launch_bounds__(32 * kKppClusterWarps)
-kpp_cluster_kernel(const float* __restrict__ X, int dp, int N0, int linear, float neg_scale,
-                   const float* __restrict__ kself, double* __restrict__ D2, double* __restrict__ P,
-                   double* __restrict__ bsum, int32_t* __restrict__ picks, const double* __restrict__ draws, int C) {
-  extern __shared__ float4 kpp_row[];  // [dp / 4]: the row of the last pick
-  __shared__ float kv_sh[kKppClusterWarps][kKppSamples];
-  __shared__ double wsh[kKppThreads / 32];
-  __shared__ double base_sh, total_sh;
-  __shared__ int blk_sh, pick_sh;
-  constexpr int S = 32 / W;                    // samples per step of a warp
-  constexpr int U = W == 32 ? 4 : W >= 8 ? 4 : W == 4 ? 4 : 2;  // steps in flight
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int sub = lane / W, c_lane = lane % W;
-  const int d4 = dp >> 2;
-  const int nb = (N0 + kKppSamples - 1) / kKppSamples;
-  float* const kv = kv_sh[w];
-  int m = picks[0];
-  for (int r = 1; r < C; ++r) {
-    const float4* xm_g = reinterpret_cast<const float4*>(X + (int64_t)m * dp);
-    for (int c = tid; c < d4; c += 32 * kKppClusterWarps) kpp_row[c] = __ldg(xm_g + c);
-    __syncthreads();
-    const double km = kself ? (double)kself[m] : 1.0;
-    for (int g = blockIdx.x * kKppClusterWarps + w; g < nb; g += kKppCluster * kKppClusterWarps) {
-      const int l0 = g * kKppSamples;
-      const int l = l0 + lane;
-      const double ks = kself && l < N0 ? (double)kself[l] : 1.0;
-      const double old = r > 1 && l < N0 ? D2[l] : 0.0;
-      for (int s0 = 0; s0 < kKppSamples; s0 += S * U) {
-        const float4* xl[U];
-        float acc[U];
-#pragma unroll
-        for (int q = 0; q < U; ++q) {
-          const int ls = l0 + s0 + q * S + sub;
-          xl[q] = ls < N0 ? reinterpret_cast<const float4*>(X + (int64_t)ls * dp) : nullptr;
-          acc[q] = 0.0f;
-        }
-        for (int c = c_lane; c < (W == 32 ? (d4 + 31) / 32 * 32 : W); c += W) {
-          float4 v[U];
-#pragma unroll
-          for (int q = 0; q < U; ++q) v[q] = (xl[q] && c < d4) ? __ldg(xl[q] + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-          const float4 b = c < d4 ? kpp_row[c] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-#pragma unroll
-          for (int q = 0; q < U; ++q) {
-            const float4 a = v[q];
-            if (linear) {
-              acc[q] = fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, acc[q]))));
-            } else {
-              const float tx = a.x - b.x, ty = a.y - b.y, tz = a.z - b.z, tw = a.w - b.w;
-              acc[q] = fmaf(tx, tx, fmaf(ty, ty, fmaf(tz, tz, fmaf(tw, tw, acc[q]))));
-            }
-          }
-        }
-#pragma unroll
-        for (int q = 0; q < U; ++q) {
-          float a = acc[q];
-#pragma unroll
-          for (int o = W / 2; o > 0; o >>= 1) a += __shfl_xor_sync(kFull, a, o);
-          if (c_lane == 0) kv[s0 + q * S + sub] = linear ? a : (l0 + s0 + q * S + sub == m ? 1.0f : exp2f(a * neg_scale));
-        }
-      }
-      __syncwarp();
-      double dv = 0.0;
-      if (l < N0) {
-        double v = ks - 2.0 * (double)kv[lane] + km;
-        v = v > 0.0 ? v : 0.0;
-        dv = (r == 1) ? v : fmin(old, v);
-        D2[l] = dv;
-      }
-      double x = dv;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const double y = __shfl_up_sync(kFull, x, o);
-        if (lane >= o) x += y;
-      }
-      if (l < N0) P[l] = x;
-      if (lane == 31) bsum[g] = x;
-      __syncwarp();
-    }
-    kpp_cluster_sync();
-    if (tid < kKppThreads) {
-      const int pick =
-          kpp_pick(N0, nb, P, bsum, D2, picks, draws[r], r, wsh, &base_sh, &total_sh, &blk_sh, &pick_sh, KppPartSync());
-      if (tid == 0 && blockIdx.x == 0) picks[r] = pick;
-    }
-    // the sums have been read, and the pick written, in every CTA
-    kpp_cluster_sync();
-    m = pick_sh;
-  }
 }
 
 __global__ void __launch_bounds__(kKppThreads)
@@ -2567,7 +2438,7 @@ kpp_fused_round_kernel(const float* __restrict__ X, int dp, int N0, int linear, 
   if (!last_sh) return;
   __threadfence();
   const int pick = kpp_pick(N0, (int)gridDim.x, P, bsum, D2, picks, draws[r], r, wsh, &base_sh, &total_sh, &blk_sh,
-                            &pick_sh, KppCtaSync());
+                            &pick_sh);
   if (tid == 0) {
     picks[r] = pick;
     *ticket = 0u;
@@ -2588,27 +2459,6 @@ cudaError_t launch_kpp_fused_round(const float* X, int dp, int N0, bool linear, 
   }
   kpp_fused_round_kernel<<<nb, kKppThreads, smem, st>>>(X, dp, N0, linear ? 1 : 0, neg_scale, kself, D2, P, bsum,
                                                         picks, draws, r, ticket);
-  return cudaGetLastError();
-}
-
-bool kpp_cluster_applies(int N0, int dp) { return (int64_t)N0 * dp * 4 <= kKppClusterBytes; }
-
-cudaError_t launch_kpp_cluster(const float* X, int dp, int N0, bool linear, float neg_scale, const float* kself,
-                               double* D2, double* P, double* bsum, int32_t* picks, const double* draws, int C,
-                               cudaStream_t st) {
-  if (C <= 1) return cudaSuccess;
-  const size_t smem = (size_t)dp * sizeof(float);
-  if ((dp & 7) != 0 || (reinterpret_cast<uintptr_t>(X) & 15) != 0 || smem > 40 * 1024) return cudaErrorInvalidValue;
-  const int d4 = dp / 4;
-#define KKM_KPP(W)                                                                                                \
-  kpp_cluster_kernel<W><<<kKppCluster, 32 * kKppClusterWarps, smem, st>>>(X, dp, N0, linear ? 1 : 0, neg_scale, kself, \
-                                                                          D2, P, bsum, picks, draws, C)
-  if (d4 <= 2) KKM_KPP(2);
-  else if (d4 <= 4) KKM_KPP(4);
-  else if (d4 <= 8) KKM_KPP(8);
-  else if (d4 <= 16) KKM_KPP(16);
-  else KKM_KPP(32);
-#undef KKM_KPP
   return cudaGetLastError();
 }
 
