@@ -465,6 +465,15 @@ kkm_status kkm_debug_step(const float* Xb, int64_t Ni, int64_t d,
                           int32_t* n_out, double* omega_out,
                           int32_t* changed_out, void* stream);
 
+/* kkm_debug_kernel_matrix -- kkm_kernel_matrix with every pipeline wait of its
+ * tensor-core kernel limited to `polls` polls, for tests of the waits' limit:
+ * KKM_ETIMEOUT when one gave up (out is then undefined); the device and the
+ * stream stay usable. */
+kkm_status kkm_debug_kernel_matrix(const float* A, int64_t nA, const float* Bm,
+                                   int64_t nB, int64_t d, const kkm_kernel* k,
+                                   int32_t precision, uint32_t polls,
+                                   float* out, void* stream);
+
 /* kkm_debug_kmeanspp -- the kernel k-means++ picks kkm_fit makes on its first
  * mini-batch X0 [N0][d] for `seed`: picks_out [C] local indices (host). */
 kkm_status kkm_debug_kmeanspp(const float* X0, int64_t N0, int64_t d,

@@ -2103,7 +2103,8 @@ static kkm_status assign_impl(const kkm_model* m, const float* Xnew_in, int64_t 
 // kkm_kernel_matrix
 // ======================================================================
 static kkm_status kernel_matrix_impl(const float* A_in, int64_t nA, const float* B_in, int64_t nB, int64_t d,
-                                     const kkm_kernel* k, int32_t precision, float* out, cudaStream_t st) {
+                                     const kkm_kernel* k, int32_t precision, float* out, cudaStream_t st,
+                                     uint32_t polls = kTcSpinLimit) {
   KernelSpec sp;
   KKM_TRY(make_spec(k, d, &sp));
   if (precision != KKM_FP32 && precision != KKM_BF16 && precision != KKM_FP8)
@@ -2135,7 +2136,7 @@ static kkm_status kernel_matrix_impl(const float* A_in, int64_t nA, const float*
     KKM_TRY(alloc_split(ws, sp, nA, nB, &SA, &SB, &word));
     KKM_RUN("split_rows", st, launch_split_rows(SA, nA, SB, nB, d, sp.dp, word + 1, st));
     KKM_RUN("gram_split", st,
-            launch_gram_split(SA, nA, SB, nB, sp.dp, sp.neg_scale(), o, nB, word, sm_count(), st));
+            launch_gram_split(SA, nA, SB, nB, sp.dp, sp.neg_scale(), o, nB, word, sm_count(), st, polls));
     if (host_out) KKM_CK(cudaMemcpyAsync(out, o, (size_t)nA * nB * 4, cudaMemcpyDeviceToHost, st));
     KKM_CK(cudaMemcpyAsync(word_h, word, 8, cudaMemcpyDeviceToHost, st));
     KKM_CK(cudaStreamSynchronize(st));
@@ -2531,6 +2532,12 @@ kkm_status kkm_debug_step(const float* Xb, int64_t Ni, int64_t d, const int32_t*
     return debug_step_impl(Xb, Ni, d, L, nL, k, C, precision, iteration, u_in, u_out, fhat_out, margin_out, ghat_out,
                            n_out, omega_out, changed_out, (cudaStream_t)stream);
   });
+}
+
+kkm_status kkm_debug_kernel_matrix(const float* A, int64_t nA, const float* Bm, int64_t nB, int64_t d,
+                                   const kkm_kernel* k, int32_t precision, uint32_t polls, float* out, void* stream) {
+  set_error("");
+  return guarded([&] { return kernel_matrix_impl(A, nA, Bm, nB, d, k, precision, out, (cudaStream_t)stream, polls); });
 }
 
 kkm_status kkm_debug_kmeanspp(const float* X0, int64_t N0, int64_t d, const kkm_kernel* k, int32_t C, uint64_t seed,

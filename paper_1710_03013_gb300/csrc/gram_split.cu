@@ -38,7 +38,8 @@
 // the drain of the first one runs beside them; running totals live in
 // registers (128 per epilogue thread), so the next tile's MMAs start when the
 // accumulators are read, before the exponentials and the stores.
-// Every wait is bounded, as in the BF16 block.
+// Every wait is bounded, and the issuing warp's lanes leave a wait together; a
+// CTA ends only when its copies and MMAs have.
 #include <cuda.h>
 #include <cuda_fp16.h>
 
@@ -87,6 +88,7 @@ struct SplitShared {
   uint64_t full[SP_STAGES], empty[SP_STAGES];
   uint64_t hfull, hempty;  // hi.hi sums of a chunk ready / read
   uint64_t rempty;         // the other products' sums of a tile read
+  uint64_t mma_idle;       // every MMA of the CTA has finished
   uint32_t tmem_base;
   int abort_flag;
   float2 ns[8][128];  // norm and scale of a warp's references
@@ -97,7 +99,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1)
 gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapP, int nQ, int nP,
                   int dk, const float* __restrict__ normQ, const float* __restrict__ normP,
                   const float* __restrict__ scaleQ, const float* __restrict__ scaleP, float neg_scale,
-                  float* __restrict__ out, int64_t ldo, int* __restrict__ err) {
+                  float* __restrict__ out, int64_t ldo, int* __restrict__ err, uint32_t polls) {
   constexpr int SP_B_BYTES = SpCfg<SP_N>::kBBytes, SP_STAGE_BYTES = SpCfg<SP_N>::kStageBytes;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* const stages = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -115,6 +117,7 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
     mbar_init(&sh.hfull, 1);
     mbar_init(&sh.hempty, 8);
     mbar_init(&sh.rempty, 8);
+    mbar_init(&sh.mma_idle, 1);
     sh.abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -136,7 +139,7 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
       for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
         const int tm = t % tiles_m, tn = t / tiles_m;
         for (int kb = 0; kb < nk; ++kb) {
-          if (!mbar_wait(&sh.empty[s], ph ^ 1u, &sh.abort_flag)) {
+          if (!mbar_wait(&sh.empty[s], ph ^ 1u, &sh.abort_flag, polls)) {
             ok = false;
             break;
           }
@@ -159,6 +162,7 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
         atomicExch(err, 1);
         sh.abort_flag = 1;
       }
+      drain_copies(sh.full, SP_STAGES, s, ph, err);
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer
@@ -171,8 +175,8 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
       const uint32_t dh = tmem, dr = tmem + SP_N;
       for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
         for (int kb = 0; kb < nk; ++kb) {
-          if (!mbar_wait(&sh.full[s], ph, &sh.abort_flag) ||
-              (kb == 0 && !mbar_wait(&sh.rempty, rph, &sh.abort_flag))) {
+          if (!mbar_wait_warp(&sh.full[s], ph, &sh.abort_flag, polls) ||
+              (kb == 0 && !mbar_wait_warp(&sh.rempty, rph, &sh.abort_flag, polls))) {
             ok = false;
             break;
           }
@@ -197,7 +201,7 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
           __syncwarp();
           const bool first = kb % SP_CHUNK == 0;
           if (first) {
-            if (!mbar_wait(&sh.hempty, hph, &sh.abort_flag)) {
+            if (!mbar_wait_warp(&sh.hempty, hph, &sh.abort_flag, polls)) {
               ok = false;
               break;
             }
@@ -222,6 +226,7 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
         if (issuer) atomicExch(err, 2);
         sh.abort_flag = 1;
       }
+      if (issuer) drain_mmas(&sh.mma_idle, err);
     }
   } else {
     // ---------------- epilogue (warps 2..9)
@@ -243,7 +248,7 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
 #pragma unroll
       for (int c = 0; c < SP_N / 2; ++c) tot[c] = 0.0f;
       for (int ch = 0; ch < chunks; ++ch) {
-        if (lane == 0) ok = mbar_wait(&sh.hfull, hph, &sh.abort_flag);
+        if (lane == 0) ok = mbar_wait(&sh.hfull, hph, &sh.abort_flag, polls);
         ok = __shfl_sync(kFull, ok ? 1 : 0, 0) != 0;
         if (!ok) break;
         hph ^= 1u;
@@ -406,7 +411,7 @@ static bool split_map(CUtensorMap* map, const __half* base, int64_t n, int ks, i
 }
 
 cudaError_t launch_gram_split(const SplitRows& P, int64_t nP, const SplitRows& Q, int64_t nQ, int ks, float neg_scale,
-                              float* out, int64_t ldo, int* err, int n_sms, cudaStream_t st) {
+                              float* out, int64_t ldo, int* err, int n_sms, cudaStream_t st, uint32_t polls) {
   if (nP <= 0 || nQ <= 0) return cudaSuccess;
   if (ks % 8 != 0 || (reinterpret_cast<uintptr_t>(P.v) & 15) || (reinterpret_cast<uintptr_t>(Q.v) & 15) ||
       3 * nP > INT32_MAX || 3 * nQ > INT32_MAX)
@@ -420,7 +425,7 @@ cudaError_t launch_gram_split(const SplitRows& P, int64_t nP, const SplitRows& Q
     if (attr != cudaSuccess) return attr;                                                                      \
     const int64_t tiles = ceil_div(nQ, SP_M) * ceil_div(nP, N);                                                \
     gram_split_kernel<N><<<(unsigned)std::min<int64_t>(tiles, std::max(n_sms, 1)), SP_THREADS, SpCfg<N>::kSmem, st>>>( \
-        mq, mp, (int)nQ, (int)nP, ks, Q.norm, P.norm, Q.scale, P.scale, neg_scale, out, ldo, err);             \
+        mq, mp, (int)nQ, (int)nP, ks, Q.norm, P.norm, Q.scale, P.scale, neg_scale, out, ldo, err, polls);      \
   } while (0)
   if (2 * ceil_div(nQ, SP_M) * ceil_div(nP, 256) <= n_sms) KKM_SPLIT_LAUNCH(64);
   else KKM_SPLIT_LAUNCH(256);

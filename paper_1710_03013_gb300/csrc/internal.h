@@ -234,6 +234,10 @@ cudaError_t launch_gram_rbf_half(const float* A, int64_t nA, const float* Bm, in
                                  const float* normB, const int64_t* idA, const int64_t* idB, float neg_scale,
                                  __half* out, int64_t ldo, cudaStream_t st, float* out32 = nullptr);
 
+// Polls of a bounded mbarrier wait of the tensor-core kernels (seconds; the
+// kernels whose launcher takes `polls` can be given less, for tests).
+constexpr uint32_t kTcSpinLimit = 1u << 24;
+
 // ---- the FP32 Gaussian block on the tensor cores (gram_split.cu) ----------
 // FP32 rows X[r * ld .. + d) as three FP16 slices: v [3][n][ks] (ks = the row
 // length rounded up to 8), a power-of-two scale per row and the squared norms
@@ -252,7 +256,8 @@ cudaError_t launch_split_rows(const SplitRows& P, int64_t nP, const SplitRows& Q
                               int* bad, cudaStream_t st);
 // out[n*ldo + m] = exp(-|p_n - q_m|^2 / (2 sigma^2)); *err as launch_gram_tc.
 cudaError_t launch_gram_split(const SplitRows& P, int64_t nP, const SplitRows& Q, int64_t nQ, int ks, float neg_scale,
-                              float* out, int64_t ldo, int* err, int n_sms, cudaStream_t st);
+                              float* out, int64_t ldo, int* err, int n_sms, cudaStream_t st,
+                              uint32_t polls = kTcSpinLimit);
 // Whether kkm_kernel_matrix and kkm_assign take it for an FP32 Gaussian block
 // against nA reference rows of d values: a rule on the references alone, so
 // that a sample's values do not depend on how many samples share the call.  Up

@@ -10,18 +10,40 @@
 #include <stdint.h>
 
 #include "device_common.cuh"
+#include "internal.h"
 
 namespace kkm {
 
-constexpr uint32_t kTcSpinLimit = 1u << 24;  // polls of a bounded mbarrier wait
-
 // Bounded wait for the phase of the given parity; false on timeout or abort.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-  for (uint32_t it = 0; it < kTcSpinLimit; ++it) {
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                          uint32_t polls = kTcSpinLimit) {
+  for (uint32_t it = 0; it < polls; ++it) {
     if (mbar_try_wait(bar, parity)) return true;
     if ((it & 1023u) == 1023u && *abort_flag) return false;
   }
   return false;
+}
+// The same by a whole converged warp, with one answer for all its lanes: each
+// lane polls and gives up by itself, and a warp that split here would leave
+// some lanes at a warp barrier for lanes that have left the loop.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                               uint32_t polls) {
+  return __all_sync(kFull, mbar_wait(bar, parity, abort_flag, polls)) != 0;
+}
+// Before a CTA ends, whatever ended it: its copies in flight write its shared
+// memory and its MMAs in flight its tensor memory, so both are waited for, with
+// a limit of their own and whatever the abort flag says.
+__device__ __forceinline__ bool mbar_drain(uint64_t* bar, uint32_t parity) {
+  for (uint32_t it = 0; it < kTcSpinLimit; ++it)
+    if (mbar_try_wait(bar, parity)) return true;
+  return false;
+}
+// The TMA producer's last act: the newest copy of every stage has landed.  s
+// and ph are the next stage it would fill and that fill's parity (a stage never
+// filled is passed at once).
+__device__ __forceinline__ void drain_copies(uint64_t* full, int stages, int s, uint32_t ph, int* err) {
+  for (int i = 0; i < stages; ++i)
+    if (!mbar_drain(&full[i], i < s ? ph : ph ^ 1u)) atomicExch(err, 4);
 }
 __device__ __forceinline__ void tma_load_2d(const CUtensorMap* map, uint64_t* bar, void* dst, int c0, int c1) {
   asm volatile(
@@ -80,6 +102,12 @@ __device__ __forceinline__ void umma_fp8(uint32_t d_tmem, uint64_t adesc, uint64
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                : "memory");
+}
+// The MMA issuer's last act: every MMA it issued has finished (bar: one
+// arrival, used for nothing else).
+__device__ __forceinline__ void drain_mmas(uint64_t* bar, int* err) {
+  umma_commit(bar);
+  if (!mbar_drain(bar, 0u)) atomicExch(err, 5);
 }
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"

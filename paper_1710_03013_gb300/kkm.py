@@ -113,6 +113,8 @@ _SIGNATURES = {
                                     ctypes.POINTER(_F32)]),
     "kkm_debug_step": (_I32, [_P, _I64, _I64, _P, _I32, ctypes.POINTER(kkm_kernel), _I32, _I32, _I32, _P, _P,
                               _P, _P, _P, _P, ctypes.POINTER(_F64), ctypes.POINTER(_I32), _P]),
+    "kkm_debug_kernel_matrix": (_I32, [_P, _I64, _P, _I64, _I64, ctypes.POINTER(kkm_kernel), _I32, ctypes.c_uint32, _P,
+                                       _P]),
     "kkm_debug_kmeanspp": (_I32, [_P, _I64, _I64, ctypes.POINTER(kkm_kernel), _I32, _U64, _P, _P]),
     "kkm_minibatch_plan": (_I32, [_I64, _I32, _I32, _F64, _U64, _I32, ctypes.POINTER(_I64),
                                   ctypes.POINTER(_I64), ctypes.POINTER(_I64), _P, ctypes.POINTER(_I64)]),
@@ -639,8 +641,8 @@ def kkm_cost(model, X, mode="supports", stream=None):
     return out.value
 
 
-def kkm_kernel_matrix(A, B, kind="rbf", sigma=1.0, n_atoms=0, precision=KKM_FP32, stream=None):
-    """kkm_kernel_matrix of the C ABI: K(A, B) as [len(A)][len(B)] float32."""
+def kkm_kernel_matrix(A, B, kind="rbf", sigma=1.0, n_atoms=0, precision=KKM_FP32, stream=None, polls=None):
+    """kkm_kernel_matrix of the C ABI: K(A, B) as [len(A)][len(B)] float32 (polls: kkm_debug_kernel_matrix's limit)."""
     lib = load()
     nA, nB = int(A.shape[0]), int(B.shape[0])
     d = int(np.prod(A.shape[1:]))
@@ -655,7 +657,10 @@ def kkm_kernel_matrix(A, B, kind="rbf", sigma=1.0, n_atoms=0, precision=KKM_FP32
         op = ctypes.c_void_p(out.ctypes.data)
     k = _kernel(kind, sigma, n_atoms)
     st = stream if stream is not None else _stream_of(A)
-    _check(lib.kkm_kernel_matrix(ap, nA, bp, nB, d, ctypes.byref(k), int(precision), op, st))
+    if polls is None:
+        _check(lib.kkm_kernel_matrix(ap, nA, bp, nB, d, ctypes.byref(k), int(precision), op, st))
+    else:
+        _check(lib.kkm_debug_kernel_matrix(ap, nA, bp, nB, d, ctypes.byref(k), int(precision), int(polls), op, st))
     del ka, kb
     return out
 
