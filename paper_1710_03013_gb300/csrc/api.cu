@@ -608,6 +608,7 @@ struct RmsdTcScratch {
   int* err = nullptr;
   int64_t nP_cap = 0, nQ_cap = 0, ld_cap = 0, pitch = 0;
   int kp = 0;
+  uint32_t polls = kTcSpinLimit;
 };
 
 // Reference sets at least this large take the tensor-core MD path, for
@@ -682,7 +683,7 @@ static kkm_status rmsd_block_tc(const KernelSpec& sp, const float* A, const floa
   KKM_RUN("rmsd_to_bf16", st, launch_rmsd_to_bf16(Bm, nB, sp.ap, sp.n_atoms, t.Q, t.kp, 1, st));
   KKM_RUN(block ? "rmsd_block" : "rmsd_gram", st,
           launch_rmsd_screen(t.P, nA, t.Q, nB, 3 * t.kp, auxA, auxB, sp.n_atoms, sp.neg_scale(), out, t.quat,
-                             t.near, pitch, ldo, t.err, sm_count(), st));
+                             t.near, pitch, ldo, t.err, sm_count(), st, t.polls));
   KKM_RUN("rmsd_plan", st,
           launch_rmsd_refine_plan(t.near, pitch, (int)nA, (int)nB, t.key, t.order, t.units, t.count, st));
   KKM_RUN("rmsd_exact", st,
@@ -706,7 +707,8 @@ static kkm_status rmsd_block_tc(const KernelSpec& sp, const float* A, const floa
 static kkm_status kernel_block_bf16(const KernelSpec& sp, const float* P, const int32_t* L, int64_t nP,
                                     const float* Q, int64_t nQ, void* out, bool out_half, int64_t ldo,
                                     __nv_bfloat16* Pb, float* nPb, __nv_bfloat16* Qb, float* nQb, int* err,
-                                    cudaStream_t st, int n_sms = 0, bool converted = false) {
+                                    cudaStream_t st, int n_sms = 0, bool converted = false,
+                                    uint32_t polls = kTcSpinLimit) {
   if (!converted) {
     KKM_RUN("to_bf16", st, launch_to_bf16(P, nP, sp.dp, Pb, nPb, st));
     KKM_RUN("to_bf16", st, launch_to_bf16(Q, nQ, sp.dp, Qb, nQb, st));
@@ -714,7 +716,7 @@ static kkm_status kernel_block_bf16(const KernelSpec& sp, const float* P, const 
   const int dk = (int)sp.d;
   KKM_RUN("gram_block", st,
           launch_gram_tc(sp.kind == KKM_LINEAR ? DK_LINEAR : DK_RBF, Pb, nP, Qb, nQ, dk, sp.dp, nPb, nQb,
-                         sp.neg_scale(), out, out_half, ldo, err, n_sms > 0 ? n_sms : sm_count(), st));
+                         sp.neg_scale(), out, out_half, ldo, err, n_sms > 0 ? n_sms : sm_count(), st, polls));
   if (L && sp.kind != KKM_LINEAR) KKM_RUN("set_diag", st, launch_set_diag(out, out_half, ldo, L, (int)nP, st));
   return KKM_OK;
 }
@@ -725,7 +727,7 @@ static kkm_status kernel_block_bf16(const KernelSpec& sp, const float* P, const 
 static kkm_status kernel_block_fp8(const KernelSpec& sp, const float* P, const int32_t* L, int64_t nP, const float* Q,
                                    int64_t nQ, void* out, bool out_half, int64_t ldo, uint8_t* P8, float* sP,
                                    float* nP8, uint8_t* Q8, float* sQ, float* nQ8, int* err, cudaStream_t st,
-                                   bool converted = false) {
+                                   bool converted = false, uint32_t polls = kTcSpinLimit) {
   const int ld8 = (int)round_up(sp.dp, 16);
   if (!converted) {
     KKM_RUN("to_fp8", st, launch_to_fp8(P, nP, sp.dp, ld8, P8, sP, nP8, st));
@@ -733,7 +735,7 @@ static kkm_status kernel_block_fp8(const KernelSpec& sp, const float* P, const i
   }
   KKM_RUN("gram_block", st,
           launch_gram_tc_fp8(sp.kind == KKM_LINEAR ? DK_LINEAR : DK_RBF, P8, nP, Q8, nQ, (int)sp.d, ld8, nP8, nQ8, sP,
-                             sQ, sp.neg_scale(), out, out_half, ldo, err, sm_count(), st));
+                             sQ, sp.neg_scale(), out, out_half, ldo, err, sm_count(), st, polls));
   if (L && sp.kind != KKM_LINEAR) KKM_RUN("set_diag", st, launch_set_diag(out, out_half, ldo, L, (int)nP, st));
   return KKM_OK;
 }
@@ -2161,7 +2163,7 @@ static kkm_status kernel_matrix_impl(const float* A_in, int64_t nA, const float*
     KKM_CK(cudaMemsetAsync(err, 0, 4, st));
     KKM_RUN("to_bf16", st, launch_rows_to_bf16(A, nA, Ab, nAb, Bm, nB, Bb, nBb, d, sp.dp, st));
     KKM_TRY(kernel_block_bf16(sp, nullptr, nullptr, nA, nullptr, nB, o, false, nB, Ab, nAb, Bb, nBb, err, st, 0,
-                              /*converted=*/true));
+                              /*converted=*/true, polls));
     KKM_CK(cudaMemcpyAsync(&tc_err_h, err, 4, cudaMemcpyDeviceToHost, st));
   } else {
     KKM_TRY(ws.alloc(&Ap, nA * sp.dp));
@@ -2183,12 +2185,14 @@ static kkm_status kernel_matrix_impl(const float* A_in, int64_t nA, const float*
       KKM_TRY(ws.alloc(&nB8, nB));
       KKM_TRY(ws.alloc(&err, 1));
       KKM_CK(cudaMemsetAsync(err, 0, 4, st));
-      KKM_TRY(kernel_block_fp8(sp, Ap, nullptr, nA, Bp, nB, o, false, nB, A8, sA, nA8, B8, sB, nB8, err, st));
+      KKM_TRY(kernel_block_fp8(sp, Ap, nullptr, nA, Bp, nB, o, false, nB, A8, sA, nA8, B8, sB, nB8, err, st,
+                               /*converted=*/false, polls));
       KKM_CK(cudaMemcpyAsync(&tc_err_h, err, 4, cudaMemcpyDeviceToHost, st));
     } else if (sp.kind == KKM_RMSD && nA >= kRmsdTcMinRefs) {
       // the MD kernel takes the same tensor-core estimate + exact-refine path as a fit
       RmsdTcScratch rtc;
       KKM_TRY(alloc_rmsd_tc(ws, sp, nA, nB, nB, &rtc));
+      rtc.polls = polls;
       KKM_TRY(kernel_block(sp, Ap, aA, nullptr, nA, Bp, aB, nullptr, nB, o, nB, st, false, false, &rtc));
       KKM_CK(cudaMemcpyAsync(&tc_err_h, rtc.err, 4, cudaMemcpyDeviceToHost, st));
     } else {

@@ -31,8 +31,8 @@
 //               warp may access) and half (w - 2) / 4 of the 256 columns
 // Two accumulators of 256 columns let the epilogue of one tile overlap the
 // MMAs of the next.  Every mbarrier wait is bounded: on timeout the kernel
-// records an error code, stops issuing work, and still frees its tensor
-// memory before returning.
+// records an error code, stops issuing work, waits for its copies and MMAs in
+// flight, and still frees its tensor memory before returning.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
@@ -80,6 +80,7 @@ struct TcShared {
   uint64_t empty[TC_STAGES];
   uint64_t tfull[2];
   uint64_t tempty[2];
+  uint64_t mma_idle;        // every MMA of the CTA has finished
   uint32_t tmem_base;
   int abort_flag;
   float nP[8][TC_N / 2];    // reference norms of the current tile, per epilogue warp
@@ -94,7 +95,7 @@ template <int KIND, typename OutT, bool FP8 = false>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 gram_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapP,
                int nQ, int nP, int dk, const float* __restrict__ normQ, const float* __restrict__ normP,
-               float neg_scale, OutT* __restrict__ out, int64_t ldo, int* __restrict__ err,
+               float neg_scale, OutT* __restrict__ out, int64_t ldo, int* __restrict__ err, uint32_t polls,
                const float* __restrict__ scaleQ = nullptr, const float* __restrict__ scaleP = nullptr) {
   constexpr int EK = FP8 ? 2 * TC_K : TC_K;  // K elements per stage (128 bytes per row either way)
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -116,6 +117,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
       mbar_init(&sh.tfull[b], 1);
       mbar_init(&sh.tempty[b], 8);
     }
+    mbar_init(&sh.mma_idle, 1);
     sh.abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -137,7 +139,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
       for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
         const int tm = t % tiles_m, tn = t / tiles_m;
         for (int kb = 0; kb < nk; ++kb) {
-          if (!mbar_wait(&sh.empty[s], ph ^ 1u, &sh.abort_flag)) {
+          if (!mbar_wait(&sh.empty[s], ph ^ 1u, &sh.abort_flag, polls)) {
             ok = false;
             break;
           }
@@ -156,6 +158,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         atomicExch(err, 1);
         sh.abort_flag = 1;
       }
+      drain_copies(sh.full, TC_STAGES, s, ph, err);
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer
@@ -168,14 +171,14 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
       for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++lt) {
         const int buf = lt & 1;
         const uint32_t tph = (uint32_t)(lt >> 1) & 1u;
-        if (!mbar_wait(&sh.tempty[buf], tph ^ 1u, &sh.abort_flag)) {
+        if (!mbar_wait(&sh.tempty[buf], tph ^ 1u, &sh.abort_flag, polls)) {
           ok = false;
           break;
         }
         tc_fence_after();
         const uint32_t d_tmem = tmem + (uint32_t)(buf * TC_N);
         for (int kb = 0; kb < nk; ++kb) {
-          if (!mbar_wait(&sh.full[s], ph, &sh.abort_flag)) {
+          if (!mbar_wait(&sh.full[s], ph, &sh.abort_flag, polls)) {
             ok = false;
             break;
           }
@@ -202,6 +205,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         atomicExch(err, 2);
         sh.abort_flag = 1;
       }
+      drain_mmas(&sh.mma_idle, err);
     }
   } else {
     // ---------------- epilogue (warps 2..9)
@@ -221,7 +225,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
       }
       __syncwarp();
       bool ok = true;
-      if (lane == 0) ok = mbar_wait(&sh.tfull[buf], tph, &sh.abort_flag);
+      if (lane == 0) ok = mbar_wait(&sh.tfull[buf], tph, &sh.abort_flag, polls);
       ok = __shfl_sync(kFull, ok ? 1 : 0, 0) != 0;
       if (!ok) {
         if (lane == 0) {
@@ -313,13 +317,13 @@ static bool make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t c
 template <typename OutT>
 static cudaError_t launch_gram_tc_t(int kind, const CUtensorMap& mq, const CUtensorMap& mp, int nQ, int nP, int dk,
                                     const float* normP, const float* normQ, float neg_scale, OutT* out,
-                                    int64_t ldo, int* err, int grid, cudaStream_t st) {
+                                    int64_t ldo, int* err, int grid, cudaStream_t st, uint32_t polls) {
   cudaError_t e;
 #define KKM_TC_LAUNCH(K)                                                                                  \
   e = cudaFuncSetAttribute(gram_tc_kernel<K, OutT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM); \
   if (e != cudaSuccess) return e;                                                                         \
   gram_tc_kernel<K, OutT><<<grid, TC_THREADS, TC_SMEM, st>>>(mq, mp, nQ, nP, dk, normQ, normP, neg_scale, out, \
-                                                             ldo, err);
+                                                             ldo, err, polls);
   if (kind == DK_DIST) {
     KKM_TC_LAUNCH(DK_DIST)
   } else if (kind == DK_LINEAR) {
@@ -333,7 +337,7 @@ static cudaError_t launch_gram_tc_t(int kind, const CUtensorMap& mq, const CUten
 
 cudaError_t launch_gram_tc(int kind, const __nv_bfloat16* P, int64_t nP, const __nv_bfloat16* Q, int64_t nQ,
                            int dk, int ldb, const float* normP, const float* normQ, float neg_scale, void* out,
-                           bool out_half, int64_t ldo, int* err, int n_sms, cudaStream_t st) {
+                           bool out_half, int64_t ldo, int* err, int n_sms, cudaStream_t st, uint32_t polls) {
   if (nP <= 0 || nQ <= 0) return cudaSuccess;
   if ((ldb * 2) % 16 != 0 || (reinterpret_cast<uintptr_t>(P) & 15) || (reinterpret_cast<uintptr_t>(Q) & 15))
     return cudaErrorInvalidValue;
@@ -344,15 +348,15 @@ cudaError_t launch_gram_tc(int kind, const __nv_bfloat16* P, int64_t nP, const _
   const int grid = (int)std::min<int64_t>(tiles, std::max(n_sms, 1));
   if (out_half)
     return launch_gram_tc_t(kind, mq, mp, (int)nQ, (int)nP, dk, normP, normQ, neg_scale,
-                            static_cast<__half*>(out), ldo, err, grid, st);
+                            static_cast<__half*>(out), ldo, err, grid, st, polls);
   return launch_gram_tc_t(kind, mq, mp, (int)nQ, (int)nP, dk, normP, normQ, neg_scale, static_cast<float*>(out),
-                          ldo, err, grid, st);
+                          ldo, err, grid, st, polls);
 }
 
 cudaError_t launch_gram_tc_fp8(int kind, const uint8_t* P, int64_t nP, const uint8_t* Q, int64_t nQ, int dk, int ld8,
                                const float* normP, const float* normQ, const float* scaleP, const float* scaleQ,
                                float neg_scale, void* out, bool out_half, int64_t ldo, int* err, int n_sms,
-                               cudaStream_t st) {
+                               cudaStream_t st, uint32_t polls) {
   if (nP <= 0 || nQ <= 0) return cudaSuccess;
   if (ld8 % 16 != 0 || (reinterpret_cast<uintptr_t>(P) & 15) || (reinterpret_cast<uintptr_t>(Q) & 15))
     return cudaErrorInvalidValue;
@@ -368,7 +372,7 @@ cudaError_t launch_gram_tc_fp8(int kind, const uint8_t* P, int64_t nP, const uin
   e = cudaFuncSetAttribute(gram_tc_kernel<K, OT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM); \
   if (e != cudaSuccess) return e;                                                                                 \
   gram_tc_kernel<K, OT, true><<<grid, TC_THREADS, TC_SMEM, st>>>(mq, mp, (int)nQ, (int)nP, dk, normQ, normP,        \
-                                                                 neg_scale, static_cast<OT*>(out), ldo, err,     \
+                                                                 neg_scale, static_cast<OT*>(out), ldo, err, polls, \
                                                                  scaleQ, scaleP);
   if (kind == DK_LINEAR) {
     KKM_TC8(DK_LINEAR, float)

@@ -280,7 +280,8 @@ constexpr bool split_applies(int kind, int64_t nA, int64_t d) {
 // a nonzero code if a bounded wait gave up.
 cudaError_t launch_gram_tc(int kind, const __nv_bfloat16* P, int64_t nP, const __nv_bfloat16* Q, int64_t nQ,
                            int dk, int ldb, const float* normP, const float* normQ, float neg_scale, void* out,
-                           bool out_half, int64_t ldo, int* err, int n_sms, cudaStream_t st);
+                           bool out_half, int64_t ldo, int* err, int n_sms, cudaStream_t st,
+                           uint32_t polls = kTcSpinLimit);
 // MD kernel screen on the tensor cores: P [3 nP][dk] and Q [3 nQ][dk] hold
 // split-BF16 centred frames (planes x, y, z; dk = 3 segments of the padded
 // atom count, see launch_rmsd_to_bf16), gP / gQ their squared radii.
@@ -296,7 +297,7 @@ constexpr float kRmsdRefine = 1e-6f;
 cudaError_t launch_rmsd_screen(const __nv_bfloat16* P, int64_t nP, const __nv_bfloat16* Q, int64_t nQ, int dk,
                                const float* gP, const float* gQ, int n_atoms, float neg_scale, float* out,
                                float4* quat, uint8_t* near, int64_t pitch, int64_t ldo, int* err, int n_sms,
-                               cudaStream_t st);
+                               cudaStream_t st, uint32_t polls = kTcSpinLimit);
 // out[k*ldo + L[k]] = 1 (the exact diagonal of a Gaussian kernel block).
 cudaError_t launch_set_diag(void* out, bool out_half, int64_t ldo, const int32_t* L, int nL, cudaStream_t st);
 // FP8 e4m3 operands with a scale per row (rows [ld8] bytes, ld8 a multiple of
@@ -305,7 +306,7 @@ cudaError_t launch_set_diag(void* out, bool out_half, int64_t ldo, const int32_t
 cudaError_t launch_gram_tc_fp8(int kind, const uint8_t* P, int64_t nP, const uint8_t* Q, int64_t nQ, int dk, int ld8,
                                const float* normP, const float* normQ, const float* scaleP, const float* scaleQ,
                                float neg_scale, void* out, bool out_half, int64_t ldo, int* err, int n_sms,
-                               cudaStream_t st);
+                               cudaStream_t st, uint32_t polls = kTcSpinLimit);
 // e4m3 rows [n][ld8] of FP32 rows [n][dp] with a scale per row (max |x| /
 // 448) and the squared norms of the decoded rows.
 cudaError_t launch_to_fp8(const float* src, int64_t n, int dp, int ld8, uint8_t* dst, float* scale, float* normsq,

@@ -29,7 +29,8 @@
 // queue takes a stage of the ring).
 // The sums of each correlation entry are the same products in the same order.
 //
-// Every mbarrier wait is bounded, as in the BF16 block (gram_tc.cu).
+// Every mbarrier wait is bounded, and a CTA ends only when its copies and MMAs
+// have, as in the BF16 block (gram_tc.cu).
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -85,6 +86,7 @@ __device__ __forceinline__ void screen_tile(int64_t t, int tiles_m, int tiles_n,
 struct ScreenShared {
   uint64_t full[SC_STAGES], empty[SC_STAGES];
   uint64_t tfull[2], tempty[2];
+  uint64_t mma_idle;  // every MMA of the CTA has finished
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -93,7 +95,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1)
 rmsd_screen_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapP, int nQ, int nP,
                    int dk, const float* __restrict__ gQ, const float* __restrict__ gP, float n_r2_far,
                    float4* __restrict__ quat, int64_t ldo, uint32_t* __restrict__ near, int64_t pitch_words,
-                   int* __restrict__ err) {
+                   int* __restrict__ err, uint32_t polls) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* const stages = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ ScreenShared sh;
@@ -111,6 +113,7 @@ rmsd_screen_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
       mbar_init(&sh.tfull[b], 1);
       mbar_init(&sh.tempty[b], SC_EPI);
     }
+    mbar_init(&sh.mma_idle, 1);
     sh.abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -133,7 +136,7 @@ rmsd_screen_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
         int tm, tn;
       screen_tile(t, tiles_m, tiles_n, tm, tn);
         for (int kb = 0; kb < nk; ++kb) {
-          if (!mbar_wait(&sh.empty[s], ph ^ 1u, &sh.abort_flag)) {
+          if (!mbar_wait(&sh.empty[s], ph ^ 1u, &sh.abort_flag, polls)) {
             ok = false;
             break;
           }
@@ -153,6 +156,7 @@ rmsd_screen_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
         atomicExch(err, 1);
         sh.abort_flag = 1;
       }
+      drain_copies(sh.full, SC_STAGES, s, ph, err);
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer
@@ -163,14 +167,14 @@ rmsd_screen_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
       const uint32_t idesc = sc_idesc();
       for (int64_t t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++lt) {
         const int buf = lt & 1;
-        if (!mbar_wait(&sh.tempty[buf], ((uint32_t)(lt >> 1) & 1u) ^ 1u, &sh.abort_flag)) {
+        if (!mbar_wait(&sh.tempty[buf], ((uint32_t)(lt >> 1) & 1u) ^ 1u, &sh.abort_flag, polls)) {
           ok = false;
           break;
         }
         tc_fence_after();
         const uint32_t d_tmem = tmem + (uint32_t)(buf * 256);
         for (int kb = 0; kb < nk; ++kb) {
-          if (!mbar_wait(&sh.full[s], ph, &sh.abort_flag)) {
+          if (!mbar_wait(&sh.full[s], ph, &sh.abort_flag, polls)) {
             ok = false;
             break;
           }
@@ -192,6 +196,7 @@ rmsd_screen_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
         atomicExch(err, 2);
         sh.abort_flag = 1;
       }
+      drain_mmas(&sh.mma_idle, err);
     }
   } else {
     // ---------------- epilogue
@@ -209,7 +214,7 @@ rmsd_screen_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
       const float gy = valid ? gQ[sf] : 0.0f;
       bool ok = true;
       __syncwarp();
-      if (lane == 0) ok = mbar_wait(&sh.tfull[buf], (uint32_t)(lt >> 1) & 1u, &sh.abort_flag);
+      if (lane == 0) ok = mbar_wait(&sh.tfull[buf], (uint32_t)(lt >> 1) & 1u, &sh.abort_flag, polls);
       ok = __shfl_sync(kFull, ok ? 1 : 0, 0) != 0;
       if (!ok) {
         if (lane == 0) {
@@ -275,7 +280,7 @@ static bool screen_map(CUtensorMap* map, const __nv_bfloat16* base, int64_t n, i
 cudaError_t launch_rmsd_screen(const __nv_bfloat16* P, int64_t nP, const __nv_bfloat16* Q, int64_t nQ, int dk,
                                const float* gP, const float* gQ, int n_atoms, float neg_scale, float* out,
                                float4* quat, uint8_t* near, int64_t pitch, int64_t ldo, int* err, int n_sms,
-                               cudaStream_t st) {
+                               cudaStream_t st, uint32_t polls) {
   if (nP <= 0 || nQ <= 0) return cudaSuccess;
   if (dk % SC_K != 0 || (reinterpret_cast<uintptr_t>(P) & 15) || (reinterpret_cast<uintptr_t>(Q) & 15) || n_atoms <= 0 ||
       !quat || !near || pitch % 16 != 0 || 8 * pitch < nQ || 3 * (nP + SC_FP) > INT32_MAX || 3 * (nQ + SC_FQ) > INT32_MAX)
@@ -293,7 +298,8 @@ cudaError_t launch_rmsd_screen(const __nv_bfloat16* P, int64_t nP, const __nv_bf
   const float n_r2_far = (log2f(kRmsdRefine) / neg_scale) / (1.0f / (float)n_atoms);
   const int64_t tiles = ceil_div(nQ, SC_FQ) * ceil_div(nP, SC_FP);
   rmsd_screen_kernel<<<(unsigned)std::min<int64_t>(tiles, std::max(n_sms, 1)), SC_THREADS, SC_SMEM, st>>>(
-      mq, mp, (int)nQ, (int)nP, dk, gQ, gP, n_r2_far, quat, ldo, reinterpret_cast<uint32_t*>(near), pitch / 4, err);
+      mq, mp, (int)nQ, (int)nP, dk, gQ, gP, n_r2_far, quat, ldo, reinterpret_cast<uint32_t*>(near), pitch / 4, err,
+      polls);
   return cudaGetLastError();
 }
 

@@ -11,7 +11,7 @@ not at all.  Several tiles a CTA and several chunks of a row."""
 import numpy as np
 import pytest
 
-from synth import mnist_like
+from synth import md_trajectory, mnist_like
 
 pytestmark = pytest.mark.gpu
 
@@ -39,3 +39,18 @@ def test_fp32_slices(lib, nA, nB, d):
     X, _ = mnist_like(nA + nB, d, 5, problem=nA + d)
     Xd = torch.from_numpy(np.ascontiguousarray(X, np.float32)).to("cuda:0")
     _limits(lib, Xd[:nA].contiguous(), Xd[nA:].contiguous(), "rbf", 0.3 * np.sqrt(d), lib.KKM_FP32)
+
+
+@pytest.mark.parametrize("prec", ["bf16", "fp8"])
+def test_reduced_precision_block(lib, prec):
+    import torch
+    X, _ = mnist_like(20601, 600, 5, problem=6)
+    Xd = torch.from_numpy(np.ascontiguousarray(X, np.float32)).to("cuda:0")
+    _limits(lib, Xd[:600].contiguous(), Xd[600:].contiguous(), "rbf", 7.0, lib.KKM_BF16 if prec == "bf16" else lib.KKM_FP8)
+
+
+def test_md_screen(lib):
+    import torch
+    F, _ = md_trajectory(n_frames=9600, n_atoms=70, n_states=5, dwell=50.0, workload=83)
+    Xd = torch.from_numpy(np.ascontiguousarray(F.reshape(9600, -1), np.float32)).to("cuda:0")
+    _limits(lib, Xd[:600].contiguous(), Xd[600:].contiguous(), "rmsd", 1.5, lib.KKM_FP32, 70)
