@@ -1,25 +1,32 @@
 // The FP32 Gaussian kernel block on the tensor cores (tcgen05): FP32 rows in
-// three 9-bit slices, products exact where it matters.
+// three FP16 slices, products exact where it matters.
 //
 //   out[n][m] = exp(-max(0, |p|^2 + |q|^2 - 2 p.q) / (2 sigma^2))
 //
 // Every row is scaled by a power of two so that its largest |value| lies in
-// [2^14, 2^15), and a scaled value is cut into hi + mid + lo, multiples of
-// 2^7, 2^-2 and 2^-11 with at most 256 steps each (27 bits below the row's
-// maximum; FP16 holds each slice exactly, all normal numbers).  The product
-// p.q is then six FP16 products: hi.hi, hi.mid, mid.hi, mid.mid, hi.lo and
-// lo.hi (the three left out are below 2^-27 of the maxima).
+// [2^14, 2^15), and a scaled value is cut into hi + mid + lo: hi a multiple of
+// 2^7 with at most 256 steps, mid the rest (at most 64) rounded to FP16, lo
+// what mid leaves (at most 2^-6) rounded to FP16.  The product p.q is then six
+// FP16 products: hi.hi, hi.mid, mid.hi, mid.mid, hi.lo and lo.hi.  Slicing the
+// operands so that the leading products sum without error is the method of
+// Ozaki, Ogita, Oishi and Rump (Numer. Algorithms 59, 2012).
 //
 // Accuracy: a tensor-core accumulator drops the bits below its last place at
 // every step, which would bias a long FP32 sum by parts in 10^6.  hi.hi is
 // kept exact instead: its products are multiples of 2^14 of at most 2^16
-// steps, so 256 of them stay below 2^24 steps and no bit is dropped; every
-// 256 values of K the epilogue adds the accumulator to FP32 sums in registers
-// (rounded to nearest).  The other five products share a second accumulator
-// whose total is about 2^-9 of the first, and so are its dropped bits.
-// Measured against 64 bits (relative error of a block; FFMA kernel in
-// brackets): k/255 features of 784 values 8.3e-8 (9.1e-8), blobs 4.1e-8
-// (4.2e-8), blobs 100 from the origin 1.6e-5 (2.4e-5).
+// steps, so 256 of them stay below 2^24 steps and no bit is dropped.  The
+// other five products share a second accumulator, small for most rows and
+// never more than 80 steps long: every 256 values of K the epilogue adds both
+// to FP32 sums in registers (rounded to nearest).  The three products left out
+// (mid.lo and smaller) come to about 0.23 sqrt(2 d) in scaled units.  Measured
+// against 64 bits (rms error of the squared distance in 2^-24 (|p|^2 + |q|^2),
+// FFMA kernel in brackets): k/255 features of 784 values 0.82 (0.89), normal
+// values 0.83 (0.83), normal + 100 0.84 (1.28); rows whose largest value stands
+// far out, 0.1 to 0.4 with one 4.0 (64 values) 0.79 (0.86), with one 8.0 (784)
+// 0.83 (0.94), with one 30.0 0.69 (0.68), log-normal of sigma 2 0.85 (0.86) at
+// 784 and 0.89 (0.88) at 2,048 values.  (mid and lo as multiples of 2^-2 and
+// 2^-11 and one second sum per tile, as before, gave 1.63, 3.34, 1.78, 1.38
+// and 1.69 on those five.)
 //
 // What bounds it: six FP16 products of 2 d flop per entry.  At 784 values a
 // 3,001 x 15,013 block takes 0.27 ms (1.57 PFLOP/s of FP16 products, 0.82 of
@@ -35,9 +42,9 @@
 // three slices of both sides, 64-byte swizzle), warp 1 issues the MMAs, warps
 // 2..9 drain and finish.  hi.hi has tensor-memory columns 0..255, the rest
 // 256..511.  In a stage the ten MMAs of the second accumulator go first, so
-// the drain of the first one runs beside them; running totals live in
-// registers (128 per epilogue thread), so the next tile's MMAs start when the
-// accumulators are read, before the exponentials and the stores.
+// the drain of one accumulator runs beside MMAs into the other; running totals
+// live in registers (128 per epilogue thread), so the next tile's MMAs start
+// when the accumulators are read, before the exponentials and the stores.
 // Every wait is bounded, and the issuing warp's lanes leave a wait together; a
 // CTA ends only when its copies and MMAs have.
 #include <cuda.h>
@@ -87,7 +94,7 @@ __device__ __forceinline__ uint64_t sw64_desc(uint32_t saddr) {
 struct SplitShared {
   uint64_t full[SP_STAGES], empty[SP_STAGES];
   uint64_t hfull, hempty;  // hi.hi sums of a chunk ready / read
-  uint64_t rempty;         // the other products' sums of a tile read
+  uint64_t rfull, rempty;  // the other products' sums of a chunk ready / read
   uint64_t mma_idle;       // every MMA of the CTA has finished
   uint32_t tmem_base;
   int abort_flag;
@@ -116,6 +123,7 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
     }
     mbar_init(&sh.hfull, 1);
     mbar_init(&sh.hempty, 8);
+    mbar_init(&sh.rfull, 1);
     mbar_init(&sh.rempty, 8);
     mbar_init(&sh.mma_idle, 1);
     sh.abort_flag = 0;
@@ -175,12 +183,13 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
       const uint32_t dh = tmem, dr = tmem + SP_N;
       for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
         for (int kb = 0; kb < nk; ++kb) {
+          const bool first = kb % SP_CHUNK == 0, last = kb % SP_CHUNK == SP_CHUNK - 1 || kb == nk - 1;
           if (!mbar_wait_warp(&sh.full[s], ph, &sh.abort_flag, polls) ||
-              (kb == 0 && !mbar_wait_warp(&sh.rempty, rph, &sh.abort_flag, polls))) {
+              (first && !mbar_wait_warp(&sh.rempty, rph, &sh.abort_flag, polls))) {
             ok = false;
             break;
           }
-          if (kb == 0) rph ^= 1u;
+          if (first) rph ^= 1u;
           tc_fence_after();
           const uint32_t a = smem_u32(stages + (size_t)s * SP_STAGE_BYTES);
           const uint32_t b = a + 3 * SP_A_BYTES;
@@ -191,15 +200,15 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
                              al = sw64_desc(a + 2 * SP_A_BYTES + k * 32);
               const uint64_t bh = sw64_desc(b + k * 32), bm = sw64_desc(b + SP_B_BYTES + k * 32),
                              bl = sw64_desc(b + 2 * SP_B_BYTES + k * 32);
-              umma_f16(dr, al, bh, idesc, (kb | k) != 0);
+              umma_f16(dr, al, bh, idesc, !(first && k == 0));
               umma_f16(dr, ah, bl, idesc, 1);
               umma_f16(dr, am, bm, idesc, 1);
               umma_f16(dr, am, bh, idesc, 1);
               umma_f16(dr, ah, bm, idesc, 1);
             }
+            if (last) umma_commit(&sh.rfull);
           }
           __syncwarp();
-          const bool first = kb % SP_CHUNK == 0;
           if (first) {
             if (!mbar_wait_warp(&sh.hempty, hph, &sh.abort_flag, polls)) {
               ok = false;
@@ -213,7 +222,7 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
             for (int k = 0; k < SP_K / 16; ++k)
               umma_f16(dh, sw64_desc(a + k * 32), sw64_desc(b + k * 32), idesc, !(first && k == 0));
             umma_commit(&sh.empty[s]);
-            if (kb % SP_CHUNK == SP_CHUNK - 1 || kb == nk - 1) umma_commit(&sh.hfull);
+            if (last) umma_commit(&sh.hfull);
           }
           __syncwarp();
           if (++s == SP_STAGES) {
@@ -233,8 +242,26 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
     const int q = warp & 3, ew = warp - 2, half = ew >> 2;
     const uint32_t th = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * (SP_N / 2));
     const int chunks = (nk + SP_CHUNK - 1) / SP_CHUNK;
-    uint32_t hph = 0;
+    uint32_t cph = 0;
     bool ok = true;
+    // adds an accumulator's sums (when they are ready) to the totals and gives it back
+    float tot[SP_N / 2];
+    auto drain = [&](uint64_t* full, uint64_t* empty, int col) {
+      if (lane == 0) ok = mbar_wait(full, cph, &sh.abort_flag, polls);
+      ok = __shfl_sync(kFull, ok ? 1 : 0, 0) != 0;
+      if (!ok) return;
+      tc_fence_after();
+#pragma unroll
+      for (int c0 = 0; c0 < SP_N / 2; c0 += 32) {
+        uint32_t r[32];
+        tmem_ld32(th + (uint32_t)(col + c0), r);
+#pragma unroll
+        for (int c = 0; c < 32; ++c) tot[c0 + c] += __uint_as_float(r[c]);
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(empty);
+    };
     for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
       const int tm = t % tiles_m, tn = t / tiles_m;
       const int n0 = tn * SP_N + half * (SP_N / 2);
@@ -244,27 +271,13 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
         sh.ns[ew][c] = n < nP ? make_float2(normP[n], scaleP[n]) : make_float2(0.0f, 0.0f);
       }
       __syncwarp();
-      float tot[SP_N / 2];
 #pragma unroll
       for (int c = 0; c < SP_N / 2; ++c) tot[c] = 0.0f;
       for (int ch = 0; ch < chunks; ++ch) {
-        if (lane == 0) ok = mbar_wait(&sh.hfull, hph, &sh.abort_flag, polls);
-        ok = __shfl_sync(kFull, ok ? 1 : 0, 0) != 0;
+        drain(&sh.rfull, &sh.rempty, SP_N);
+        if (ok) drain(&sh.hfull, &sh.hempty, 0);
         if (!ok) break;
-        hph ^= 1u;
-        tc_fence_after();
-#pragma unroll
-        for (int c0 = 0; c0 < SP_N / 2; c0 += 32) {
-          uint32_t r[32];
-          tmem_ld32(th + (uint32_t)c0, r);
-#pragma unroll
-          for (int c = 0; c < 32; ++c) tot[c0 + c] += __uint_as_float(r[c]);
-        }
-        if (ch + 1 < chunks) {
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&sh.hempty);
-        }
+        cph ^= 1u;
       }
       if (!ok) {
         if (lane == 0) {
@@ -272,19 +285,6 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
           sh.abort_flag = 1;
         }
         break;
-      }
-#pragma unroll
-      for (int c0 = 0; c0 < SP_N / 2; c0 += 32) {
-        uint32_t r[32];
-        tmem_ld32(th + (uint32_t)(SP_N + c0), r);
-#pragma unroll
-        for (int c = 0; c < 32; ++c) tot[c0 + c] += __uint_as_float(r[c]);
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) {
-        mbar_arrive(&sh.hempty);
-        mbar_arrive(&sh.rempty);
       }
       const int m = tm * SP_M + q * 32 + lane;
       const int ncols = min(SP_N / 2, nP - n0);
@@ -375,11 +375,10 @@ __global__ void split_rows_kernel(SplitSource A, SplitSource B, int d, int ks, i
     for (int q = 0; q < 4; ++q) {
       const float hi = rintf(t[q] * 0x1p-7f) * 0x1p7f;
       const float r1 = t[q] - hi;  // exact
-      const float mid = rintf(r1 * 0x1p2f) * 0x1p-2f;
-      const float r2 = r1 - mid;   // exact
+      const __half mid = __float2half_rn(r1);
       h[0][q] = __float2half_rn(hi);
-      h[1][q] = __float2half_rn(mid);
-      h[2][q] = __float2half_rn(rintf(r2 * 0x1p11f) * 0x1p-11f);
+      h[1][q] = mid;
+      h[2][q] = __float2half_rn(r1 - __half2float(mid));  // an exact difference
     }
 #pragma unroll
     for (int w = 0; w < 3; ++w) *reinterpret_cast<uint2*>(o + w * slice + c) = *reinterpret_cast<const uint2*>(h[w]);
