@@ -52,7 +52,15 @@ typedef enum kkm_kernel_kind { KKM_RBF = 0, KKM_RMSD = 1, KKM_LINEAR = 2 } kkm_k
 /* Arithmetic of the kernel-block evaluation K(X^i, L).  KKM_FP32 is the
  * FP32 path: FFMA, or for the Gaussian blocks of kkm_kernel_matrix and
  * kkm_assign (more than 32 reference rows, d >= 64) FP16 products of three
- * slices of each row on the tensor cores, as accurate as FFMA.  KKM_BF16 (RBF and linear kernels) runs the Gram product
+ * slices of each row on the tensor cores, whose error against 64 bits is no
+ * larger than FFMA's: squared distances to about one unit of
+ * 2^-24 (|x|^2 + |y|^2) rms on either.  Rows that the slices do not hold as
+ * well (NaN, Inf, a squared norm outside the FP32 range, a largest value far
+ * above the rest: more than about 11 times the root mean square at d = 784,
+ * 7 times at d = 128) keep the FFMA sums; a value depends on its two rows
+ * alone.  kkm_cost and the fits use FFMA throughout, so a cost is the sum of
+ * kkm_assign's distances to FP32 rounding, not to the last bit.
+ * KKM_BF16 (RBF and linear kernels) runs the Gram product
  * on the tensor cores from BF16-rounded rows with FP32 accumulation; the
  * C-column blocks (Eq. 8, 12, k-means++) and all sums stay FP32/FP64.
  * KKM_FP8 (RBF and linear kernels) runs it on e4m3 rows, each scaled by

@@ -128,12 +128,6 @@ void prof_add_work(const char* name, double units) {
   g_prof[name].work += units;
 }
 
-#define KKM_RUN(name, st, call)                 \
-  do {                                          \
-    ::kkm::ProfScope _ps(name, st);             \
-    KKM_CK(call);                               \
-  } while (0)
-
 // First k entries of a partial Fisher-Yates shuffle of [0, n): step a swaps
 // positions a and a + floor(u (n - a)).  When k is small against n only the
 // positions the swaps touched are held (open addressing, identity elsewhere),
@@ -740,26 +734,24 @@ static kkm_status kernel_block_fp8(const KernelSpec& sp, const float* P, const i
   return KKM_OK;
 }
 
-// Scratch of the FP32 Gaussian block on the tensor cores, one allocation: the
-// slices, scales and (unless given) norms of nP references and nQ samples, and
-// two zeroed words (pipeline error, a row with NaN or Inf).
-static kkm_status alloc_split(Workspace& ws, const KernelSpec& sp, int64_t nP, int64_t nQ, SplitRows* P, SplitRows* Q,
-                              int** word) {
+// Scratch of the FP32 Gaussian block on the tensor cores for nP references and
+// nQ samples, one allocation.
+static kkm_status alloc_split(Workspace& ws, const KernelSpec& sp, int64_t nP, int64_t nQ, SplitScratch* t) {
   auto part = [](int64_t bytes) { return round_up(bytes, 256); };
   char* at;
-  KKM_TRY(ws.alloc(&at, 256 + part(6 * nP * sp.dp) + part(6 * nQ * sp.dp) + 2 * part(4 * nP) + 2 * part(4 * nQ)));
-  KKM_CK(cudaMemsetAsync(at, 0, 8, ws.st));
+  KKM_TRY(ws.alloc(&at, 256 + part(6 * nP * sp.dp) + part(6 * nQ * sp.dp) + 3 * part(4 * nP) + 3 * part(4 * nQ)));
   auto take = [&](int64_t bytes) {
     char* const p = at;
     at += part(bytes);
     return p;
   };
-  *word = reinterpret_cast<int*>(take(8));
-  for (SplitRows* s : {P, Q}) {
-    const int64_t n = s == P ? nP : nQ;
-    s->v = reinterpret_cast<__half*>(take(6 * n * sp.dp));
-    s->scale = reinterpret_cast<float*>(take(4 * n));
-    if (s->form_norm) s->norm = reinterpret_cast<float*>(take(4 * n));
+  t->words = reinterpret_cast<int*>(take(4 * kSplitWords));
+  for (SplitBufs* s : {&t->P, &t->Q}) {
+    s->cap = s == &t->P ? nP : nQ;
+    s->v = reinterpret_cast<__half*>(take(6 * s->cap * sp.dp));
+    s->scale = reinterpret_cast<float*>(take(4 * s->cap));
+    s->norm = reinterpret_cast<float*>(take(4 * s->cap));
+    s->rows = reinterpret_cast<int32_t*>(take(4 * s->cap));
   }
   return KKM_OK;
 }
@@ -2001,16 +1993,11 @@ static kkm_status assign_impl(const kkm_model* m, const float* Xnew_in, int64_t 
   // the FP32 Gaussian block on the tensor cores (kkm_cost keeps the FFMA block,
   // so that costs compare bit for bit with those of the fits' own kernels)
   const bool split = !omega_out && split_applies(sp.kind, rows_ref, d) && 3 * ldm <= INT32_MAX;
-  SplitRows SP, SX;
-  int* split_err = nullptr;
+  SplitScratch slices;
+  const SplitSide ref{mode == KKM_ASSIGN_SUPPORTS ? m->sup : m->med, sp.dp,
+                      mode == KKM_ASSIGN_SUPPORTS ? m->sup_aux : m->med_aux};
   if (split) {
-    const bool sup = mode == KKM_ASSIGN_SUPPORTS;
-    SP.X = sup ? m->sup : m->med;
-    SP.ld = sp.dp;
-    SP.norm = sup ? m->sup_aux : m->med_aux;
-    SP.form_norm = false;
-    SX.ld = d;
-    KKM_TRY(alloc_split(ws, sp, rows_ref, std::min(chunk, M), &SP, &SX, &split_err));
+    KKM_TRY(alloc_split(ws, sp, rows_ref, std::min(chunk, M), &slices));
   } else {
     KKM_TRY(ws.alloc(&Xc, ldm * sp.dp));
     KKM_TRY(ws.alloc(&auxc, ldm));
@@ -2040,23 +2027,8 @@ static kkm_status assign_impl(const kkm_model* m, const float* Xnew_in, int64_t 
     lb.I.ghat_in = m->ghat;
     lb.I.done = bad_d;
   }
-  for (int64_t c0 = 0; c0 < M; c0 += chunk) {
-    const int n = (int)std::min<int64_t>(chunk, M - c0);
-    if (split) {
-      SX.X = X + c0 * d;
-      KKM_RUN("split_rows", st,  // the references with the first chunk
-              launch_split_rows(SP, c0 == 0 ? rows_ref : 0, SX, n, d, sp.dp, nullptr, st));
-      KKM_RUN("gram_split", st,
-              launch_gram_split(SP, rows_ref, SX, n, sp.dp, sp.neg_scale(), Kb, ldm, split_err, sm_count(), st));
-    } else {
-      KKM_TRY(prep_rows(sp, X, c0, 1, n, Xc, auxc, st));
-      if (mode == KKM_ASSIGN_SUPPORTS)
-        KKM_TRY(kernel_block(sp, m->sup, m->sup_aux, nullptr, m->nL, Xc, auxc, nullptr, n, Kb, ldm, st, false, false,
-                             use_rtc ? &rtc : nullptr));
-      else
-        KKM_TRY(kernel_block(sp, m->med, m->med_aux, nullptr, C, Xc, auxc, nullptr, n, Kb, ldm, st, false, false,
-                             use_rtc ? &rtc : nullptr));
-    }
+  // labels and distances of rows c0 .. c0 + n - 1 from their kernel values
+  auto label = [&](int64_t c0, int n) -> kkm_status {
     if (mode == KKM_ASSIGN_SUPPORTS) {
       KKM_RUN("fhat_partial", st, launch_fhat_partial(Kb, ldm, n, lb.S, lb.I, st));
       KKM_RUN("assign", st,
@@ -2066,6 +2038,47 @@ static kkm_status assign_impl(const kkm_model* m, const float* Xnew_in, int64_t 
       KKM_RUN("nearest", st,
               launch_nearest(Kb, ldm, n, C, kself, sp.kind == KKM_LINEAR ? m->med_aux : nullptr, lab + c0,
                              dist + c0, st, bad_d));
+    }
+    return KKM_OK;
+  };
+  auto wide_pairs = [&](int64_t c0, int n) -> kkm_status {
+    KKM_RUN("gram_wide", st,
+            launch_gram_wide(slices, ref, rows_ref, SplitSide{X + c0 * d, d}, n, d, sp.dp, sp.neg_scale(), Kb, ldm,
+                             sm_count(), st));
+    return KKM_OK;
+  };
+  for (int64_t c0 = 0; c0 < M; c0 += chunk) {
+    const int n = (int)std::min<int64_t>(chunk, M - c0);
+    if (split) {
+      KKM_TRY(split_block(slices, ref, rows_ref, SplitSide{X + c0 * d, d}, n, d, sp.dp, sp.neg_scale(), Kb, ldm,
+                          /*p_ready=*/c0 > 0, sm_count(), st));
+      if (M > chunk) KKM_TRY(wide_pairs(c0, n));
+    } else {
+      KKM_TRY(prep_rows(sp, X, c0, 1, n, Xc, auxc, st));
+      if (mode == KKM_ASSIGN_SUPPORTS)
+        KKM_TRY(kernel_block(sp, m->sup, m->sup_aux, nullptr, m->nL, Xc, auxc, nullptr, n, Kb, ldm, st, false, false,
+                             use_rtc ? &rtc : nullptr));
+      else
+        KKM_TRY(kernel_block(sp, m->med, m->med_aux, nullptr, C, Xc, auxc, nullptr, n, Kb, ldm, st, false, false,
+                             use_rtc ? &rtc : nullptr));
+    }
+    KKM_TRY(label(c0, n));
+  }
+  int tc_err_h = 0;
+  bool waited = false;
+  if (split) {
+    int words_h[kSplitWords] = {};
+    KKM_CK(cudaMemcpyAsync(words_h, slices.words, sizeof words_h, cudaMemcpyDeviceToHost, st));
+    KKM_CK(cudaStreamSynchronize(st));
+    waited = true;
+    tc_err_h = words_h[kSplitErr];
+    // one chunk: its block is still there, and the pairs of wide rows are
+    // written into it only now that the wait has told of some (a launch that
+    // finds none is 6 us of a call of 100)
+    if (M <= chunk && (words_h[kSplitWideQ] || words_h[kSplitWideP])) {
+      KKM_TRY(wide_pairs(0, (int)M));
+      KKM_TRY(label(0, (int)M));
+      waited = false;
     }
   }
   if (omega_out || lab_host || dist_host) {  // nothing is copied out for bad input
@@ -2083,17 +2096,15 @@ static kkm_status assign_impl(const kkm_model* m, const float* Xnew_in, int64_t 
   }
   if (lab_host) KKM_CK(cudaMemcpyAsync(labels_out, lab, (size_t)M * 4, cudaMemcpyDeviceToHost, st));
   if (dist_host) KKM_CK(cudaMemcpyAsync(dist_out, dist, (size_t)M * 4, cudaMemcpyDeviceToHost, st));
-  int rtc_err_h = 0;
-  if (use_rtc) KKM_CK(cudaMemcpyAsync(&rtc_err_h, rtc.err, 4, cudaMemcpyDeviceToHost, st));
-  if (split) KKM_CK(cudaMemcpyAsync(&rtc_err_h, split_err, 4, cudaMemcpyDeviceToHost, st));
-  KKM_CK(cudaStreamSynchronize(st));
+  if (use_rtc) KKM_CK(cudaMemcpyAsync(&tc_err_h, rtc.err, 4, cudaMemcpyDeviceToHost, st));
+  if (!waited || lab_host || dist_host) KKM_CK(cudaStreamSynchronize(st));
   prof_collect();
   {
     bool bad = false;
     KKM_TRY(chk.wait(&bad));
     if (bad) return invalid("X holds NaN or Inf");
   }
-  if (rtc_err_h) {
+  if (tc_err_h) {
     set_error(split ? "tensor-core kernel block: a bounded pipeline wait gave up"
                     : "tensor-core MD estimate: a bounded pipeline wait gave up");
     return KKM_ETIMEOUT;
@@ -2128,30 +2139,23 @@ static kkm_status kernel_matrix_impl(const float* A_in, int64_t nA, const float*
   float *Ap, *Bp, *aA, *aB, *o;
   const bool host_out = !is_device_ptr(out);
   if (host_out) KKM_TRY(ws.alloc(&o, nA * nB)); else o = out;
-  if (precision == KKM_FP32 && split_applies(sp.kind, nA, d) && 3 * nB <= INT32_MAX) {
-    SplitRows SA, SB;
-    int* word;
-    int word_h[2] = {0, 0};
-    SA.X = A;
-    SB.X = Bm;
-    SA.ld = SB.ld = d;
-    KKM_TRY(alloc_split(ws, sp, nA, nB, &SA, &SB, &word));
-    KKM_RUN("split_rows", st, launch_split_rows(SA, nA, SB, nB, d, sp.dp, word + 1, st));
-    KKM_RUN("gram_split", st,
-            launch_gram_split(SA, nA, SB, nB, sp.dp, sp.neg_scale(), o, nB, word, sm_count(), st, polls));
-    if (host_out) KKM_CK(cudaMemcpyAsync(out, o, (size_t)nA * nB * 4, cudaMemcpyDeviceToHost, st));
-    KKM_CK(cudaMemcpyAsync(word_h, word, 8, cudaMemcpyDeviceToHost, st));
-    KKM_CK(cudaStreamSynchronize(st));
-    prof_collect();
-    if (word_h[0]) {
-      set_error("tensor-core kernel block: a bounded pipeline wait gave up");
-      return KKM_ETIMEOUT;
-    }
-    if (!word_h[1]) return KKM_OK;
-    // rows with NaN or Inf have no slices: the FFMA kernel below gives their values
-  }
   int tc_err_h = 0;
-  if (precision == KKM_BF16) {
+  bool waited = false;
+  if (precision == KKM_FP32 && split_applies(sp.kind, nA, d) && 3 * nB <= INT32_MAX) {
+    SplitScratch t;
+    const SplitSide sA{A, d}, sB{Bm, d};
+    int words_h[kSplitWords] = {};
+    KKM_TRY(alloc_split(ws, sp, nA, nB, &t));
+    KKM_TRY(split_block(t, sA, nA, sB, nB, d, sp.dp, sp.neg_scale(), o, nB, /*p_ready=*/false, sm_count(), st, polls));
+    KKM_CK(cudaMemcpyAsync(words_h, t.words, sizeof words_h, cudaMemcpyDeviceToHost, st));
+    KKM_CK(cudaStreamSynchronize(st));
+    tc_err_h = words_h[kSplitErr];
+    waited = true;
+    if (words_h[kSplitWideQ] || words_h[kSplitWideP]) {
+      KKM_RUN("gram_wide", st, launch_gram_wide(t, sA, nA, sB, nB, d, sp.dp, sp.neg_scale(), o, nB, sm_count(), st));
+      waited = false;
+    }
+  } else if (precision == KKM_BF16) {
     __nv_bfloat16 *Ab, *Bb;
     float *nAb, *nBb;
     int* err;
@@ -2200,7 +2204,7 @@ static kkm_status kernel_matrix_impl(const float* A_in, int64_t nA, const float*
     }
   }
   if (host_out) KKM_CK(cudaMemcpyAsync(out, o, (size_t)nA * nB * 4, cudaMemcpyDeviceToHost, st));
-  KKM_CK(cudaStreamSynchronize(st));
+  if (!waited || host_out) KKM_CK(cudaStreamSynchronize(st));
   prof_collect();
   if (tc_err_h) {
     set_error("tensor-core kernel block: a bounded pipeline wait gave up");

@@ -276,51 +276,32 @@ constexpr size_t kGramChunkSmem = sizeof(float) * 64 * 256;   // [64 outputs][25
 template <int KIND>
 constexpr bool gram_chunked() { return KIND == DK_RBF || KIND == DK_LINEAR; }
 
-// OutT: float, or __half for a Gaussian block stored in FP16 (values in [0, 1]).
-template <int KIND, typename OutT>
-__global__ void __launch_bounds__(256, 2)
-gram_tiled_kernel(const float* __restrict__ A, int nA, const float* __restrict__ Bm, int nB,
-                  int dp, const float* __restrict__ normA, const float* __restrict__ normB,
-                  const int64_t* __restrict__ idA, const int64_t* __restrict__ idB,
-                  float neg_scale, OutT* __restrict__ out, int64_t ldo, int vec_ok, int upper_only,
-                  float* __restrict__ out32) {
-  __shared__ __align__(16) float As[2][TB_K][TB_M];
-  __shared__ __align__(16) float Bs[2][TB_K][TB_N];
-  const int tid = threadIdx.x;
-  const int a0 = blockIdx.y * TB_M, b0 = blockIdx.x * TB_N;
-  // only the strict upper triangle (b > a) is wanted: tiles wholly at or
-  // below the diagonal are skipped (their outputs are left unwritten)
-  if (upper_only && b0 + TB_N - 1 <= a0) return;
-  // split K (DK_RAW): slice z of gridDim.z takes its share of the k-tiles and
-  // stores raw products in out + z * nA * ldo
-  const int nk_all = dp / TB_K;
-  const int kt0 = (int)((int64_t)nk_all * blockIdx.z / gridDim.z);
-  const int nk = (int)((int64_t)nk_all * (blockIdx.z + 1) / gridDim.z) - kt0;
-  if (KIND == DK_RAW) out += (int64_t)blockIdx.z * nA * ldo;
-  const int lr = tid >> 1, lk = (tid & 1) << 2;
-  // Rows past the end re-read the last valid row; their outputs are dropped.
-  const float* pa = A + (int64_t)min(a0 + lr, nA - 1) * dp + lk + kt0 * TB_K;
-  const float* pb = Bm + (int64_t)min(b0 + lr, nB - 1) * dp + lk + kt0 * TB_K;
-  float4 ga = __ldg(reinterpret_cast<const float4*>(pa));
-  float4 gb = __ldg(reinterpret_cast<const float4*>(pb));
+// The product of a 128 x 128 tile: acc[i][j] = sum over nk k-tiles of the rows
+// {ty*4+i, 64+ty*4+i} x {tx*4+j, 64+tx*4+j}.  load_a(kt), load_b(kt): the four
+// values 8 kt + 4 (tid & 1).. of the tile's row tid / 2.
+typedef float TileShared[2][TB_K][TB_M];
+template <bool CHUNKED, typename LA, typename LB>
+__device__ __forceinline__ void ffma_product(const LA& load_a, const LB& load_b, int nk, TileShared& As, TileShared& Bs,
+                                             float* chunk_sum, float (&acc)[8][8]) {
+  const int tid = threadIdx.x, lr = tid >> 1, lk = (tid & 1) << 2;
+  float4 ga = load_a(0);
+  float4 gb = load_b(0);
   As[0][lk + 0][lr] = ga.x; As[0][lk + 1][lr] = ga.y; As[0][lk + 2][lr] = ga.z; As[0][lk + 3][lr] = ga.w;
   Bs[0][lk + 0][lr] = gb.x; Bs[0][lk + 1][lr] = gb.y; Bs[0][lk + 2][lr] = gb.z; Bs[0][lk + 3][lr] = gb.w;
   __syncthreads();
 
   const int tx = tid & 15, ty = tid >> 4;
-  float acc[8][8];
 #pragma unroll
   for (int i = 0; i < 8; ++i)
 #pragma unroll
     for (int j = 0; j < 8; ++j) acc[i][j] = 0.0f;
-  extern __shared__ float chunk_sum[];  // [64][256] when gram_chunked<KIND>()
   bool have_chunk = false;
 
   for (int kt = 0; kt < nk; ++kt) {
     const int cur = kt & 1;
     if (kt + 1 < nk) {
-      ga = __ldg(reinterpret_cast<const float4*>(pa + (kt + 1) * TB_K));
-      gb = __ldg(reinterpret_cast<const float4*>(pb + (kt + 1) * TB_K));
+      ga = load_a(kt + 1);
+      gb = load_b(kt + 1);
     }
 #pragma unroll
     for (int k = 0; k < TB_K; ++k) {
@@ -340,7 +321,7 @@ gram_tiled_kernel(const float* __restrict__ A, int nA, const float* __restrict__
       As[nx][lk + 0][lr] = ga.x; As[nx][lk + 1][lr] = ga.y; As[nx][lk + 2][lr] = ga.z; As[nx][lk + 3][lr] = ga.w;
       Bs[nx][lk + 0][lr] = gb.x; Bs[nx][lk + 1][lr] = gb.y; Bs[nx][lk + 2][lr] = gb.z; Bs[nx][lk + 3][lr] = gb.w;
     }
-    if constexpr (gram_chunked<KIND>()) {
+    if constexpr (CHUNKED) {
       if ((kt + 1) % kGramChunkTiles == 0 && kt + 1 < nk) {  // close a chunk (not the last one)
 #pragma unroll
         for (int i = 0; i < 8; ++i)
@@ -355,7 +336,7 @@ gram_tiled_kernel(const float* __restrict__ A, int nA, const float* __restrict__
     }
     __syncthreads();
   }
-  if constexpr (gram_chunked<KIND>()) {
+  if constexpr (CHUNKED) {
     if (have_chunk) {  // the open chunk joins the closed ones
 #pragma unroll
       for (int i = 0; i < 8; ++i)
@@ -363,6 +344,38 @@ gram_tiled_kernel(const float* __restrict__ A, int nA, const float* __restrict__
         for (int j = 0; j < 8; ++j) acc[i][j] += chunk_sum[(i * 8 + j) * 256 + tid];
     }
   }
+}
+
+// OutT: float, or __half for a Gaussian block stored in FP16 (values in [0, 1]).
+template <int KIND, typename OutT>
+__global__ void __launch_bounds__(256, 2)
+gram_tiled_kernel(const float* __restrict__ A, int nA, const float* __restrict__ Bm, int nB,
+                  int dp, const float* __restrict__ normA, const float* __restrict__ normB,
+                  const int64_t* __restrict__ idA, const int64_t* __restrict__ idB,
+                  float neg_scale, OutT* __restrict__ out, int64_t ldo, int vec_ok, int upper_only,
+                  float* __restrict__ out32) {
+  __shared__ __align__(16) TileShared As, Bs;
+  const int tid = threadIdx.x;
+  const int a0 = blockIdx.y * TB_M, b0 = blockIdx.x * TB_N;
+  // only the strict upper triangle (b > a) is wanted: tiles wholly at or
+  // below the diagonal are skipped (their outputs are left unwritten)
+  if (upper_only && b0 + TB_N - 1 <= a0) return;
+  // split K (DK_RAW): slice z of gridDim.z takes its share of the k-tiles and
+  // stores raw products in out + z * nA * ldo
+  const int nk_all = dp / TB_K;
+  const int kt0 = (int)((int64_t)nk_all * blockIdx.z / gridDim.z);
+  const int nk = (int)((int64_t)nk_all * (blockIdx.z + 1) / gridDim.z) - kt0;
+  if (KIND == DK_RAW) out += (int64_t)blockIdx.z * nA * ldo;
+  const int lr = tid >> 1, lk = (tid & 1) << 2;
+  // Rows past the end re-read the last valid row; their outputs are dropped.
+  const float* pa = A + (int64_t)min(a0 + lr, nA - 1) * dp + lk + kt0 * TB_K;
+  const float* pb = Bm + (int64_t)min(b0 + lr, nB - 1) * dp + lk + kt0 * TB_K;
+  float acc[8][8];
+  extern __shared__ float chunk_sum[];  // [64][256] when gram_chunked<KIND>()
+  ffma_product<gram_chunked<KIND>()>(
+      [&](int kt) { return __ldg(reinterpret_cast<const float4*>(pa + kt * TB_K)); },
+      [&](int kt) { return __ldg(reinterpret_cast<const float4*>(pb + kt * TB_K)); }, nk, As, Bs, chunk_sum, acc);
+  const int tx = tid & 15, ty = tid >> 4;
 
   // Epilogue: rows a0 + {ty*4+i, 64+ty*4+i}, columns b0 + {tx*4+j, 64+tx*4+j}.
   float nb[8];
@@ -424,6 +437,92 @@ gram_tiled_kernel(const float* __restrict__ A, int nA, const float* __restrict__
         if (b + q < nB) orow[b + q] = OutT(v[h * 4 + q]);
     }
   }
+}
+
+// ------------------------------------------------------ rows without slices
+// The pairs of the tensor-core block's wide rows (gram_split.cu), by the tiled
+// kernel's sums: first the wide references against every sample, then the
+// others against the wide samples, 128 x 128 pairs of the listed rows a tile.
+// The lists are made on the device, so the tiles are counted there and
+// persistent CTAs share them; without wide rows a launch ends at once.  The rows
+// are read where they lie: d and the alignment are the caller's.
+struct WideSide {
+  const float* X;
+  int64_t ld;
+  const float* norm;
+  const int32_t* rows;
+  int vec;  // 16-byte loads
+};
+__global__ void __launch_bounds__(256, 2)
+gram_wide_kernel(WideSide P, WideSide Q, const int* __restrict__ words, int nP, int nQ, int d, int dp, float neg_scale,
+                 float* __restrict__ out, int64_t ldo, int vec_ok) {
+  __shared__ __align__(16) TileShared As, Bs;
+  extern __shared__ float chunk_sum[];
+  const int wide_p = words[kSplitWideP], clean_p = words[kSplitCleanP], wide_q = words[kSplitWideQ];
+  auto tiles = [](int n) { return (n + TB_M - 1) / TB_M; };
+  const int64_t n1 = (int64_t)tiles(wide_p) * tiles(nQ), n2 = (int64_t)tiles(clean_p) * tiles(wide_q);
+  const int tid = threadIdx.x, lr = tid >> 1, lk = (tid & 1) << 2, tx = tid & 15, ty = tid >> 4;
+  for (int64_t t = blockIdx.x; t < n1 + n2; t += gridDim.x) {
+    const bool all = t < n1;  // every sample
+    const int64_t u = all ? t : t - n1;
+    const int tb = tiles(all ? nQ : wide_q);
+    const int a0 = (int)(u / tb) * TB_M, b0 = (int)(u % tb) * TB_N;
+    const int na = all ? wide_p : clean_p, nb = all ? nQ : wide_q;
+    auto row_a = [&](int a) { return (int64_t)P.rows[all ? nP - 1 - a : a]; };
+    auto row_b = [&](int b) { return (int64_t)(all ? b : Q.rows[b]); };
+    // rows past the end repeat the last one; their outputs are dropped
+    const float* const pa = P.X + row_a(min(a0 + lr, na - 1)) * P.ld;
+    const float* const pb = Q.X + row_b(min(b0 + lr, nb - 1)) * Q.ld;
+    auto load = [&](const float* p, int vec, int kt) {
+      const int c = kt * TB_K + lk;
+      if (vec) return c < d ? __ldg(reinterpret_cast<const float4*>(p + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      return make_float4(c < d ? __ldg(p + c) : 0.f, c + 1 < d ? __ldg(p + c + 1) : 0.f,
+                         c + 2 < d ? __ldg(p + c + 2) : 0.f, c + 3 < d ? __ldg(p + c + 3) : 0.f);
+    };
+    float acc[8][8];
+    ffma_product<true>([&](int kt) { return load(pa, P.vec, kt); }, [&](int kt) { return load(pb, Q.vec, kt); },
+                       dp / TB_K, As, Bs, chunk_sum, acc);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int a = a0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + i - 4);
+      if (a >= na) continue;
+      const int64_t ra = row_a(a);
+      const float norm_a = P.norm[ra];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int b = b0 + h * 64 + tx * 4;
+        float v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          v[q] = b + q < nb ? gram_epilogue<DK_RBF>(acc[i][h * 4 + q], norm_a, Q.norm[row_b(b + q)], false, neg_scale)
+                            : 0.0f;
+        if (all && vec_ok && b + 3 < nb) {
+          *reinterpret_cast<float4*>(out + ra * ldo + b) = make_float4(v[0], v[1], v[2], v[3]);
+        } else {
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (b + q < nb) out[ra * ldo + row_b(b + q)] = v[q];
+        }
+      }
+    }
+  }
+}
+cudaError_t launch_gram_wide(const SplitScratch& t, const SplitSide& P, int64_t nP, const SplitSide& Q, int64_t nQ,
+                             int64_t d, int dp, float neg_scale, float* out, int64_t ldo, int n_sms, cudaStream_t st) {
+  if (nP <= 0 || nQ <= 0) return cudaSuccess;
+  if (dp % TB_K != 0) return cudaErrorInvalidValue;
+  auto side = [&](const SplitSide& s, const SplitBufs& b) {
+    return WideSide{s.X, s.ld, s.norm ? s.norm : b.norm, b.rows, d % 4 == 0 && s.ld % 4 == 0 && aligned16(s.X)};
+  };
+  const cudaError_t e =
+      cudaFuncSetAttribute(gram_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGramChunkSmem);
+  if (e != cudaSuccess) return e;
+  // at most all tiles of either part; two CTAs fit an SM
+  const int64_t most = (ceil_div(nP, TB_M) + 1) * ceil_div(nQ, TB_N);
+  gram_wide_kernel<<<(unsigned)std::min<int64_t>(most, 2 * std::max(n_sms, 1)), 256, kGramChunkSmem, st>>>(
+      side(P, t.P), side(Q, t.Q), t.words, (int)nP, (int)nQ, (int)d, dp, neg_scale, out, ldo,
+      ldo % 4 == 0 && aligned16(out));
+  return cudaGetLastError();
 }
 
 // ------------------------------------------------ skinny (<= 32 reference rows)

@@ -26,7 +26,8 @@
 // 0.83 (0.94), with one 30.0 0.69 (0.68), log-normal of sigma 2 0.85 (0.86) at
 // 784 and 0.89 (0.88) at 2,048 values.  (mid and lo as multiples of 2^-2 and
 // 2^-11 and one second sum per tile, as before, gave 1.63, 3.34, 1.78, 1.38
-// and 1.69 on those five.)
+// and 1.69 on those five.)  Rows beyond those bounds are left to FFMA sums, row
+// by row (see split_rows_kernel).
 //
 // What bounds it: six FP16 products of 2 d flop per entry.  At 784 values a
 // 3,001 x 15,013 block takes 0.27 ms (1.57 PFLOP/s of FP16 products, 0.82 of
@@ -101,19 +102,24 @@ struct SplitShared {
   float2 ns[8][128];  // norm and scale of a warp's references
 };
 
+// static and dynamic share together: 227 KB
+static_assert((sizeof(SplitShared) + 1023) / 1024 * 1024 + SpCfg<256>::kSmem <= 227 * 1024, "shared memory");
+
 template <int SP_N>
 __global__ void __launch_bounds__(SP_THREADS, 1)
 gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapP, int nQ, int nP,
-                  int dk, const float* __restrict__ normQ, const float* __restrict__ normP,
+                  int capQ, int capP, int dk, const float* __restrict__ normQ, const float* __restrict__ normP,
                   const float* __restrict__ scaleQ, const float* __restrict__ scaleP, float neg_scale,
-                  float* __restrict__ out, int64_t ldo, int* __restrict__ err, uint32_t polls) {
+                  float* __restrict__ out, int64_t ldo, int* __restrict__ words, uint32_t polls) {
   constexpr int SP_B_BYTES = SpCfg<SP_N>::kBBytes, SP_STAGE_BYTES = SpCfg<SP_N>::kStageBytes;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* const stages = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ SplitShared sh;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int* const err = words + kSplitErr;
   const int tiles_m = (nQ + SP_M - 1) / SP_M, tiles_n = (nP + SP_N - 1) / SP_N;
-  const int n_tiles = tiles_m * tiles_n;
+  // nothing to do when a whole side is wide: every value is then the FFMA sums'
+  const int n_tiles = words[kSplitWideP] < nP && words[kSplitWideQ] < nQ ? tiles_m * tiles_n : 0;
   const int nk = (dk + SP_K - 1) / SP_K;
 
   if (threadIdx.x == 0) {
@@ -154,11 +160,11 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
           uint8_t* const a = stages + (size_t)s * SP_STAGE_BYTES;
           uint8_t* const b = a + 3 * SP_A_BYTES;
           mbar_expect_tx(&sh.full[s], SP_STAGE_BYTES);
-          // slice v of row r is row v * n + r of the slice array
+          // slice v of row r is row v * cap + r of the slice array
 #pragma unroll
           for (int v = 0; v < 3; ++v) {
-            tma_load_2d(&mapQ, &sh.full[s], a + v * SP_A_BYTES, kb * SP_K, v * nQ + tm * SP_M);
-            tma_load_2d(&mapP, &sh.full[s], b + v * SP_B_BYTES, kb * SP_K, v * nP + tn * SP_N);
+            tma_load_2d(&mapQ, &sh.full[s], a + v * SP_A_BYTES, kb * SP_K, v * capQ + tm * SP_M);
+            tma_load_2d(&mapP, &sh.full[s], b + v * SP_B_BYTES, kb * SP_K, v * capP + tn * SP_N);
           }
           if (++s == SP_STAGES) {
             s = 0;
@@ -322,51 +328,96 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
 }
 
 // ------------------------------------------------------------- row slices
-// One warp per row of the two sets (references, then samples): the
-// power-of-two scale, the three slices, and (when asked) the squared norm;
-// *bad is set for a row holding NaN or Inf (its slices are then meaningless).
+// One warp per row of the two sets (references, then samples): the squared norm
+// (when asked), the power-of-two scale and the three slices.
+//
+// A row whose values the slices do not hold as well as FP32 does is wide: it
+// gets no slices, and its pairs come from the FFMA sums (launch_gram_wide).
+// That is a row with NaN or Inf, one whose squared norm leaves the FP32 range
+// (the scaled sums would meet it as Inf - Inf), and one whose largest value
+// stands so far out that the products left out matter: against the FFMA
+// kernel's error of about 0.8 units of 2^-24 (|p|^2 + |q|^2) they add
+// 0.23 sqrt(2 d) 2^24 / |scaled row|^2, at most 0.08 from 2^26 sqrt(d) on (the
+// largest value at most 11 to 21 times the root mean square at d = 784, 7 to 13
+// times at d = 128).
+// The slices stay at their rows' places (compacted, with the block's rows
+// through a list, a 3,001 x 15,013 x 784 call took 375 instead of 360 us), so
+// a block with wide rows pays for their tensor-core pairs as well: at most the
+// 0.27 ms beside the FFMA sums' 1.57, and nothing when a whole side is wide.
 struct SplitSource {
   const float* X;
-  int64_t ld, n;
+  int64_t ld, n, cap;
   __half* v;
-  float *scale, *normsq;
+  float *scale, *norm_out;
+  const float* norm;
+  int32_t* rows;
   int vec;  // 16-byte loads
 };
+static float wide_below(int64_t d) { return 0x1p26f * sqrtf((float)d); }
 
-__global__ void split_rows_kernel(SplitSource A, SplitSource B, int d, int ks, int* __restrict__ bad) {
-  const int lane = threadIdx.x & 31;
-  int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (row >= A.n + B.n) return;
-  const bool second = row >= A.n;
-  if (second) row -= A.n;
-  const SplitSource S = second ? B : A;
+__global__ void __launch_bounds__(256)
+split_rows_kernel(SplitSource P, SplitSource Q, int d, int ks, float least, int* __restrict__ words) {
+  __shared__ int state[8];  // the block's references: 1 holds slices, 2 wide (0: no reference)
+  __shared__ int first[2];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int64_t row = (int64_t)blockIdx.x * 8 + warp;
+  const bool some = row < P.n + Q.n, sample = row >= P.n;
+  if (sample) row -= P.n;
+  const SplitSource S = sample ? Q : P;
   const float* x = S.X + row * S.ld;
   auto load4 = [&](int c) -> float4 {  // values c..c+3, zero past d
     if (S.vec) return c < d ? __ldg(reinterpret_cast<const float4*>(x + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
     return make_float4(c < d ? __ldg(x + c) : 0.f, c + 1 < d ? __ldg(x + c + 1) : 0.f,
                        c + 2 < d ? __ldg(x + c + 2) : 0.f, c + 3 < d ? __ldg(x + c + 3) : 0.f);
   };
-  float2 acc = make_float2(0.0f, 0.0f);
-  uint32_t top = 0;  // the largest |value|, as an integer (NaN and Inf sort above)
-  for (int c = lane * 4; c < d; c += 128) {
-    const float4 v = load4(c);
-    top = max(max(top, max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu)),
-              max(__float_as_uint(v.z) & 0x7fffffffu, __float_as_uint(v.w) & 0x7fffffffu));
-    if (S.normsq) acc = df_add_sq(df_add_sq(df_add_sq(df_add_sq(acc, v.x), v.y), v.z), v.w);
+  float s = 0.0f, unscale = 0.0f;
+  bool wide = false;
+  if (some) {
+    float2 acc = make_float2(0.0f, 0.0f);
+    uint32_t top = 0;  // the largest |value|, as an integer (NaN and Inf sort above)
+    for (int c = lane * 4; c < d; c += 128) {
+      const float4 v = load4(c);
+      top = max(max(top, max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu)),
+                max(__float_as_uint(v.z) & 0x7fffffffu, __float_as_uint(v.w) & 0x7fffffffu));
+      if (!S.norm) acc = df_add_sq(df_add_sq(df_add_sq(df_add_sq(acc, v.x), v.y), v.z), v.w);
+    }
+    top = __reduce_max_sync(kFull, top);
+    float norm;
+    if (S.norm) {
+      norm = S.norm[row];
+    } else {
+      norm = df_to_float(warp_sum_df(acc));
+      if (lane == 0) S.norm_out[row] = norm;
+    }
+    // scaled maximum in [2^14, 2^15); the exponents stay within the normal range
+    const int up = min(141 - (int)(top >> 23), 126);  // 14 - (e - 127), e biased (0: zero or subnormal)
+    s = __uint_as_float((uint32_t)(127 + up) << 23);
+    unscale = __uint_as_float((uint32_t)(127 - up) << 23);
+    const float scaled = norm * s * s;
+    wide = top != 0 && !(scaled >= least && scaled <= 3.4028235e38f);
   }
-  top = __reduce_max_sync(kFull, top);
-  if (S.normsq) {
-    acc = warp_sum_df(acc);
-    if (lane == 0) S.normsq[row] = df_to_float(acc);
+  if (blockIdx.x * (int64_t)8 < P.n) {  // (no rows of references in the other blocks)
+    if (lane == 0) state[warp] = some && !sample ? 1 + wide : 0;
+    __syncthreads();
+    if (threadIdx.x < 2) {  // places in the list for the block's references of either kind
+      int n = 0;
+      for (int w = 0; w < 8; ++w) n += state[w] == 1 + (int)threadIdx.x;
+      if (n) first[threadIdx.x] = atomicAdd(words + kSplitCleanP + threadIdx.x, n);
+    }
+    __syncthreads();
+    if (lane == 0 && state[warp]) {
+      int64_t place = first[wide];
+      for (int w = 0; w < warp; ++w) place += state[w] == 1 + (int)wide;
+      S.rows[wide ? S.n - 1 - place : place] = (int32_t)row;
+    }
   }
-  const int e = (int)(top >> 23);  // biased exponent (0: zero or subnormal)
-  if (e == 255 && bad && lane == 0) *bad = 1;
-  // scaled maximum in [2^14, 2^15); the exponent stays within the normal range
-  const int up = min(141 - e, 126);  // 14 - (e - 127)
-  const float s = __uint_as_float((uint32_t)(127 + up) << 23);
-  if (lane == 0) S.scale[row] = __uint_as_float((uint32_t)(127 - up) << 23);
+  if (!some) return;
+  if (sample && wide && lane == 0) S.rows[atomicAdd(words + kSplitWideQ, 1)] = (int32_t)row;
+  // (a wide row's slices enter its own pairs only, which are written again)
+  if (lane == 0) S.scale[row] = unscale;
+  if (wide) return;
   __half* const o = S.v + row * ks;
-  const int64_t slice = S.n * (int64_t)ks;
+  const int64_t slice = S.cap * (int64_t)ks;
   for (int c = lane * 4; c < ks; c += 128) {
     const float4 v = load4(c);
     const float t[4] = {v.x * s, v.y * s, v.z * s, v.w * s};
@@ -385,14 +436,15 @@ __global__ void split_rows_kernel(SplitSource A, SplitSource B, int d, int ks, i
   }
 }
 
-cudaError_t launch_split_rows(const SplitRows& P, int64_t nP, const SplitRows& Q, int64_t nQ, int64_t d, int ks,
-                              int* bad, cudaStream_t st) {
+static cudaError_t launch_split_rows(const SplitSide& P, const SplitBufs& bP, int64_t nP, const SplitSide& Q,
+                                     const SplitBufs& bQ, int64_t nQ, int64_t d, int ks, int* words, cudaStream_t st) {
   if (nP + nQ <= 0) return cudaSuccess;
-  auto source = [&](const SplitRows& r, int64_t n) {
+  auto source = [&](const SplitSide& r, const SplitBufs& b, int64_t n) {
     const int vec = d % 4 == 0 && r.ld % 4 == 0 && (reinterpret_cast<uintptr_t>(r.X) & 15) == 0;
-    return SplitSource{r.X, r.ld, n, r.v, r.scale, r.form_norm ? r.norm : nullptr, vec};
+    return SplitSource{r.X, r.ld, n, b.cap, b.v, b.scale, b.norm, r.norm, b.rows, vec};
   };
-  split_rows_kernel<<<(unsigned)ceil_div(nP + nQ, 8), 256, 0, st>>>(source(P, nP), source(Q, nQ), (int)d, ks, bad);
+  split_rows_kernel<<<(unsigned)ceil_div(nP + nQ, 8), 256, 0, st>>>(source(P, bP, nP), source(Q, bQ, nQ), (int)d, ks,
+                                                                    wide_below(d), words);
   return cudaGetLastError();
 }
 
@@ -409,27 +461,44 @@ static bool split_map(CUtensorMap* map, const __half* base, int64_t n, int ks, i
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-cudaError_t launch_gram_split(const SplitRows& P, int64_t nP, const SplitRows& Q, int64_t nQ, int ks, float neg_scale,
-                              float* out, int64_t ldo, int* err, int n_sms, cudaStream_t st, uint32_t polls) {
-  if (nP <= 0 || nQ <= 0) return cudaSuccess;
-  if (ks % 8 != 0 || (reinterpret_cast<uintptr_t>(P.v) & 15) || (reinterpret_cast<uintptr_t>(Q.v) & 15) ||
-      3 * nP > INT32_MAX || 3 * nQ > INT32_MAX)
+static cudaError_t launch_gram_split(const SplitBufs& bP, const float* normP, int64_t nP, const SplitBufs& bQ,
+                                     const float* normQ, int64_t nQ, int ks, float neg_scale, float* out, int64_t ldo,
+                                     int* words, int n_sms, cudaStream_t st, uint32_t polls) {
+  if (ks % 8 != 0 || (reinterpret_cast<uintptr_t>(bP.v) & 15) || (reinterpret_cast<uintptr_t>(bQ.v) & 15) ||
+      nP > bP.cap || nQ > bQ.cap || 3 * bP.cap > INT32_MAX || 3 * bQ.cap > INT32_MAX)
     return cudaErrorInvalidValue;
   alignas(64) CUtensorMap mq, mp;
 #define KKM_SPLIT_LAUNCH(N)                                                                                    \
   do {                                                                                                         \
-    if (!split_map(&mq, Q.v, nQ, ks, SP_M) || !split_map(&mp, P.v, nP, ks, N)) return cudaErrorInvalidValue;   \
+    if (!split_map(&mq, bQ.v, bQ.cap, ks, SP_M) || !split_map(&mp, bP.v, bP.cap, ks, N))                       \
+      return cudaErrorInvalidValue;                                                                            \
     static const cudaError_t attr = cudaFuncSetAttribute(                                                      \
         gram_split_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SpCfg<N>::kSmem);              \
     if (attr != cudaSuccess) return attr;                                                                      \
     const int64_t tiles = ceil_div(nQ, SP_M) * ceil_div(nP, N);                                                \
     gram_split_kernel<N><<<(unsigned)std::min<int64_t>(tiles, std::max(n_sms, 1)), SP_THREADS, SpCfg<N>::kSmem, st>>>( \
-        mq, mp, (int)nQ, (int)nP, ks, Q.norm, P.norm, Q.scale, P.scale, neg_scale, out, ldo, err, polls);      \
+        mq, mp, (int)nQ, (int)nP, (int)bQ.cap, (int)bP.cap, ks, normQ, normP, bQ.scale, bP.scale, neg_scale, out, ldo, \
+        words, polls);                                                                                         \
   } while (0)
   if (2 * ceil_div(nQ, SP_M) * ceil_div(nP, 256) <= n_sms) KKM_SPLIT_LAUNCH(64);
   else KKM_SPLIT_LAUNCH(256);
 #undef KKM_SPLIT_LAUNCH
   return cudaGetLastError();
+}
+
+kkm_status split_block(SplitScratch& t, const SplitSide& P, int64_t nP, const SplitSide& Q, int64_t nQ, int64_t d,
+                       int dp, float neg_scale, float* out, int64_t ldo, bool p_ready, int n_sms, cudaStream_t st,
+                       uint32_t polls) {
+  if (nP <= 0 || nQ <= 0) return KKM_OK;
+  // the error word lasts, the counts start anew with their side
+  const int from = t.fresh ? kSplitErr : kSplitWideQ, to = p_ready ? kSplitCleanP : kSplitWords;
+  KKM_CK(cudaMemsetAsync(t.words + from, 0, 4 * (to - from), st));
+  t.fresh = false;
+  KKM_RUN("split_rows", st, launch_split_rows(P, t.P, p_ready ? 0 : nP, Q, t.Q, nQ, d, dp, t.words, st));
+  KKM_RUN("gram_split", st,
+          launch_gram_split(t.P, P.norm ? P.norm : t.P.norm, nP, t.Q, Q.norm ? Q.norm : t.Q.norm, nQ, dp, neg_scale, out,
+                            ldo, t.words, n_sms, st, polls));
+  return KKM_OK;
 }
 
 }  // namespace kkm

@@ -130,6 +130,11 @@ struct ProfScope {
   cudaStream_t stream;
   const char* prev_scope = nullptr;
 };
+#define KKM_RUN(name, st, call)                 \
+  do {                                          \
+    ::kkm::ProfScope _ps(name, st);             \
+    KKM_CK(call);                               \
+  } while (0)
 void prof_collect();  // after a stream sync: fold finished events into totals
 
 // NVTX range for the phases of a call (visible to a profiler attached to the
@@ -239,25 +244,45 @@ cudaError_t launch_gram_rbf_half(const float* A, int64_t nA, const float* Bm, in
 constexpr uint32_t kTcSpinLimit = 1u << 24;
 
 // ---- the FP32 Gaussian block on the tensor cores (gram_split.cu) ----------
-// FP32 rows X[r * ld .. + d) as three FP16 slices: v [3][n][ks] (ks = the row
-// length rounded up to 8), a power-of-two scale per row and the squared norms
-// (formed with the slices, or given).
-struct SplitRows {
+// One side of the block: FP32 rows X[r * ld .. + d), with their squared norms
+// or without (they are then formed).
+struct SplitSide {
   const float* X = nullptr;
   int64_t ld = 0;
+  const float* norm = nullptr;
+};
+// Scratch of a side for up to cap rows: the three FP16 slices v [3][cap][ks]
+// (ks = the row length rounded up to 8), a power-of-two scale per row, the
+// norms formed, and the wide rows (those the slices do not hold, see
+// gram_split.cu): of the samples, `rows` lists them; of the references, `rows`
+// has the others from the start and the wide ones from the end.
+struct SplitBufs {
+  int64_t cap = 0;
   __half* v = nullptr;
   float* scale = nullptr;
   float* norm = nullptr;
-  bool form_norm = true;
+  int32_t* rows = nullptr;
 };
-// The slices of both sides in one launch; *bad (nullable) is set when a value
-// is NaN or Inf.
-cudaError_t launch_split_rows(const SplitRows& P, int64_t nP, const SplitRows& Q, int64_t nQ, int64_t d, int ks,
-                              int* bad, cudaStream_t st);
-// out[n*ldo + m] = exp(-|p_n - q_m|^2 / (2 sigma^2)); *err as launch_gram_tc.
-cudaError_t launch_gram_split(const SplitRows& P, int64_t nP, const SplitRows& Q, int64_t nQ, int ks, float neg_scale,
-                              float* out, int64_t ldo, int* err, int n_sms, cudaStream_t st,
-                              uint32_t polls = kTcSpinLimit);
+// words[kSplitErr]: as *err of launch_gram_tc; then the numbers of wide samples,
+// of references that are not wide and of those that are.
+enum SplitWord { kSplitErr = 0, kSplitWideQ = 1, kSplitCleanP = 2, kSplitWideP = 3, kSplitWords = 4 };
+struct SplitScratch {
+  SplitBufs P, Q;
+  int* words = nullptr;
+  bool fresh = true;  // nothing has run in it yet
+};
+// out[n*ldo + m] = exp(-|p_n - q_m|^2 / (2 sigma^2)) but for the pairs of wide
+// rows, which launch_gram_wide has to write (it returns at once when there are
+// none; a caller that waits for the words anyway need not launch it).  A value
+// depends on its two rows alone.  p_ready: the references are those of the last
+// call.  The error word is for the caller to read.
+kkm_status split_block(SplitScratch& t, const SplitSide& P, int64_t nP, const SplitSide& Q, int64_t nQ, int64_t d,
+                       int dp, float neg_scale, float* out, int64_t ldo, bool p_ready, int n_sms, cudaStream_t st,
+                       uint32_t polls = kTcSpinLimit);
+// The pairs of the wide rows, by the FFMA kernel's sums (rows read in place,
+// dp = d rounded up to 8).
+cudaError_t launch_gram_wide(const SplitScratch& t, const SplitSide& P, int64_t nP, const SplitSide& Q, int64_t nQ,
+                             int64_t d, int dp, float neg_scale, float* out, int64_t ldo, int n_sms, cudaStream_t st);
 // Whether kkm_kernel_matrix and kkm_assign take it for an FP32 Gaussian block
 // against nA reference rows of d values: a rule on the references alone, so
 // that a sample's values do not depend on how many samples share the call.  Up

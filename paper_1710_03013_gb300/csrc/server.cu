@@ -99,7 +99,7 @@ static uint64_t assign_bytes(const kkm_model* m, int64_t M, int32_t mode) {
   uint64_t b = 4ull * M * m->d + 8ull * M;     // rows and outputs on the device
   b += 4ull * ldm * (m->dp + 1) + 4ull * rows_ref * ldm;
   if (mode == KKM_ASSIGN_SUPPORTS) b += 4ull * units * ldm + 8ull * units * ceil_div(ldm, kStripCols);
-  if (split_applies(m->kind, rows_ref, m->d)) b += 6ull * m->dp * (rows_ref + ldm) + 4ull * (rows_ref + ldm);
+  if (split_applies(m->kind, rows_ref, m->d)) b += (6ull * m->dp + 12) * (rows_ref + ldm);
   if (m->kind == KKM_RMSD)  // tensor-core MD path
     b += 18ull * round_up(m->n_atoms, 64) * (rows_ref + ldm) + 16ull * rows_ref * ldm + 8ull * rows_ref +
          rows_ref * rmsd_near_pitch(ldm) + 8ull * rmsd_max_units(rows_ref, ldm);
