@@ -519,7 +519,7 @@ kkm_status kkm_minibatch_plan(int64_t N, int32_t B, int32_t sampling, double s,
  *   returns when its work is done: it waits for the stream once after the
  *   non-finite-input check and once at the end.
  * It allocates nothing: its working memory is one fixed scratch array of
- * about 21 MB that every GPU loading this library keeps until exit.  The
+ * about 30 MB that every GPU loading this library keeps until exit.  The
  * first call on each device looks up that array's device address (and may
  * load the library's device code); make it before any stream capture.  All
  * calls share the array: calls whose GPU work overlaps (several streams or

@@ -657,7 +657,7 @@ static kkm_status kernel_block(const KernelSpec& sp, const float* A, const float
   return KKM_OK;
 }
 
-static int sm_count() {
+int sm_count() {
   static const int n = []() {
     int dev = 0, v = 1;
     cudaGetDevice(&dev);
@@ -2051,7 +2051,7 @@ static kkm_status assign_impl(const kkm_model* m, const float* Xnew_in, int64_t 
     const int n = (int)std::min<int64_t>(chunk, M - c0);
     if (split) {
       KKM_TRY(split_block(slices, ref, rows_ref, SplitSide{X + c0 * d, d}, n, d, sp.dp, sp.neg_scale(), Kb, ldm,
-                          /*p_ready=*/c0 > 0, sm_count(), st));
+                          /*p_ready=*/c0 > 0, /*q_ready=*/false, sm_count(), st));
       if (M > chunk) KKM_TRY(wide_pairs(c0, n));
     } else {
       KKM_TRY(prep_rows(sp, X, c0, 1, n, Xc, auxc, st));
@@ -2146,7 +2146,8 @@ static kkm_status kernel_matrix_impl(const float* A_in, int64_t nA, const float*
     const SplitSide sA{A, d}, sB{Bm, d};
     int words_h[kSplitWords] = {};
     KKM_TRY(alloc_split(ws, sp, nA, nB, &t));
-    KKM_TRY(split_block(t, sA, nA, sB, nB, d, sp.dp, sp.neg_scale(), o, nB, /*p_ready=*/false, sm_count(), st, polls));
+    KKM_TRY(split_block(t, sA, nA, sB, nB, d, sp.dp, sp.neg_scale(), o, nB, /*p_ready=*/false,
+                        /*q_ready=*/false, sm_count(), st, polls));
     KKM_CK(cudaMemcpyAsync(words_h, t.words, sizeof words_h, cudaMemcpyDeviceToHost, st));
     KKM_CK(cudaStreamSynchronize(st));
     tc_err_h = words_h[kSplitErr];

@@ -487,14 +487,17 @@ static cudaError_t launch_gram_split(const SplitBufs& bP, const float* normP, in
 }
 
 kkm_status split_block(SplitScratch& t, const SplitSide& P, int64_t nP, const SplitSide& Q, int64_t nQ, int64_t d,
-                       int dp, float neg_scale, float* out, int64_t ldo, bool p_ready, int n_sms, cudaStream_t st,
-                       uint32_t polls) {
+                       int dp, float neg_scale, float* out, int64_t ldo, bool p_ready, bool q_ready, int n_sms,
+                       cudaStream_t st, uint32_t polls) {
   if (nP <= 0 || nQ <= 0) return KKM_OK;
   // the error word lasts, the counts start anew with their side
-  const int from = t.fresh ? kSplitErr : kSplitWideQ, to = p_ready ? kSplitCleanP : kSplitWords;
-  KKM_CK(cudaMemsetAsync(t.words + from, 0, 4 * (to - from), st));
-  t.fresh = false;
-  KKM_RUN("split_rows", st, launch_split_rows(P, t.P, p_ready ? 0 : nP, Q, t.Q, nQ, d, dp, t.words, st));
+  const int from = t.fresh ? kSplitErr : q_ready ? kSplitCleanP : kSplitWideQ, to = p_ready ? kSplitCleanP : kSplitWords;
+  if (from < to) {
+    KKM_CK(cudaMemsetAsync(t.words + from, 0, 4 * (to - from), st));
+    t.fresh = false;
+    KKM_RUN("split_rows", st,
+            launch_split_rows(P, t.P, p_ready ? 0 : nP, Q, t.Q, q_ready ? 0 : nQ, d, dp, t.words, st));
+  }
   KKM_RUN("gram_split", st,
           launch_gram_split(t.P, P.norm ? P.norm : t.P.norm, nP, t.Q, Q.norm ? Q.norm : t.Q.norm, nQ, dp, neg_scale, out,
                             ldo, t.words, n_sms, st, polls));

@@ -243,6 +243,8 @@ cudaError_t launch_gram_rbf_half(const float* A, int64_t nA, const float* Bm, in
 // kernels whose launcher takes `polls` can be given less, for tests).
 constexpr uint32_t kTcSpinLimit = 1u << 24;
 
+int sm_count();  // of the current device
+
 // ---- the FP32 Gaussian block on the tensor cores (gram_split.cu) ----------
 // One side of the block: FP32 rows X[r * ld .. + d), with their squared norms
 // or without (they are then formed).
@@ -274,11 +276,11 @@ struct SplitScratch {
 // out[n*ldo + m] = exp(-|p_n - q_m|^2 / (2 sigma^2)) but for the pairs of wide
 // rows, which launch_gram_wide has to write (it returns at once when there are
 // none; a caller that waits for the words anyway need not launch it).  A value
-// depends on its two rows alone.  p_ready: the references are those of the last
-// call.  The error word is for the caller to read.
+// depends on its two rows alone.  p_ready, q_ready: the references, the samples
+// are those of the last call.  The error word is for the caller to read.
 kkm_status split_block(SplitScratch& t, const SplitSide& P, int64_t nP, const SplitSide& Q, int64_t nQ, int64_t d,
-                       int dp, float neg_scale, float* out, int64_t ldo, bool p_ready, int n_sms, cudaStream_t st,
-                       uint32_t polls = kTcSpinLimit);
+                       int dp, float neg_scale, float* out, int64_t ldo, bool p_ready, bool q_ready, int n_sms,
+                       cudaStream_t st, uint32_t polls = kTcSpinLimit);
 // The pairs of the wide rows, by the FFMA kernel's sums (rows read in place,
 // dp = d rounded up to 8).
 cudaError_t launch_gram_wide(const SplitScratch& t, const SplitSide& P, int64_t nP, const SplitSide& Q, int64_t nQ,

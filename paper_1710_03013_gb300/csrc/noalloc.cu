@@ -9,7 +9,7 @@
 // fixed scratch area instead.
 //
 // The scratch is the file-scope array below.  Every GPU that loads this
-// library holds it (about 21 MB) until the process exits.  All calls share it
+// library holds it (about 30 MB) until the process exits.  All calls share it
 // and it keeps the contents of the last call, so two calls whose work overlaps
 // on the GPU (different streams, or threads calling concurrently) race on it;
 // calls on one stream, one after the other, are safe.  What must start at zero
@@ -23,6 +23,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "internal.h"
@@ -35,10 +36,23 @@ constexpr int64_t kNaRowLen = KKM_NOALLOC_MAX_ROWLEN;  // prepared row length
 constexpr int64_t kNaUnits = (kNaRef + kUnitRows - 1) / kUnitRows + kMaxC;
 constexpr int64_t kNaGrid = kNaRows / 32;              // assign CTAs (32 rows each)
 
+// Gaussian models that kkm_assign labels from the block of FP16 slices
+// (gram_split.cu) take it here too; the references pass through the scratch
+// kNaSplitRef at a time (a value does not depend on the others in its block).
+constexpr int64_t kNaSplitRef = 1024;
+
 constexpr size_t na_align(size_t x) { return (x + 255) & ~size_t(255); }
-constexpr size_t kOffRows = 0;                                               // float [rows][rowlen]
-constexpr size_t kOffAux = na_align(kOffRows + sizeof(float) * kNaRows * kNaRowLen);  // float [rows]
-constexpr size_t kOffK = na_align(kOffAux + sizeof(float) * kNaRows);         // float [ref][rows]
+// float [rows][rowlen], or the slices of the rows and of a block of references
+constexpr size_t kOffRows = 0;
+constexpr size_t kNaSliceBytes = 3 * sizeof(__half) * kNaRowLen;  // of a row
+constexpr size_t kOffSliceP = na_align(kOffRows + kNaSliceBytes * kNaRows);
+constexpr size_t kOffAux = na_align(kOffSliceP + kNaSliceBytes * kNaSplitRef);  // float [rows]: |x|^2
+constexpr size_t kOffScaleQ = na_align(kOffAux + sizeof(float) * kNaRows);       // float [rows]
+constexpr size_t kOffListQ = na_align(kOffScaleQ + sizeof(float) * kNaRows);     // int32_t [rows]
+constexpr size_t kOffScaleP = na_align(kOffListQ + sizeof(int32_t) * kNaRows);   // float [references]
+constexpr size_t kOffListP = na_align(kOffScaleP + sizeof(float) * kNaSplitRef);  // int32_t [references]
+constexpr size_t kOffWords = na_align(kOffListP + sizeof(int32_t) * kNaSplitRef);  // int [kSplitWords]
+constexpr size_t kOffK = na_align(kOffWords + sizeof(int) * kSplitWords);     // float [ref][rows]
 constexpr size_t kOffPart = na_align(kOffK + sizeof(float) * kNaRef * kNaRows);  // float [units][rows]
 constexpr size_t kOffOmega = na_align(kOffPart + sizeof(float) * kNaUnits * kNaRows);  // float2 [grid]
 constexpr size_t kOffChanged = na_align(kOffOmega + sizeof(float2) * kNaGrid);   // int [grid]
@@ -126,14 +140,31 @@ static kkm_status assign_noalloc_impl(const kkm_model* m, const float* X, int64_
   const int ap = rmsd ? m->dp / 3 : 0;
   const float neg_scale = (float)(-1.4426950408889634 / (2.0 * (double)m->sigma * (double)m->sigma));
   const int dk = rmsd ? DK_RBF : (m->kind == KKM_LINEAR ? DK_LINEAR : DK_RBF);
+  const bool split = split_applies(m->kind, rows_ref, m->d);
   if (rmsd)
     KKM_CK(launch_rmsd_prep_rows(X, m->n_atoms, 0, 1, M, Xc, ap, auxc, st));
-  else
+  else if (!split)
     KKM_CK(launch_gather_rows(X, m->d, 0, 1, M, Xc, m->dp, auxc, st));
   const float* kself = m->kind == KKM_LINEAR ? auxc : nullptr;
   const float* P = mode == KKM_ASSIGN_SUPPORTS ? m->sup : m->med;
   const float* Paux = mode == KKM_ASSIGN_SUPPORTS ? m->sup_aux : m->med_aux;
-  if (rmsd)
+  SplitScratch slices;
+  if (split) {
+    slices.words = reinterpret_cast<int*>(base + kOffWords);
+    slices.Q = SplitBufs{kNaRows, reinterpret_cast<__half*>(base + kOffRows), reinterpret_cast<float*>(base + kOffScaleQ),
+                         auxc, reinterpret_cast<int32_t*>(base + kOffListQ)};
+    slices.P = SplitBufs{kNaSplitRef, reinterpret_cast<__half*>(base + kOffSliceP),
+                         reinterpret_cast<float*>(base + kOffScaleP), nullptr,
+                         reinterpret_cast<int32_t*>(base + kOffListP)};
+    const SplitSide q{X, m->d};
+    for (int64_t p0 = 0; p0 < rows_ref; p0 += kNaSplitRef) {
+      const int64_t n = std::min<int64_t>(kNaSplitRef, rows_ref - p0);
+      const SplitSide p{P + p0 * m->dp, m->dp, Paux + p0};
+      KKM_TRY(split_block(slices, p, n, q, M, m->d, m->dp, neg_scale, Kb + p0 * ldm, ldm, /*p_ready=*/false,
+                          /*q_ready=*/p0 > 0, sm_count(), st));
+      KKM_CK(launch_gram_wide(slices, p, n, q, M, m->d, m->dp, neg_scale, Kb + p0 * ldm, ldm, sm_count(), st));
+    }
+  } else if (rmsd)
     KKM_CK(launch_rmsd_gram(dk, P, rows_ref, Xc, M, ap, m->n_atoms, Paux, auxc, nullptr, nullptr, neg_scale, Kb,
                             ldm, st));
   else
@@ -171,7 +202,13 @@ static kkm_status assign_noalloc_impl(const kkm_model* m, const float* X, int64_
     KKM_CK(launch_nearest(Kb, ldm, (int)M, m->C, kself, m->kind == KKM_LINEAR ? m->med_aux : nullptr, labels_out,
                           dist_out, st));
   }
+  int err = 0;
+  if (split) KKM_CK(cudaMemcpyAsync(&err, slices.words + kSplitErr, sizeof(int), cudaMemcpyDeviceToHost, st));
   KKM_CK(cudaStreamSynchronize(st));
+  if (err) {
+    set_error("tensor-core kernel block: a bounded pipeline wait gave up");
+    return KKM_ETIMEOUT;
+  }
   return KKM_OK;
 }
 
