@@ -2042,10 +2042,8 @@ static kkm_status assign_impl(const kkm_model* m, const float* Xnew_in, int64_t 
     return KKM_OK;
   };
   auto wide_pairs = [&](int64_t c0, int n) -> kkm_status {
-    KKM_RUN("gram_wide", st,
-            launch_gram_wide(slices, ref, rows_ref, SplitSide{X + c0 * d, d}, n, d, sp.dp, sp.neg_scale(), Kb, ldm,
-                             sm_count(), st));
-    return KKM_OK;
+    return split_wide_pairs(slices, ref, rows_ref, SplitSide{X + c0 * d, d}, n, d, sp.dp, sp.neg_scale(), Kb, ldm,
+                            sm_count(), st);
   };
   for (int64_t c0 = 0; c0 < M; c0 += chunk) {
     const int n = (int)std::min<int64_t>(chunk, M - c0);
@@ -2153,7 +2151,7 @@ static kkm_status kernel_matrix_impl(const float* A_in, int64_t nA, const float*
     tc_err_h = words_h[kSplitErr];
     waited = true;
     if (words_h[kSplitWideQ] || words_h[kSplitWideP]) {
-      KKM_RUN("gram_wide", st, launch_gram_wide(t, sA, nA, sB, nB, d, sp.dp, sp.neg_scale(), o, nB, sm_count(), st));
+      KKM_TRY(split_wide_pairs(t, sA, nA, sB, nB, d, sp.dp, sp.neg_scale(), o, nB, sm_count(), st));
       waited = false;
     }
   } else if (precision == KKM_BF16) {

@@ -458,7 +458,7 @@ gram_wide_kernel(WideSide P, WideSide Q, const int* __restrict__ words, int nP, 
                  float* __restrict__ out, int64_t ldo, int vec_ok) {
   __shared__ __align__(16) TileShared As, Bs;
   extern __shared__ float chunk_sum[];
-  const int wide_p = words[kSplitWideP], clean_p = words[kSplitCleanP], wide_q = words[kSplitWideQ];
+  const int wide_p = words[kSplitWideP], clean_p = nP - wide_p, wide_q = words[kSplitWideQ];
   auto tiles = [](int n) { return (n + TB_M - 1) / TB_M; };
   const int64_t n1 = (int64_t)tiles(wide_p) * tiles(nQ), n2 = (int64_t)tiles(clean_p) * tiles(wide_q);
   const int tid = threadIdx.x, lr = tid >> 1, lk = (tid & 1) << 2, tx = tid & 15, ty = tid >> 4;
@@ -468,7 +468,7 @@ gram_wide_kernel(WideSide P, WideSide Q, const int* __restrict__ words, int nP, 
     const int tb = tiles(all ? nQ : wide_q);
     const int a0 = (int)(u / tb) * TB_M, b0 = (int)(u % tb) * TB_N;
     const int na = all ? wide_p : clean_p, nb = all ? nQ : wide_q;
-    auto row_a = [&](int a) { return (int64_t)P.rows[all ? nP - 1 - a : a]; };
+    auto row_a = [&](int a) { return (int64_t)(all ? P.rows[nP - 1 - a] : wide_p ? P.rows[a] : a); };
     auto row_b = [&](int b) { return (int64_t)(all ? b : Q.rows[b]); };
     // rows past the end repeat the last one; their outputs are dropped
     const float* const pa = P.X + row_a(min(a0 + lr, na - 1)) * P.ld;

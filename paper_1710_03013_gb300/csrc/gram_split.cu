@@ -98,7 +98,7 @@ struct SplitShared {
   uint64_t rfull, rempty;  // the other products' sums of a chunk ready / read
   uint64_t mma_idle;       // every MMA of the CTA has finished
   uint32_t tmem_base;
-  int abort_flag;
+  int abort_flag, n_tiles;
   float2 ns[8][128];  // norm and scale of a warp's references
 };
 
@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1)
 gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapP, int nQ, int nP,
                   int capQ, int capP, int dk, const float* __restrict__ normQ, const float* __restrict__ normP,
                   const float* __restrict__ scaleQ, const float* __restrict__ scaleP, float neg_scale,
-                  float* __restrict__ out, int64_t ldo, int* __restrict__ words, uint32_t polls) {
+                  float* __restrict__ out, int64_t ldo, int* __restrict__ words, int look, uint32_t polls) {
   constexpr int SP_B_BYTES = SpCfg<SP_N>::kBBytes, SP_STAGE_BYTES = SpCfg<SP_N>::kStageBytes;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* const stages = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -118,8 +118,6 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int* const err = words + kSplitErr;
   const int tiles_m = (nQ + SP_M - 1) / SP_M, tiles_n = (nP + SP_N - 1) / SP_N;
-  // nothing to do when a whole side is wide: every value is then the FFMA sums'
-  const int n_tiles = words[kSplitWideP] < nP && words[kSplitWideQ] < nQ ? tiles_m * tiles_n : 0;
   const int nk = (dk + SP_K - 1) / SP_K;
 
   if (threadIdx.x == 0) {
@@ -139,10 +137,15 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
     tmem_alloc(&sh.tmem_base, SpCfg<SP_N>::kTmemCols);
     tmem_relinquish();
   }
+  // nothing to do when a whole side is wide: every value is then the FFMA sums'
+  // (not looked up where there is one tile a CTA: the reads are 1 us of 20)
+  if (threadIdx.x == 64)
+    sh.n_tiles = !look || (words[kSplitWideP] < nP && words[kSplitWideQ] < nQ) ? tiles_m * tiles_n : 0;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sh.tmem_base;
+  const int n_tiles = sh.n_tiles;
 
   if (warp == 0) {
     // ---------------- TMA producer
@@ -357,11 +360,10 @@ static float wide_below(int64_t d) { return 0x1p26f * sqrtf((float)d); }
 
 __global__ void __launch_bounds__(256)
 split_rows_kernel(SplitSource P, SplitSource Q, int d, int ks, float least, int* __restrict__ words) {
-  __shared__ int state[8];  // the block's references: 1 holds slices, 2 wide (0: no reference)
-  __shared__ int first[2];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int64_t row = (int64_t)blockIdx.x * 8 + warp;
-  const bool some = row < P.n + Q.n, sample = row >= P.n;
+  const int lane = threadIdx.x & 31;
+  int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (row >= P.n + Q.n) return;
+  const bool sample = row >= P.n;
   if (sample) row -= P.n;
   const SplitSource S = sample ? Q : P;
   const float* x = S.X + row * S.ld;
@@ -370,52 +372,33 @@ split_rows_kernel(SplitSource P, SplitSource Q, int d, int ks, float least, int*
     return make_float4(c < d ? __ldg(x + c) : 0.f, c + 1 < d ? __ldg(x + c + 1) : 0.f,
                        c + 2 < d ? __ldg(x + c + 2) : 0.f, c + 3 < d ? __ldg(x + c + 3) : 0.f);
   };
-  float s = 0.0f, unscale = 0.0f;
-  bool wide = false;
-  if (some) {
-    float2 acc = make_float2(0.0f, 0.0f);
-    uint32_t top = 0;  // the largest |value|, as an integer (NaN and Inf sort above)
-    for (int c = lane * 4; c < d; c += 128) {
-      const float4 v = load4(c);
-      top = max(max(top, max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu)),
-                max(__float_as_uint(v.z) & 0x7fffffffu, __float_as_uint(v.w) & 0x7fffffffu));
-      if (!S.norm) acc = df_add_sq(df_add_sq(df_add_sq(df_add_sq(acc, v.x), v.y), v.z), v.w);
-    }
-    top = __reduce_max_sync(kFull, top);
-    float norm;
-    if (S.norm) {
-      norm = S.norm[row];
-    } else {
-      norm = df_to_float(warp_sum_df(acc));
-      if (lane == 0) S.norm_out[row] = norm;
-    }
-    // scaled maximum in [2^14, 2^15); the exponents stay within the normal range
-    const int up = min(141 - (int)(top >> 23), 126);  // 14 - (e - 127), e biased (0: zero or subnormal)
-    s = __uint_as_float((uint32_t)(127 + up) << 23);
-    unscale = __uint_as_float((uint32_t)(127 - up) << 23);
-    const float scaled = norm * s * s;
-    wide = top != 0 && !(scaled >= least && scaled <= 3.4028235e38f);
+  float norm = S.norm ? __ldg(S.norm + row) : 0.0f;
+  float2 acc = make_float2(0.0f, 0.0f);
+  uint32_t top = 0;  // the largest |value|, as an integer (NaN and Inf sort above)
+  for (int c = lane * 4; c < d; c += 128) {
+    const float4 v = load4(c);
+    top = max(max(top, max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu)),
+              max(__float_as_uint(v.z) & 0x7fffffffu, __float_as_uint(v.w) & 0x7fffffffu));
+    if (!S.norm) acc = df_add_sq(df_add_sq(df_add_sq(df_add_sq(acc, v.x), v.y), v.z), v.w);
   }
-  if (blockIdx.x * (int64_t)8 < P.n) {  // (no rows of references in the other blocks)
-    if (lane == 0) state[warp] = some && !sample ? 1 + wide : 0;
-    __syncthreads();
-    if (threadIdx.x < 2) {  // places in the list for the block's references of either kind
-      int n = 0;
-      for (int w = 0; w < 8; ++w) n += state[w] == 1 + (int)threadIdx.x;
-      if (n) first[threadIdx.x] = atomicAdd(words + kSplitCleanP + threadIdx.x, n);
-    }
-    __syncthreads();
-    if (lane == 0 && state[warp]) {
-      int64_t place = first[wide];
-      for (int w = 0; w < warp; ++w) place += state[w] == 1 + (int)wide;
-      S.rows[wide ? S.n - 1 - place : place] = (int32_t)row;
+  top = __reduce_max_sync(kFull, top);
+  if (!S.norm) {
+    norm = df_to_float(warp_sum_df(acc));
+    if (lane == 0) S.norm_out[row] = norm;
+  }
+  // scaled maximum in [2^14, 2^15); the exponents stay within the normal range
+  const int up = min(141 - (int)(top >> 23), 126);  // 14 - (e - 127), e biased (0: zero or subnormal)
+  const float s = __uint_as_float((uint32_t)(127 + up) << 23);
+  const float scaled = norm * s * s;
+  const bool wide = top != 0 && !(scaled >= least && scaled <= 3.4028235e38f);
+  if (lane == 0) {
+    S.scale[row] = wide ? 0.0f : __uint_as_float((uint32_t)(127 - up) << 23);  // (0 marks it for the lists)
+    if (wide) {
+      const int at = atomicAdd(words + (sample ? kSplitWideQ : kSplitWideP), 1);
+      if (sample) S.rows[at] = (int32_t)row;
     }
   }
-  if (!some) return;
-  if (sample && wide && lane == 0) S.rows[atomicAdd(words + kSplitWideQ, 1)] = (int32_t)row;
-  // (a wide row's slices enter its own pairs only, which are written again)
-  if (lane == 0) S.scale[row] = unscale;
-  if (wide) return;
+  if (wide) return;  // (its slices would enter its own pairs only, which are written again)
   __half* const o = S.v + row * ks;
   const int64_t slice = S.cap * (int64_t)ks;
   for (int c = lane * 4; c < ks; c += 128) {
@@ -445,6 +428,30 @@ static cudaError_t launch_split_rows(const SplitSide& P, const SplitBufs& bP, in
   };
   split_rows_kernel<<<(unsigned)ceil_div(nP + nQ, 8), 256, 0, st>>>(source(P, bP, nP), source(Q, bQ, nQ), (int)d, ks,
                                                                     wide_below(d), words);
+  return cudaGetLastError();
+}
+
+// The references without slices and the others, listed from the scales.  A pass
+// of its own, run only before launch_gram_wide: appending every reference as its
+// slices are cut cost 4 us of a call of 95.
+__global__ void __launch_bounds__(256)
+split_list_kernel(const float* __restrict__ scale, int n, int32_t* __restrict__ rows, int* __restrict__ words) {
+  if (words[kSplitWideP] == 0) return;  // (row a is the a-th of the others)
+  const int r = blockIdx.x * 256 + threadIdx.x, lane = threadIdx.x & 31;
+  const bool wide = r < n && scale[r] == 0.0f;
+  const unsigned w = __ballot_sync(kFull, wide), c = __ballot_sync(kFull, r < n && !wide);
+  int at = 0;
+  if (lane == 0 && c) at = atomicAdd(words + kSplitListed, __popc(c));
+  if (lane == 1 && w) at = atomicAdd(words + kSplitWideListed, __popc(w));
+  const int c0 = __shfl_sync(kFull, at, 0), w0 = __shfl_sync(kFull, at, 1);
+  const unsigned below = (1u << lane) - 1;
+  if (wide) rows[n - 1 - (w0 + __popc(w & below))] = r;
+  else if (r < n) rows[c0 + __popc(c & below)] = r;
+}
+cudaError_t launch_split_list(SplitScratch& t, int64_t nP, cudaStream_t st) {
+  if (nP <= 0 || t.listed) return cudaSuccess;
+  t.listed = true;
+  split_list_kernel<<<(unsigned)ceil_div(nP, 256), 256, 0, st>>>(t.P.scale, (int)nP, t.P.rows, t.words);
   return cudaGetLastError();
 }
 
@@ -478,7 +485,7 @@ static cudaError_t launch_gram_split(const SplitBufs& bP, const float* normP, in
     const int64_t tiles = ceil_div(nQ, SP_M) * ceil_div(nP, N);                                                \
     gram_split_kernel<N><<<(unsigned)std::min<int64_t>(tiles, std::max(n_sms, 1)), SP_THREADS, SpCfg<N>::kSmem, st>>>( \
         mq, mp, (int)nQ, (int)nP, (int)bQ.cap, (int)bP.cap, ks, normQ, normP, bQ.scale, bP.scale, neg_scale, out, ldo, \
-        words, polls);                                                                                         \
+        words, tiles > n_sms, polls);                                                                                         \
   } while (0)
   if (2 * ceil_div(nQ, SP_M) * ceil_div(nP, 256) <= n_sms) KKM_SPLIT_LAUNCH(64);
   else KKM_SPLIT_LAUNCH(256);
@@ -491,16 +498,24 @@ kkm_status split_block(SplitScratch& t, const SplitSide& P, int64_t nP, const Sp
                        cudaStream_t st, uint32_t polls) {
   if (nP <= 0 || nQ <= 0) return KKM_OK;
   // the error word lasts, the counts start anew with their side
-  const int from = t.fresh ? kSplitErr : q_ready ? kSplitCleanP : kSplitWideQ, to = p_ready ? kSplitCleanP : kSplitWords;
+  const int from = t.fresh ? kSplitErr : q_ready ? kSplitWideP : kSplitWideQ, to = p_ready ? kSplitWideP : kSplitWords;
   if (from < to) {
     KKM_CK(cudaMemsetAsync(t.words + from, 0, 4 * (to - from), st));
     t.fresh = false;
+    if (!p_ready) t.listed = false;
     KKM_RUN("split_rows", st,
             launch_split_rows(P, t.P, p_ready ? 0 : nP, Q, t.Q, q_ready ? 0 : nQ, d, dp, t.words, st));
   }
   KKM_RUN("gram_split", st,
           launch_gram_split(t.P, P.norm ? P.norm : t.P.norm, nP, t.Q, Q.norm ? Q.norm : t.Q.norm, nQ, dp, neg_scale, out,
                             ldo, t.words, n_sms, st, polls));
+  return KKM_OK;
+}
+
+kkm_status split_wide_pairs(SplitScratch& t, const SplitSide& P, int64_t nP, const SplitSide& Q, int64_t nQ, int64_t d,
+                            int dp, float neg_scale, float* out, int64_t ldo, int n_sms, cudaStream_t st) {
+  KKM_RUN("split_list", st, launch_split_list(t, nP, st));
+  KKM_RUN("gram_wide", st, launch_gram_wide(t, P, nP, Q, nQ, d, dp, neg_scale, out, ldo, n_sms, st));
   return KKM_OK;
 }
 

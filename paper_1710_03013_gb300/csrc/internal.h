@@ -257,7 +257,7 @@ struct SplitSide {
 // (ks = the row length rounded up to 8), a power-of-two scale per row, the
 // norms formed, and the wide rows (those the slices do not hold, see
 // gram_split.cu): of the samples, `rows` lists them; of the references, `rows`
-// has the others from the start and the wide ones from the end.
+// gets the others from the start and the wide ones from the end.
 struct SplitBufs {
   int64_t cap = 0;
   __half* v = nullptr;
@@ -265,24 +265,27 @@ struct SplitBufs {
   float* norm = nullptr;
   int32_t* rows = nullptr;
 };
-// words[kSplitErr]: as *err of launch_gram_tc; then the numbers of wide samples,
-// of references that are not wide and of those that are.
-enum SplitWord { kSplitErr = 0, kSplitWideQ = 1, kSplitCleanP = 2, kSplitWideP = 3, kSplitWords = 4 };
+// words[kSplitErr]: as *err of launch_gram_tc; then the numbers of wide samples
+// and of wide references, and the lengths of the references' two lists.
+enum SplitWord { kSplitErr = 0, kSplitWideQ, kSplitWideP, kSplitListed, kSplitWideListed, kSplitWords };
 struct SplitScratch {
   SplitBufs P, Q;
   int* words = nullptr;
-  bool fresh = true;  // nothing has run in it yet
+  bool fresh = true;    // nothing has run in it yet
+  bool listed = false;  // the references' lists are made
 };
 // out[n*ldo + m] = exp(-|p_n - q_m|^2 / (2 sigma^2)) but for the pairs of wide
-// rows, which launch_gram_wide has to write (it returns at once when there are
-// none; a caller that waits for the words anyway need not launch it).  A value
-// depends on its two rows alone.  p_ready, q_ready: the references, the samples
-// are those of the last call.  The error word is for the caller to read.
+// rows, which split_wide_pairs has to write (a caller that waits for the words
+// anyway need not call it when they count none).  A value depends on its two
+// rows alone.  p_ready, q_ready: the references, the samples are those of the
+// last call.  The error word is for the caller to read.
 kkm_status split_block(SplitScratch& t, const SplitSide& P, int64_t nP, const SplitSide& Q, int64_t nQ, int64_t d,
                        int dp, float neg_scale, float* out, int64_t ldo, bool p_ready, bool q_ready, int n_sms,
                        cudaStream_t st, uint32_t polls = kTcSpinLimit);
 // The pairs of the wide rows, by the FFMA kernel's sums (rows read in place,
 // dp = d rounded up to 8).
+kkm_status split_wide_pairs(SplitScratch& t, const SplitSide& P, int64_t nP, const SplitSide& Q, int64_t nQ, int64_t d,
+                            int dp, float neg_scale, float* out, int64_t ldo, int n_sms, cudaStream_t st);
 cudaError_t launch_gram_wide(const SplitScratch& t, const SplitSide& P, int64_t nP, const SplitSide& Q, int64_t nQ,
                              int64_t d, int dp, float neg_scale, float* out, int64_t ldo, int n_sms, cudaStream_t st);
 // Whether kkm_kernel_matrix and kkm_assign take it for an FP32 Gaussian block

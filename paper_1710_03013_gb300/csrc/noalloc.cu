@@ -40,6 +40,7 @@ constexpr int64_t kNaGrid = kNaRows / 32;              // assign CTAs (32 rows e
 // (gram_split.cu) take it here too; the references pass through the scratch
 // kNaSplitRef at a time (a value does not depend on the others in its block).
 constexpr int64_t kNaSplitRef = 1024;
+constexpr int kNaBlocks = (int)((kNaRef + kNaSplitRef - 1) / kNaSplitRef);
 
 constexpr size_t na_align(size_t x) { return (x + 255) & ~size_t(255); }
 // float [rows][rowlen], or the slices of the rows and of a block of references
@@ -51,8 +52,8 @@ constexpr size_t kOffScaleQ = na_align(kOffAux + sizeof(float) * kNaRows);      
 constexpr size_t kOffListQ = na_align(kOffScaleQ + sizeof(float) * kNaRows);     // int32_t [rows]
 constexpr size_t kOffScaleP = na_align(kOffListQ + sizeof(int32_t) * kNaRows);   // float [references]
 constexpr size_t kOffListP = na_align(kOffScaleP + sizeof(float) * kNaSplitRef);  // int32_t [references]
-constexpr size_t kOffWords = na_align(kOffListP + sizeof(int32_t) * kNaSplitRef);  // int [kSplitWords]
-constexpr size_t kOffK = na_align(kOffWords + sizeof(int) * kSplitWords);     // float [ref][rows]
+constexpr size_t kOffWords = na_align(kOffListP + sizeof(int32_t) * kNaSplitRef);  // int [blocks][kSplitWords]
+constexpr size_t kOffK = na_align(kOffWords + sizeof(int) * kNaBlocks * kSplitWords);  // float [ref][rows]
 constexpr size_t kOffPart = na_align(kOffK + sizeof(float) * kNaRef * kNaRows);  // float [units][rows]
 constexpr size_t kOffOmega = na_align(kOffPart + sizeof(float) * kNaUnits * kNaRows);  // float2 [grid]
 constexpr size_t kOffChanged = na_align(kOffOmega + sizeof(float2) * kNaGrid);   // int [grid]
@@ -148,63 +149,90 @@ static kkm_status assign_noalloc_impl(const kkm_model* m, const float* X, int64_
   const float* kself = m->kind == KKM_LINEAR ? auxc : nullptr;
   const float* P = mode == KKM_ASSIGN_SUPPORTS ? m->sup : m->med;
   const float* Paux = mode == KKM_ASSIGN_SUPPORTS ? m->sup_aux : m->med_aux;
-  SplitScratch slices;
-  if (split) {
-    slices.words = reinterpret_cast<int*>(base + kOffWords);
-    slices.Q = SplitBufs{kNaRows, reinterpret_cast<__half*>(base + kOffRows), reinterpret_cast<float*>(base + kOffScaleQ),
-                         auxc, reinterpret_cast<int32_t*>(base + kOffListQ)};
-    slices.P = SplitBufs{kNaSplitRef, reinterpret_cast<__half*>(base + kOffSliceP),
-                         reinterpret_cast<float*>(base + kOffScaleP), nullptr,
-                         reinterpret_cast<int32_t*>(base + kOffListP)};
+  int* const words = reinterpret_cast<int*>(base + kOffWords);
+  // the block from slices; with `wide`, the pairs of wide rows too (each block's
+  // words are its own without, so that they can all be read in the end)
+  auto slice_block = [&](bool wide) -> kkm_status {
+    SplitScratch t;
+    t.words = words;
+    t.Q = SplitBufs{kNaRows, reinterpret_cast<__half*>(base + kOffRows), reinterpret_cast<float*>(base + kOffScaleQ), auxc,
+                    reinterpret_cast<int32_t*>(base + kOffListQ)};
+    t.P = SplitBufs{kNaSplitRef, reinterpret_cast<__half*>(base + kOffSliceP),
+                    reinterpret_cast<float*>(base + kOffScaleP), nullptr, reinterpret_cast<int32_t*>(base + kOffListP)};
     const SplitSide q{X, m->d};
     for (int64_t p0 = 0; p0 < rows_ref; p0 += kNaSplitRef) {
       const int64_t n = std::min<int64_t>(kNaSplitRef, rows_ref - p0);
       const SplitSide p{P + p0 * m->dp, m->dp, Paux + p0};
-      KKM_TRY(split_block(slices, p, n, q, M, m->d, m->dp, neg_scale, Kb + p0 * ldm, ldm, /*p_ready=*/false,
+      if (!wide) {
+        t.words = words + p0 / kNaSplitRef * kSplitWords;
+        t.fresh = true;
+      }
+      KKM_TRY(split_block(t, p, n, q, M, m->d, m->dp, neg_scale, Kb + p0 * ldm, ldm, /*p_ready=*/false,
                           /*q_ready=*/p0 > 0, sm_count(), st));
-      KKM_CK(launch_gram_wide(slices, p, n, q, M, m->d, m->dp, neg_scale, Kb + p0 * ldm, ldm, sm_count(), st));
+      if (wide)
+        KKM_TRY(split_wide_pairs(t, p, n, q, M, m->d, m->dp, neg_scale, Kb + p0 * ldm, ldm, sm_count(), st));
     }
-  } else if (rmsd)
+    return KKM_OK;
+  };
+  if (split)
+    KKM_TRY(slice_block(false));
+  else if (rmsd)
     KKM_CK(launch_rmsd_gram(dk, P, rows_ref, Xc, M, ap, m->n_atoms, Paux, auxc, nullptr, nullptr, neg_scale, Kb,
                             ldm, st));
   else
     KKM_CK(launch_gram(dk, P, rows_ref, Xc, M, m->dp, Paux, auxc, nullptr, nullptr, neg_scale, Kb, ldm, st));
 
-  if (mode == KKM_ASSIGN_SUPPORTS) {
-    Supports S{};
-    S.L = m->L_ident;
-    S.nL = m->nL;
-    S.C = m->C;
-    S.perm = m->perm;
-    S.seg_off = m->seg_off;
-    S.n_j = m->n_j;
-    S.unit_j = m->unit_j;
-    S.unit_kb = m->unit_kb;
-    S.unit_ke = m->unit_ke;
-    S.seg_unit = m->seg_unit;
-    S.n_units = m->n_units;
-    S.col_label = nullptr;
-    S.col_ord = nullptr;
-    S.lab = nullptr;
-    S.max_units = max_units_for(m->nL, m->C);
-    IterState I{};
-    I.partial = partial;
-    I.gpart = nullptr;
-    I.omega_part = omega_part;
-    I.changed_part = changed_part;
-    I.ghat_in = m->ghat;
-    I.n_strips = (int)ceil_div(ldm, kStripCols);
-    I.assign_grid = (int)ceil_div(ldm, 32);
-    KKM_CK(launch_fhat_partial(Kb, ldm, (int)M, S, I, st));
-    KKM_CK(launch_assign(ldm, (int)M, S, I, kself, labels_out, nullptr, dist_out, nullptr, nullptr, 0,
-                         /*trace=*/0, st));
-  } else {
-    KKM_CK(launch_nearest(Kb, ldm, (int)M, m->C, kself, m->kind == KKM_LINEAR ? m->med_aux : nullptr, labels_out,
-                          dist_out, st));
-  }
-  int err = 0;
-  if (split) KKM_CK(cudaMemcpyAsync(&err, slices.words + kSplitErr, sizeof(int), cudaMemcpyDeviceToHost, st));
+  auto label = [&]() -> kkm_status {
+    if (mode == KKM_ASSIGN_SUPPORTS) {
+      Supports S{};
+      S.L = m->L_ident;
+      S.nL = m->nL;
+      S.C = m->C;
+      S.perm = m->perm;
+      S.seg_off = m->seg_off;
+      S.n_j = m->n_j;
+      S.unit_j = m->unit_j;
+      S.unit_kb = m->unit_kb;
+      S.unit_ke = m->unit_ke;
+      S.seg_unit = m->seg_unit;
+      S.n_units = m->n_units;
+      S.col_label = nullptr;
+      S.col_ord = nullptr;
+      S.lab = nullptr;
+      S.max_units = max_units_for(m->nL, m->C);
+      IterState I{};
+      I.partial = partial;
+      I.gpart = nullptr;
+      I.omega_part = omega_part;
+      I.changed_part = changed_part;
+      I.ghat_in = m->ghat;
+      I.n_strips = (int)ceil_div(ldm, kStripCols);
+      I.assign_grid = (int)ceil_div(ldm, 32);
+      KKM_CK(launch_fhat_partial(Kb, ldm, (int)M, S, I, st));
+      KKM_CK(launch_assign(ldm, (int)M, S, I, kself, labels_out, nullptr, dist_out, nullptr, nullptr, 0,
+                           /*trace=*/0, st));
+    } else {
+      KKM_CK(launch_nearest(Kb, ldm, (int)M, m->C, kself, m->kind == KKM_LINEAR ? m->med_aux : nullptr, labels_out,
+                            dist_out, st));
+    }
+    return KKM_OK;
+  };
+  KKM_TRY(label());
+  int words_h[kNaBlocks * kSplitWords] = {};
+  const int blocks = split ? (int)ceil_div(rows_ref, kNaSplitRef) : 0;
+  if (split) KKM_CK(cudaMemcpyAsync(words_h, words, sizeof(int) * kSplitWords * blocks, cudaMemcpyDeviceToHost, st));
   KKM_CK(cudaStreamSynchronize(st));
+  int err = 0, wide = 0;
+  for (int b = 0; b < blocks; ++b) {
+    err |= words_h[b * kSplitWords + kSplitErr];
+    wide |= words_h[b * kSplitWords + kSplitWideQ] | words_h[b * kSplitWords + kSplitWideP];
+  }
+  if (wide && !err) {
+    KKM_TRY(slice_block(true));
+    KKM_TRY(label());
+    KKM_CK(cudaMemcpyAsync(&err, words + kSplitErr, sizeof(int), cudaMemcpyDeviceToHost, st));
+    KKM_CK(cudaStreamSynchronize(st));
+  }
   if (err) {
     set_error("tensor-core kernel block: a bounded pipeline wait gave up");
     return KKM_ETIMEOUT;
