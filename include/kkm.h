@@ -51,8 +51,8 @@ typedef enum kkm_kernel_kind { KKM_RBF = 0, KKM_RMSD = 1, KKM_LINEAR = 2 } kkm_k
 
 /* Arithmetic of the kernel-block evaluation K(X^i, L).  KKM_FP32 is the
  * FP32 path: FFMA, or for the Gaussian blocks of kkm_kernel_matrix and
- * kkm_assign (more than 32 reference rows, d >= 64) FP16 products of three
- * slices of each row on the tensor cores, whose error against 64 bits is no
+ * kkm_assign (from 1,024 reference rows with d >= 64, 128 with d >= 96, 33 with
+ * d >= 128) FP16 products of three slices of each row on the tensor cores, whose error against 64 bits is no
  * larger than FFMA's: squared distances to about one unit of
  * 2^-24 (|x|^2 + |y|^2) rms on either.  Rows that the slices do not hold as
  * well (NaN, Inf, a squared norm outside the FP32 range, a largest value far

@@ -291,16 +291,19 @@ cudaError_t launch_gram_wide(const SplitScratch& t, const SplitSide& P, int64_t 
 // Whether kkm_kernel_matrix and kkm_assign take it for an FP32 Gaussian block
 // against nA reference rows of d values: a rule on the references alone, so
 // that a sample's values do not depend on how many samples share the call.  Up
-// to 32 references have the skinny kernel.  From 64 values on it is no slower
-// than the FFMA kernel at any size measured (us a call, FFMA / here: assign of
-// 1 row to 200 supports 73.8 / 76.8 at d = 64 and 82.8 / 75.5 at d = 128, of
-// 2,000 rows to 3,000 supports 98 / 101 and 119 / 101; a 5,000 x 20,000 matrix
-// 382 / 332 at d = 48, 695 / 355 at d = 128; at d = 16 245 / 325).  Fits keep
-// the FFMA kernel: their labels at near ties follow the block's last bits, and
-// a resumed checkpoint has to go on as it began.
-constexpr int64_t kSplitMinDim = 64;
+// to 32 references have the skinny kernel.  Measured (us a call of kkm_assign,
+// median of 3 runs, FFMA / slices, for 1, 4,000 and 20,000 rows):
+//   d    40 references              400                       2,000
+//   64   77/85    83/86   100/113   79/79   84/87   135/121   80/81  112/106  258/190
+//   96   76/77    82/82   102/110   82/78   88/87   144/122   83/81  123/106  309/196
+//   128  79/75    86/83   110/112   84/78   92/89   161/120   86/81  134/105  361/199
+// Few references leave most of a tile empty and short rows little to do in it,
+// so a line between them costs the less the more references there are; where
+// slices lose at all from these lines on, it is within 3 us of a call.  Fits
+// keep the FFMA kernel: their labels at near ties follow the block's last bits,
+// and a resumed checkpoint has to go on as it began.
 constexpr bool split_applies(int kind, int64_t nA, int64_t d) {
-  return kind == KKM_RBF && nA > 32 && d >= kSplitMinDim && 3 * nA <= INT32_MAX;
+  return kind == KKM_RBF && nA > 32 && d >= (nA >= 1024 ? 64 : nA >= 128 ? 96 : 128) && 3 * nA <= INT32_MAX;
 }
 
 // ---- tensor-core (tcgen05) BF16 kernel block ----------------------------

@@ -1,6 +1,6 @@
 """kkm_assign_noalloc gives the bits of kkm_assign for RBF and linear models, as
 the header says, on either kernel block: FFMA (short rows, few references) and
-the FP16 slices (more than 32 references, 64 values and more), with the
+the FP16 slices (more references, longer rows), with the
 references in one block of its scratch, in several, and one past a block's end,
 and with rows that the slices do not hold among references and samples."""
 
@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("kind,n,d,C,mode", [
     ("rbf", 700, 100, 5, "supports"), ("rbf", 1025, 784, 10, "supports"), ("rbf", 3001, 130, 8, "supports"),
-    ("rbf", 600, 66, 40, "medoids"), ("rbf", 900, 1024, 33, "medoids"), ("rbf", 500, 48, 5, "supports"),
+    ("rbf", 1300, 66, 6, "supports"), ("rbf", 600, 130, 40, "medoids"), ("rbf", 900, 1024, 33, "medoids"), ("rbf", 500, 48, 5, "supports"),
     ("rbf", 300, 200, 7, "medoids"), ("linear", 800, 90, 5, "supports")])
 @pytest.mark.parametrize("wide", [False, True])
 def test_same_bits_as_assign(lib, kind, n, d, C, mode, wide):

@@ -44,8 +44,9 @@ def _ffma_sq_dist(A, B):
 def test_error_no_larger_than_ffma(lib, name, d):
     import torch
     g = np.random.default_rng(d)
-    X = _rows(name, 256 + 400, d, g).astype(np.float32)
-    A, B = X[:256], X[256:]
+    n = 1024 if d < 96 else 256
+    X = _rows(name, n + 400, d, g).astype(np.float32)
+    A, B = X[:n], X[n:]
     a, b = A.astype(np.float64), B.astype(np.float64)
     norms = (a * a).sum(1)[:, None] + (b * b).sum(1)[None, :]
     d2 = np.maximum(norms - 2 * a @ b.T, 0)

@@ -43,7 +43,7 @@ def _widen(X, which, g):
     return X
 
 
-@pytest.mark.parametrize("nA,nB,d", [(40, 1, 64), (129, 127, 66), (300, 700, 131), (257, 4100, 784), (513, 300, 100)])
+@pytest.mark.parametrize("nA,nB,d", [(33, 1, 128), (1025, 127, 66), (300, 700, 131), (257, 4100, 784), (513, 300, 100)])
 @pytest.mark.parametrize("share", ["one", "few", "half", "most", "all"])
 def test_wide_rows_against_64_bits(lib, nA, nB, d, share):
     g = np.random.default_rng(nA + d)
@@ -71,7 +71,7 @@ def test_a_value_depends_on_its_two_rows_alone(lib):
     ra, rb = np.setdiff1d(np.arange(500), [3, 400, 250]), np.setdiff1d(np.arange(1200), [0, 700, 17, 40])
     assert np.array_equal(K2[np.ix_(ra, rb)], K[np.ix_(ra, rb)])
     # the wide rows' values do not depend on the company either
-    sub = _matrix(lib, A2[[3, 400] + list(range(40, 80))], B2[[700, 0]], sigma)
+    sub = _matrix(lib, A2[[3, 400] + list(range(40, 180))], B2[[700, 0]], sigma)
     assert np.array_equal(sub[:2], K2[np.ix_([3, 400], [700, 0])])
     # nor on where the rows lie: unaligned rows of an odd pitch
     import torch
