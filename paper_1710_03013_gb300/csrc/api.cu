@@ -735,14 +735,28 @@ static kkm_status kernel_block_fp8(const KernelSpec& sp, const float* P, const i
 }
 
 // Scratch of the FP32 Gaussian block on the tensor cores for nP references and
-// nQ samples, one allocation.
+// nQ samples, one allocation.  The slices take half as much again as the FP32
+// rows that the FFMA kernel reads; where that is not to be had, the block is
+// made in parts of at most kSplitPartBytes of slices a side (its values are the
+// same), so that what fits with the FFMA kernel fits.
+constexpr int64_t kSplitPartBytes = (int64_t)64 << 20;
 static kkm_status alloc_split(Workspace& ws, const KernelSpec& sp, int64_t nP, int64_t nQ, SplitScratch* t) {
   auto part = [](int64_t bytes) { return round_up(bytes, 256); };
+  auto bytes = [&](int64_t p, int64_t q) {
+    return 256 + part(6 * p * sp.dp) + part(6 * q * sp.dp) + 3 * part(4 * p) + 3 * part(4 * q);
+  };
   char* at;
-  KKM_TRY(ws.alloc(&at, 256 + part(6 * nP * sp.dp) + part(6 * nQ * sp.dp) + 3 * part(4 * nP) + 3 * part(4 * nQ)));
-  auto take = [&](int64_t bytes) {
+  kkm_status rc = ws.alloc(&at, bytes(nP, nQ));
+  if (rc == KKM_ENOMEM) {
+    const int64_t rows = std::max<int64_t>(256, kSplitPartBytes / (6 * sp.dp));
+    nP = std::min(nP, rows);
+    nQ = std::min(nQ, rows);
+    rc = ws.alloc(&at, bytes(nP, nQ));
+  }
+  if (rc != KKM_OK) return rc;
+  auto take = [&](int64_t n) {
     char* const p = at;
-    at += part(bytes);
+    at += part(n);
     return p;
   };
   t->words = reinterpret_cast<int*>(take(4 * kSplitWords));
@@ -753,6 +767,27 @@ static kkm_status alloc_split(Workspace& ws, const KernelSpec& sp, int64_t nP, i
     s->norm = reinterpret_cast<float*>(take(4 * s->cap));
     s->rows = reinterpret_cast<int32_t*>(take(4 * s->cap));
   }
+  return KKM_OK;
+}
+// split_block in the parts that the scratch holds.  Returns in *whole whether it
+// was one: the pairs of wide rows are then the caller's to write when the words
+// count some, else they are written.  again: the references are those of the
+// last call.
+static kkm_status split_parts(SplitScratch& t, const KernelSpec& sp, const SplitSide& P, int64_t nP, const SplitSide& Q,
+                              int64_t nQ, float* out, int64_t ldo, bool again, bool* whole, cudaStream_t st,
+                              uint32_t polls = kTcSpinLimit) {
+  const bool one_p = nP <= t.P.cap;
+  *whole = one_p && nQ <= t.Q.cap;
+  for (int64_t q0 = 0; q0 < nQ; q0 += t.Q.cap)
+    for (int64_t p0 = 0; p0 < nP; p0 += t.P.cap) {
+      const int64_t np = std::min(t.P.cap, nP - p0), nq = std::min(t.Q.cap, nQ - q0);
+      const SplitSide p{P.X + p0 * P.ld, P.ld, P.norm ? P.norm + p0 : nullptr}, q{Q.X + q0 * Q.ld, Q.ld};
+      float* const o = out + p0 * ldo + q0;
+      KKM_TRY(split_block(t, p, np, q, nq, sp.d, sp.dp, sp.neg_scale(), o, ldo, one_p && (again || q0 > 0), p0 > 0,
+                          sm_count(), st, polls));
+      if (!*whole)
+        KKM_TRY(split_wide_pairs(t, p, np, q, nq, sp.d, sp.dp, sp.neg_scale(), o, ldo, sm_count(), st));
+    }
   return KKM_OK;
 }
 
@@ -2045,12 +2080,12 @@ static kkm_status assign_impl(const kkm_model* m, const float* Xnew_in, int64_t 
     return split_wide_pairs(slices, ref, rows_ref, SplitSide{X + c0 * d, d}, n, d, sp.dp, sp.neg_scale(), Kb, ldm,
                             sm_count(), st);
   };
+  bool whole = true;
   for (int64_t c0 = 0; c0 < M; c0 += chunk) {
     const int n = (int)std::min<int64_t>(chunk, M - c0);
     if (split) {
-      KKM_TRY(split_block(slices, ref, rows_ref, SplitSide{X + c0 * d, d}, n, d, sp.dp, sp.neg_scale(), Kb, ldm,
-                          /*p_ready=*/c0 > 0, /*q_ready=*/false, sm_count(), st));
-      if (M > chunk) KKM_TRY(wide_pairs(c0, n));
+      KKM_TRY(split_parts(slices, sp, ref, rows_ref, SplitSide{X + c0 * d, d}, n, Kb, ldm, /*again=*/c0 > 0, &whole, st));
+      if (M > chunk && whole) KKM_TRY(wide_pairs(c0, n));
     } else {
       KKM_TRY(prep_rows(sp, X, c0, 1, n, Xc, auxc, st));
       if (mode == KKM_ASSIGN_SUPPORTS)
@@ -2073,7 +2108,7 @@ static kkm_status assign_impl(const kkm_model* m, const float* Xnew_in, int64_t 
     // one chunk: its block is still there, and the pairs of wide rows are
     // written into it only now that the wait has told of some (a launch that
     // finds none is 6 us of a call of 100)
-    if (M <= chunk && (words_h[kSplitWideQ] || words_h[kSplitWideP])) {
+    if (M <= chunk && whole && (words_h[kSplitWideQ] || words_h[kSplitWideP])) {
       KKM_TRY(wide_pairs(0, (int)M));
       KKM_TRY(label(0, (int)M));
       waited = false;
@@ -2144,13 +2179,13 @@ static kkm_status kernel_matrix_impl(const float* A_in, int64_t nA, const float*
     const SplitSide sA{A, d}, sB{Bm, d};
     int words_h[kSplitWords] = {};
     KKM_TRY(alloc_split(ws, sp, nA, nB, &t));
-    KKM_TRY(split_block(t, sA, nA, sB, nB, d, sp.dp, sp.neg_scale(), o, nB, /*p_ready=*/false,
-                        /*q_ready=*/false, sm_count(), st, polls));
+    bool whole = true;
+    KKM_TRY(split_parts(t, sp, sA, nA, sB, nB, o, nB, /*again=*/false, &whole, st, polls));
     KKM_CK(cudaMemcpyAsync(words_h, t.words, sizeof words_h, cudaMemcpyDeviceToHost, st));
     KKM_CK(cudaStreamSynchronize(st));
     tc_err_h = words_h[kSplitErr];
     waited = true;
-    if (words_h[kSplitWideQ] || words_h[kSplitWideP]) {
+    if (whole && (words_h[kSplitWideQ] || words_h[kSplitWideP])) {
       KKM_TRY(split_wide_pairs(t, sA, nA, sB, nB, d, sp.dp, sp.neg_scale(), o, nB, sm_count(), st));
       waited = false;
     }
