@@ -738,19 +738,25 @@ static kkm_status kernel_block_fp8(const KernelSpec& sp, const float* P, const i
 // nQ samples, one allocation.  The slices take half as much again as the FP32
 // rows that the FFMA kernel reads; where that is not to be had, the block is
 // made in parts of at most kSplitPartBytes of slices a side (its values are the
-// same), so that what fits with the FFMA kernel fits.
+// same), so that what fits with the FFMA kernel fits.  limit (0: none): the
+// bytes that the caller has for it.
 constexpr int64_t kSplitPartBytes = (int64_t)64 << 20;
-static kkm_status alloc_split(Workspace& ws, const KernelSpec& sp, int64_t nP, int64_t nQ, SplitScratch* t) {
+static kkm_status alloc_split(Workspace& ws, const KernelSpec& sp, int64_t nP, int64_t nQ, SplitScratch* t,
+                              int64_t limit = 0) {
   auto part = [](int64_t bytes) { return round_up(bytes, 256); };
   auto bytes = [&](int64_t p, int64_t q) {
     return 256 + part(6 * p * sp.dp) + part(6 * q * sp.dp) + 3 * part(4 * p) + 3 * part(4 * q);
   };
-  char* at;
-  kkm_status rc = ws.alloc(&at, bytes(nP, nQ));
-  if (rc == KKM_ENOMEM) {
-    const int64_t rows = std::max<int64_t>(256, kSplitPartBytes / (6 * sp.dp));
+  auto cut = [&](int64_t part_bytes) {
+    const int64_t rows = std::max<int64_t>(32, part_bytes / split_bytes(1, sp.dp));
     nP = std::min(nP, rows);
     nQ = std::min(nQ, rows);
+  };
+  char* at;
+  if (limit > 0 && split_bytes(nP + nQ, sp.dp) > limit) cut(limit / 2);
+  kkm_status rc = ws.alloc(&at, bytes(nP, nQ));
+  if (rc == KKM_ENOMEM) {
+    cut(kSplitPartBytes);
     rc = ws.alloc(&at, bytes(nP, nQ));
   }
   if (rc != KKM_OK) return rc;
@@ -1984,7 +1990,7 @@ namespace kkm {
 // ======================================================================
 static kkm_status assign_impl(const kkm_model* m, const float* Xnew_in, int64_t M, int32_t mode,
                               int32_t* labels_out, float* dist_out, double* omega_out,
-                              cudaStream_t st) {
+                              cudaStream_t st, int64_t slice_bytes = 0) {
   NvtxRange nv("kkm_assign");
   if (!m) return invalid("model is NULL");
   if (M < 0 || M > INT32_MAX) return invalid("M must be in [0, 2^31)");
@@ -2032,7 +2038,7 @@ static kkm_status assign_impl(const kkm_model* m, const float* Xnew_in, int64_t 
   const SplitSide ref{mode == KKM_ASSIGN_SUPPORTS ? m->sup : m->med, sp.dp,
                       mode == KKM_ASSIGN_SUPPORTS ? m->sup_aux : m->med_aux};
   if (split) {
-    KKM_TRY(alloc_split(ws, sp, rows_ref, std::min(chunk, M), &slices));
+    KKM_TRY(alloc_split(ws, sp, rows_ref, std::min(chunk, M), &slices, slice_bytes));
   } else {
     KKM_TRY(ws.alloc(&Xc, ldm * sp.dp));
     KKM_TRY(ws.alloc(&auxc, ldm));
@@ -2405,6 +2411,12 @@ static kkm_status guarded(F&& f) {
     set_error("internal exception");
     return KKM_EINTERNAL;
   }
+}
+
+kkm_status assign_within(const kkm_model* m, const float* X, int64_t M, int32_t mode, int32_t* labels_out,
+                         float* dist_out, cudaStream_t st, int64_t slice_bytes) {
+  set_error("");
+  return guarded([&] { return assign_impl(m, X, M, mode, labels_out, dist_out, nullptr, st, slice_bytes); });
 }
 
 }  // namespace kkm

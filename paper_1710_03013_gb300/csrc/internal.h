@@ -306,6 +306,13 @@ constexpr bool split_applies(int kind, int64_t nA, int64_t d) {
   return kind == KKM_RBF && nA > 32 && d >= (nA >= 1024 ? 64 : nA >= 128 ? 96 : 128) && 3 * nA <= INT32_MAX;
 }
 
+// Bytes of the slices and their rows' other scratch for n rows of a side.
+constexpr int64_t split_bytes(int64_t n, int64_t dp) { return n * (6 * dp + 12); }
+// kkm_assign with at most slice_bytes of that scratch (0: as much as it takes,
+// parts when memory is short; see alloc_split).
+kkm_status assign_within(const kkm_model* m, const float* X, int64_t M, int32_t mode, int32_t* labels_out,
+                         float* dist_out, cudaStream_t st, int64_t slice_bytes);
+
 // ---- tensor-core (tcgen05) BF16 kernel block ----------------------------
 // out[n*ldo + m] = kappa(P_n, Q_m) for BF16 rows P [nP][ldb], Q [nQ][ldb]
 // (dk valid columns), with the squared norms of the BF16 rows; out is float,

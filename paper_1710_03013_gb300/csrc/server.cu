@@ -90,16 +90,26 @@ static uint64_t fit_bytes(const kkm_problem& p) {
 }
 
 // Device bytes of one kkm_assign call on M rows (device input and outputs
-// included), following its chunking of the kernel block.
-static uint64_t assign_bytes(const kkm_model* m, int64_t M, int32_t mode) {
+// included), following its chunking of the kernel block.  Of these, *slices are
+// the FP16 slices of a Gaussian block, for which the call makes do with
+// *slices_least (what the FP32 rows of the FFMA block would take) in parts.
+static uint64_t assign_bytes(const kkm_model* m, int64_t M, int32_t mode, uint64_t* slices, uint64_t* slices_least) {
   const int64_t rows_ref = mode == KKM_ASSIGN_SUPPORTS ? m->nL : m->C;
   const int64_t chunk = std::max<int64_t>(1024, std::min<int64_t>(M, ((int64_t)1 << 27) / std::max<int64_t>(rows_ref, 1)));
   const int64_t ldm = round_up(std::min(chunk, M), 32);
   const int64_t units = ceil_div(m->nL, kUnitRows) + m->C;
+  const uint64_t rows = 4ull * ldm * (m->dp + 1);
   uint64_t b = 4ull * M * m->d + 8ull * M;     // rows and outputs on the device
-  b += 4ull * ldm * (m->dp + 1) + 4ull * rows_ref * ldm;
+  b += 4ull * rows_ref * ldm;
   if (mode == KKM_ASSIGN_SUPPORTS) b += 4ull * units * ldm + 8ull * units * ceil_div(ldm, kStripCols);
-  if (split_applies(m->kind, rows_ref, m->d)) b += (6ull * m->dp + 12) * (rows_ref + ldm);
+  if (split_applies(m->kind, rows_ref, m->d)) {
+    *slices = (uint64_t)split_bytes(rows_ref + ldm, m->dp);
+    *slices_least = std::min(*slices, rows);
+    b += *slices;
+  } else {
+    *slices = *slices_least = 0;
+    b += rows;
+  }
   if (m->kind == KKM_RMSD)  // tensor-core MD path
     b += 18ull * round_up(m->n_atoms, 64) * (rows_ref + ldm) + 16ull * rows_ref * ldm + 8ull * rows_ref +
          rows_ref * rmsd_near_pitch(ldm) + 8ull * rmsd_max_units(rows_ref, ldm);
@@ -126,6 +136,8 @@ struct Job {
   float* dist_out = nullptr;
   // bookkeeping
   uint64_t bytes = 0;
+  uint64_t slices = 0, slices_least = 0;  // of an assign's bytes (see assign_bytes)
+  bool in_parts = false;                  // slices has been cut to slices_least
   int passed = 0;
   double evals = 0.0;
   Clock::time_point t_submit, t_start, t_end;
@@ -175,6 +187,16 @@ static double fit_evals(const kkm_problem& p) {
   return e + (double)(p.C - 1) * (double)((p.N + B - 1) / B);
 }
 
+// Whether a job fits in `room` bytes, an assign with its slices in parts if need be.
+static bool fits(Job& J, uint64_t room) {
+  if (J.bytes <= room) return true;
+  if (J.in_parts || J.bytes - (J.slices - J.slices_least) > room) return false;
+  J.bytes -= J.slices - J.slices_least;
+  J.slices = J.slices_least;
+  J.in_parts = true;
+  return true;
+}
+
 // Takes the next admissible job (and, for an assign, the waiting assigns it
 // can be fused with).  Called with the lock held.
 static std::vector<std::shared_ptr<Job>> take_jobs(kkm_server* s) {
@@ -186,7 +208,7 @@ static std::vector<std::shared_ptr<Job>> take_jobs(kkm_server* s) {
   bool refused = false;
   for (size_t qi = 0; qi < s->queue.size();) {
     auto& J = s->queue[qi];
-    if (resident + J->bytes > s->budget) {
+    if (!fits(*J, s->budget - std::min(s->budget, resident))) {
       J->status = KKM_EBUDGET;
       J->error = "the resident models grew: the job no longer fits in the budget";
       J->done = true;
@@ -268,8 +290,13 @@ static kkm_status run_assigns(kkm_server* s, std::vector<std::shared_ptr<Job>>& 
     m = s->models[js[0]->model_id].m;
   }
   const int64_t d = m->d;
-  int64_t R = 0;
-  for (auto& J : js) R += J->M;
+  int64_t R = 0, slices = 0;
+  bool in_parts = false;
+  for (auto& J : js) {
+    R += J->M;
+    slices += (int64_t)J->slices;
+    in_parts |= J->in_parts;
+  }
   if (R == 0) return KKM_OK;
   float* X = nullptr;
   int32_t* lab = nullptr;
@@ -296,7 +323,7 @@ static kkm_status run_assigns(kkm_server* s, std::vector<std::shared_ptr<Job>>& 
     if (e != cudaSuccess) {
       r = fail(e, "cudaMemcpyAsync");
     } else {
-      r = kkm_assign(m, X, R, js[0]->mode, lab, dist, st);
+      r = assign_within(m, X, R, js[0]->mode, lab, dist, st, in_parts ? std::max<int64_t>(slices, 1) : 0);
       if (r != KKM_OK) {
         *err = kkm_last_error();
       } else {
@@ -404,7 +431,7 @@ static kkm_status enqueue(kkm_server* s, std::shared_ptr<Job> J, uint64_t* ticke
   }
   uint64_t resident = 0;
   for (auto& kv : s->models) resident += kv.second.bytes;
-  if (resident + J->bytes > s->budget) {
+  if (!fits(*J, s->budget - std::min(s->budget, resident))) {
     s->refused += 1;
     set_error("job needs about " + std::to_string(J->bytes >> 20) + " MiB of device memory; the budget leaves " +
               std::to_string((s->budget - std::min(s->budget, resident)) >> 20) + " MiB beside the resident models");
@@ -562,7 +589,7 @@ kkm_status kkm_server_submit_assign(kkm_server* s, int32_t model_id, const float
       set_error("unknown model id");
       return KKM_EINVAL;
     }
-    J->bytes = assign_bytes(it->second.m, M, mode);
+    J->bytes = assign_bytes(it->second.m, M, mode, &J->slices, &J->slices_least);
   }
   J->kind = Job::ASSIGN;
   J->model_id = model_id;
