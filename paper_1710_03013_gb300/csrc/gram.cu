@@ -763,7 +763,7 @@ static cudaError_t gram_dispatch(const float* A, int64_t nA, const float* Bm, in
   const int vec_ok = (ldo % 4 == 0) && ((reinterpret_cast<uintptr_t>(out) & 15) == 0);
   const size_t smem = gram_chunked<KIND>() ? kGramChunkSmem : 0;
   if (smem) {
-    static const cudaError_t attr =
+    const cudaError_t attr =
         cudaFuncSetAttribute(gram_tiled_kernel<KIND, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (attr != cudaSuccess) return attr;
   }
@@ -818,7 +818,7 @@ cudaError_t launch_gram_rbf_half(const float* A, int64_t nA, const float* Bm, in
   dim3 grid((unsigned)ceil_div(nB, TB_N), (unsigned)ceil_div(nA, TB_M));
   const int vec_ok = (ldo % 4 == 0) && ((reinterpret_cast<uintptr_t>(out) & 7) == 0) &&
                      ((reinterpret_cast<uintptr_t>(out32) & 15) == 0);
-  static const cudaError_t attr = cudaFuncSetAttribute(
+  const cudaError_t attr = cudaFuncSetAttribute(
       gram_tiled_kernel<DK_RBF, __half>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGramChunkSmem);
   if (attr != cudaSuccess) return attr;
   gram_tiled_kernel<DK_RBF, __half><<<grid, 256, kGramChunkSmem, st>>>(A, (int)nA, Bm, (int)nB, dp, normA, normB,

@@ -479,7 +479,7 @@ static cudaError_t launch_gram_split(const SplitBufs& bP, const float* normP, in
   do {                                                                                                         \
     if (!split_map(&mq, bQ.v, bQ.cap, ks, SP_M) || !split_map(&mp, bP.v, bP.cap, ks, N))                       \
       return cudaErrorInvalidValue;                                                                            \
-    static const cudaError_t attr = cudaFuncSetAttribute(                                                      \
+    const cudaError_t attr = cudaFuncSetAttribute(                                                             \
         gram_split_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SpCfg<N>::kSmem);              \
     if (attr != cudaSuccess) return attr;                                                                      \
     const int64_t tiles = ceil_div(nQ, SP_M) * ceil_div(nP, N);                                                \

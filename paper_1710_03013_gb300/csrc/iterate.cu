@@ -944,7 +944,7 @@ cudaError_t launch_assign(int64_t ldk, int Ni, const Supports& S, const IterStat
   if (smem > (size_t)kAssignMaxDynSmem) return cudaErrorInvalidValue;
   // one attribute for every launch (set once: launches from several host
   // threads never race on it)
-  static const cudaError_t attr =
+  const cudaError_t attr =
       cudaFuncSetAttribute(assign_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAssignMaxDynSmem);
   if (attr != cudaSuccess) return attr;
   const int blocks = (int)ceil_div(Ni, kAssignRows);
@@ -1090,8 +1090,8 @@ cudaError_t launch_assign_multi(const LoopItem* items, const RoundList& L, int n
                                 cudaStream_t st) {
   if (L.n <= 0 || L.cta_off[L.n] <= 0) return cudaSuccess;
   if (nw < 1 || nw > kAssignWarps || smem > kAssignMaxDynSmem || RG < 1) return cudaErrorInvalidValue;
-  static const cudaError_t attr = cudaFuncSetAttribute(assign_multi_kernel,
-                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, kAssignMaxDynSmem);
+  const cudaError_t attr = cudaFuncSetAttribute(assign_multi_kernel,
+                                                cudaFuncAttributeMaxDynamicSharedMemorySize, kAssignMaxDynSmem);
   if (attr != cudaSuccess) return attr;
   return launch_pdl(assign_multi_kernel, dim3((unsigned)L.cta_off[L.n]), dim3(32 * nw), (size_t)smem, st, items, L,
                     RG);
@@ -1712,9 +1712,8 @@ static cudaError_t launch_iterate_t(const T* KT, int64_t ldk, int Ni, const Supp
   size_t smem = 0;
   if (!fused_shape(Ni, S.nL, S.C, (int)sizeof(T), n_sms, &F, &smem)) return cudaErrorInvalidValue;
   if (F.n_cta > I.fused_cap) return cudaErrorInvalidValue;  // gcta / per-CTA slot capacity
-  static const cudaError_t attr = cudaFuncSetAttribute(iterate_fused_kernel<T>,
-                                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                       kFusedMaxDynSmem);
+  const cudaError_t attr = cudaFuncSetAttribute(iterate_fused_kernel<T>,
+                                                cudaFuncAttributeMaxDynamicSharedMemorySize, kFusedMaxDynSmem);
   if (attr != cudaSuccess) return attr;
   // the barrier counter and the fixed-point accumulators start at zero in
   // every launch
@@ -2452,8 +2451,8 @@ cudaError_t launch_kpp_fused_round(const float* X, int dp, int N0, bool linear, 
   const int nb = (int)ceil_div(N0, kKppSamples);
   const size_t smem = (size_t)dp * sizeof(float);
   if (smem > 48 * 1024) {
-    static const cudaError_t e = cudaFuncSetAttribute(kpp_fused_round_kernel,
-                                                      cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    const cudaError_t e = cudaFuncSetAttribute(kpp_fused_round_kernel,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e != cudaSuccess) return e;
     if (smem > 200 * 1024) return cudaErrorInvalidValue;
   }

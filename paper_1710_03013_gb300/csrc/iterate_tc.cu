@@ -1096,7 +1096,7 @@ cudaError_t launch_iterate_tc(const __half* KT, int64_t ldk, int Ni, const Suppo
           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorInvalidValue;
-  static const cudaError_t attr =
+  const cudaError_t attr =
       cudaFuncSetAttribute(iterate_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcMaxDynSmem);
   if (attr != cudaSuccess) return attr;
   // the barrier counter and the fixed-point accumulators start at zero

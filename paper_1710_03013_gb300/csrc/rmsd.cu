@@ -373,7 +373,7 @@ cudaError_t launch_rmsd_exact(const float* A, int64_t nA, const float* Bm, int64
                               const uint8_t* near, int64_t pitch, const int* order, const uint2* units,
                               const unsigned* count, const float4* quat, cudaStream_t st) {
   if (nA <= 0 || nB <= 0) return cudaSuccess;
-  static const cudaError_t attr =
+  const cudaError_t attr =
       cudaFuncSetAttribute(rmsd_exact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RX_SMEM);
   if (attr != cudaSuccess) return attr;
   const int64_t units_max = ceil_div(nA, RX_A) * ceil_div(nB, RX_B);

@@ -287,7 +287,7 @@ cudaError_t launch_rmsd_screen(const __nv_bfloat16* P, int64_t nP, const __nv_bf
     return cudaErrorInvalidValue;
   alignas(64) CUtensorMap mq, mp;
   if (!screen_map(&mq, Q, nQ, dk, 30) || !screen_map(&mp, P, nP, dk, SC_N)) return cudaErrorInvalidValue;
-  static const cudaError_t attr =
+  const cudaError_t attr =
       cudaFuncSetAttribute(rmsd_screen_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SC_SMEM);
   if (attr != cudaSuccess) return attr;
   cudaError_t e = ldo == nQ ? cudaMemsetAsync(out, 0, (size_t)nP * nQ * 4, st)
