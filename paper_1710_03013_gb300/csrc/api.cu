@@ -1137,14 +1137,24 @@ static RescoreArgs rescore_args(const KernelSpec& sp, const BlockBufs& b, int64_
 
 // Scratch of the tensor-core loop's re-score (see RescoreArgs), sized for the
 // largest mini-batch; one loop of a fit runs at a time, so one set serves all.
+// The values it keeps take 4 bytes a kernel value (180 MB for 15,000 x 3,000);
+// when that is not to be had, the loop does without: it reads the block's own
+// FP32 values where they are there (K32; kept by row they are read 6 to 16 %
+// faster, fit included), else forms each again in every iteration.  The sums
+// are the same either way.
 static kkm_status alloc_tc_rescore(Workspace& ws, int64_t Nmax, int64_t nLmax, int C, RescoreArgs* t) {
   t->ldc32 = round_up(nLmax, 32);
   // one allocation, 256-byte aligned parts
   const int64_t have = round_up(Nmax * tc_rescore_blocks((int)nLmax) * 32, 64);
   const int64_t vals = round_up(Nmax * t->ldc32, 64);
-  KKM_TRY(ws.alloc(&t->have, have + vals + ceil_div(Nmax, 128) * tc_rescore_list_words(C, (int)nLmax)));
-  t->C32 = reinterpret_cast<float*>(t->have + have);
-  t->lists = t->have + have + vals;
+  const int64_t lists = ceil_div(Nmax, 128) * tc_rescore_list_words(C, (int)nLmax);
+  uint32_t* at;
+  const kkm_status rc = ws.alloc(&at, have + vals + lists);
+  if (rc == KKM_ENOMEM) return ws.alloc(&t->lists, lists);
+  if (rc != KKM_OK) return rc;
+  t->have = at;
+  t->C32 = reinterpret_cast<float*>(at + have);
+  t->lists = at + have + vals;
   return KKM_OK;
 }
 static void use_tc_rescore(const RescoreArgs& t, RescoreArgs* R) {

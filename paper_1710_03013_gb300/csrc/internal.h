@@ -489,7 +489,8 @@ struct RescoreArgs {
   // scratch of the tensor-core loop: the FP32 values it has formed so far
   // ([sample][ldc32], by the landmark's place), a bit per (sample, landmark)
   // that says so ([sample][tc_rescore_blocks(nL)][32 words]), and per CTA the
-  // clusters' landmark lists and the landmarks' places
+  // clusters' landmark lists and the landmarks' places.  C32 and have may be
+  // null (no memory for them): nothing is then kept
   float* C32 = nullptr;
   int64_t ldc32 = 0;
   uint32_t* have = nullptr;

@@ -166,6 +166,9 @@ __device__ __forceinline__ uint32_t z_offset(int k, int n) {
 // they are bound by the latency of their loads from L2 (no shared memory is
 // left for tiles), which the rows of a group share.
 //
+// Without memory for kept values (R.C32 null) the sums read the block's own FP32
+// values in place, or form each value as they go.
+//
 // MNIST-shaped fit with C = 12 (classes split, a quarter of the rows flagged
 // in each of 120 iterations): 1,024 ms when every iteration formed every
 // value again, a row at a time, against 7.6 ms.
@@ -393,7 +396,7 @@ __device__ __noinline__ unsigned rescore_step(const TcIterShared& sh, const uint
   unsigned full = state & 0xffffu;
   if (state & kRsFresh) {
     const bool first = (state & kRsFirst) != 0;
-    if (first) {  // no value of the tile's rows is there yet
+    if (first && R.C32) {  // no value of the tile's rows is there yet
       const int quads = rows * nblk * 8;
       uint4* const h4 = reinterpret_cast<uint4*>(R.have + (int64_t)i0 * nblk * 32);
       for (int x = et; x < quads; x += kTcEpiWarps * 32) h4[x] = make_uint4(0u, 0u, 0u, 0u);
@@ -406,7 +409,7 @@ __device__ __noinline__ unsigned rescore_step(const TcIterShared& sh, const uint
   cands[q * 32 + lane] = (cand & ~full) ? cand : 0u;
   full |= cand;
   epi_sync();
-  {
+  if (R.C32) {
     unsigned cq[kTcEpiWarps], cmask;
 #pragma unroll
     for (int w = 0; w < kTcEpiWarps; ++w) cq[w] = cands[32 * w + lane];
@@ -421,6 +424,30 @@ __device__ __noinline__ unsigned rescore_step(const TcIterShared& sh, const uint
   for (unsigned todo = __ballot_sync(kFull, cand != 0); todo;) {
     const unsigned cmask = __shfl_sync(kFull, cand, __ffs(todo) - 1);
     unsigned same = __ballot_sync(kFull, cand == cmask) & todo;
+    if (!R.C32) {  // nothing is kept: one row at a time, every value read from the block or formed
+      const int l = __ffs(todo) - 1, i = i0 + q * 32 + l;
+      todo &= todo - 1;
+      for (unsigned c = cmask; c; c &= c - 1) {
+        const int j = __ffs(c) - 1, n = (int)rounds[j];
+        const uint32_t* lj = list + (int64_t)j * nS * 32 + lane;
+        float a = 0.0f;
+        for (int m = 0; m < n; ++m) {
+          const uint32_t e = lj[32 * m];
+          if (e == kRsNone) continue;
+          const int k = (int)(e & 0xffffu);
+          float v;
+          if (R.K32)
+            v = __ldg(R.K32 + (int64_t)k * R.ldk32 + i);
+          else
+            rescore_values<1>(R.XL + (int64_t)k * R.dp, R.nXL[k], L[k], R.Xi + (int64_t)i * R.dp, R.nXi + i, i,
+                              make_uint2(0u, 0u), R.dp, R.neg_scale, &v, 0);
+          a += v;
+        }
+        const float f = warp_sum_f32(a);
+        if (lane == 0) dist[l * kTcN + j] = ks - 2.0f * (f / (float)sh.nj[j]) + sh.ghf[j];
+      }
+      continue;
+    }
     int rl[kRsSumRows];  // their lanes (the last one repeated)
     const float* row_c[kRsSumRows];
 #pragma unroll
@@ -1080,7 +1107,7 @@ cudaError_t launch_iterate_tc(const __half* KT, int64_t ldk, int Ni, const Suppo
   int nstages = 0;
   size_t smem = 0;
   if (!tc_iter_shape(Ni, S.nL, S.C, n_sms, &nstages, &smem)) return cudaErrorInvalidValue;
-  if (R.Xi && I.flag_tau > 0.0f && (!R.lists || !R.C32 || !R.have || R.dp % 8 != 0 || S.nL > 0xffff))
+  if (R.Xi && I.flag_tau > 0.0f && (!R.lists || (R.C32 && !R.have) || R.dp % 8 != 0 || S.nL > 0xffff))
     return cudaErrorInvalidValue;
   if (!I.facc || !I.lm_list || !I.bar || !I.err || (ldk * 2) % 16 != 0 ||
       (reinterpret_cast<uintptr_t>(KT) & 15) != 0)

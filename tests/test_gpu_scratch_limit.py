@@ -1,5 +1,7 @@
-"""Calls that fit beside the scratch of the FFMA block and not beside that of the
-FP16 slices (half as much again): they run, in parts, with the same bits.
+"""Calls that fit in device memory without the scratch that makes them faster:
+kernel blocks beside the scratch of the FFMA block and not beside that of the
+FP16 slices (half as much again), and reduced-precision fits without the re-score's
+kept values.  They run, in parts or without, with the same bits.
 
 Device memory is filled until the free part lies between the two (inputs and
 outputs are there already); no call is made that has to fail.  In a process of
@@ -89,3 +91,63 @@ def test_calls_that_fit_beside_the_ffma_scratch_run(lib):
     done = subprocess.run([sys.executable, "-c", CHILD], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert done.returncode == 0, done.stderr[-2000:]
     assert "both ran in parts" in done.stdout
+
+
+FIT = """
+import ctypes
+import numpy as np
+import torch
+from paper_1710_03013_gb300 import kkm
+from synth import mnist_like
+
+kkm.load()
+rt = ctypes.CDLL("libcudart.so.13")
+pool = ctypes.c_void_p()
+assert rt.cudaDeviceGetDefaultMemPool(ctypes.byref(pool), 0) == 0
+RESERVED, RESERVED_HIGH = 5, 6
+
+
+def trim():
+    torch.cuda.synchronize()
+    assert rt.cudaMemPoolTrimTo(pool, ctypes.c_size_t(0)) == 0
+    torch.cuda.empty_cache()
+
+
+for d, classes, C in ((200, 5, 12), (100, 4, 9)):
+    X, _ = mnist_like(18000, d, classes, problem=d)
+    X = torch.from_numpy(np.ascontiguousarray(X, np.float32)).to("cuda")
+
+    def fit():
+        lab, model = kkm.kkm_fit(X, C, 1, 0.16, "rbf", 0.32 * d ** 0.5, iters=6, seed=3, precision=kkm.KKM_BF16,
+                                 iteration="tc", early_stop=False)
+        return (lab.cpu().numpy(),) + tuple(model.trace())
+
+    fit()
+    trim()
+    zero = ctypes.c_uint64(0)
+    assert rt.cudaMemPoolSetAttribute(pool, RESERVED_HIGH, ctypes.byref(zero)) == 0
+    want = fit()
+    high = ctypes.c_uint64(0)
+    assert rt.cudaMemPoolGetAttribute(pool, RESERVED_HIGH, ctypes.byref(high)) == 0
+    trim()
+    kept = 18000 * 2880 * 4  # the values alone
+    free = high.value - kept // 2
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - free, dtype=torch.uint8, device="cuda")
+    got = fit()
+    again = ctypes.c_uint64(0)
+    assert rt.cudaMemPoolSetAttribute(pool, RESERVED_HIGH, ctypes.byref(zero)) == 0
+    assert rt.cudaMemPoolGetAttribute(pool, RESERVED, ctypes.byref(again)) == 0
+    assert again.value <= free
+    del fill
+    trim()
+    assert want[2][1:].sum() > 0
+    for a, b in zip(got, want):
+        assert np.array_equal(a, b)
+print("both fits ran without kept values")
+"""
+
+
+def test_fits_run_without_the_kept_values(lib):
+    done = subprocess.run([sys.executable, "-c", FIT], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert done.returncode == 0, done.stderr[-2000:]
+    assert "ran without kept values" in done.stdout
