@@ -436,7 +436,8 @@ kkm_status kkm_model_load(const char* path, kkm_model** model_out);
 
 /* kkm_kernel_matrix -- out[a][b] = K(A_a, B_b) for A [nA][d], B [nB][d]
  * (the kernel-block evaluation of Alg. 1 line 3 as a standalone call).
- * out is [nA][nB] float32, device or host.  sigma must be > 0.
+ * out is [nA][nB] float32, device or host.  sigma must be > 0.  With A == Bm and
+ * nA == nB an RBF or linear matrix is symmetric to the last bit.
  * precision KKM_BF16 (RBF and linear kernels) evaluates the product on the
  * tensor cores from BF16-rounded rows with FP32 accumulation; the result is
  * then the kernel of the rounded rows. */

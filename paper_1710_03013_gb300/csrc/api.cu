@@ -2197,6 +2197,8 @@ static kkm_status kernel_matrix_impl(const float* A_in, int64_t nA, const float*
     KKM_TRY(alloc_split(ws, sp, nA, nB, &t));
     bool whole = true;
     KKM_TRY(split_parts(t, sp, sA, nA, sB, nB, o, nB, /*again=*/false, &whole, st, polls));
+    const bool self = A_in == B_in && nA == nB;  // K(A, A) is symmetric to the last bit
+    if (self) KKM_RUN("mirror", st, launch_mirror(o, nA, nB, st));
     KKM_CK(cudaMemcpyAsync(words_h, t.words, sizeof words_h, cudaMemcpyDeviceToHost, st));
     KKM_CK(cudaStreamSynchronize(st));
     tc_err_h = words_h[kSplitErr];

@@ -288,6 +288,8 @@ kkm_status split_wide_pairs(SplitScratch& t, const SplitSide& P, int64_t nP, con
                             int dp, float neg_scale, float* out, int64_t ldo, int n_sms, cudaStream_t st);
 cudaError_t launch_gram_wide(const SplitScratch& t, const SplitSide& P, int64_t nP, const SplitSide& Q, int64_t nQ,
                              int64_t d, int dp, float neg_scale, float* out, int64_t ldo, int n_sms, cudaStream_t st);
+// The lower triangle of a set's matrix with itself from the upper one.
+cudaError_t launch_mirror(float* out, int64_t n, int64_t ldo, cudaStream_t st);
 // Whether kkm_kernel_matrix and kkm_assign take it for an FP32 Gaussian block
 // against nA reference rows of d values: a rule on the references alone, so
 // that a sample's values do not depend on how many samples share the call.  Up

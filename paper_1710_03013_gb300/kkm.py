@@ -647,7 +647,7 @@ def kkm_kernel_matrix(A, B, kind="rbf", sigma=1.0, n_atoms=0, precision=KKM_FP32
     nA, nB = int(A.shape[0]), int(B.shape[0])
     d = int(np.prod(A.shape[1:]))
     ap, ka = _as_input(A, np.float32)
-    bp, kb = _as_input(B, np.float32)
+    bp, kb = (ap, ka) if B is A else _as_input(B, np.float32)
     if _is_cuda(A):
         torch = _torch()
         out = torch.empty((nA, nB), dtype=torch.float32, device=A.device)
