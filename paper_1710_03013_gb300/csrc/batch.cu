@@ -437,8 +437,10 @@ kkm_status loop_executor_run(LoopExecutor* ex, const LoopItem& item, int iters, 
 
 // Default number of concurrent streams for a batch.
 // (32: a fit waits while the work lists run its inner loop, so more fits are
-// in flight than loops; measured on 256 uneven problems: 8 -> 200 ms,
-// 16 -> 177 ms, 32 -> 171 ms, 64 -> 174 ms)
+// in flight than loops; chosen when 256 uneven problems took 200 ms with 8,
+// 177 with 16, 171 with 32 and 174 with 64.  With the present kernels 8 / 12 /
+// 16 / 24 / 32 take 202 / 188 / 183 / 181 / 188 ms on 256 problems, 49 / 46 /
+// 47 / 50 / 60 on 64 and 12 / 13 / 15 / 15 / 15 on 16: fewer would do.)
 constexpr int kBatchStreams = 32;
 constexpr int kBatchMaxStreams = 64;
 

@@ -126,8 +126,7 @@ cudaError_t launch_rmsd_to_bf16(const float* src, int64_t n, int ap, int n_atoms
 // references are reordered so that 16 of them are too: key = the first near
 // sample (references of one state share it; references near nothing sort
 // last), ties by index.
-__global__ void rmsd_near_key_kernel(const uint8_t* __restrict__ near, int64_t pitch, int nA, int nB,
-                                     int* __restrict__ key) {
+__global__ void rmsd_near_key_kernel(const uint8_t* __restrict__ near, int64_t pitch, int nA, int* __restrict__ key) {
   const int lane = threadIdx.x & 31;
   const int a = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (a >= nA) return;
@@ -141,8 +140,7 @@ __global__ void rmsd_near_key_kernel(const uint8_t* __restrict__ near, int64_t p
       const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
       for (int q = 3; q >= 0; --q)
-        if (w[q]) f = (int)(b * 128 + q * 32 + __ffs(w[q]) - 1);
-      if (f >= nB) f = INT_MAX;  // (bytes past the last tile of samples are not written)
+        if (w[q]) f = (int)(b * 128 + q * 32 + __ffs(w[q]) - 1);  // (no bit is set past the last sample)
     }
     first = (int)__reduce_min_sync(kFull, (unsigned)f);
   }
@@ -203,7 +201,7 @@ cudaError_t launch_rmsd_refine_plan(const uint8_t* near, int64_t pitch, int nA, 
   if (pitch % 16 != 0 || (reinterpret_cast<uintptr_t>(near) & 15)) return cudaErrorInvalidValue;
   const cudaError_t e = cudaMemsetAsync(count, 0, sizeof(unsigned), st);
   if (e != cudaSuccess) return e;
-  rmsd_near_key_kernel<<<(unsigned)ceil_div(nA, 8), 256, 0, st>>>(near, pitch, nA, nB, key);
+  rmsd_near_key_kernel<<<(unsigned)ceil_div(nA, 8), 256, 0, st>>>(near, pitch, nA, key);
   if ((size_t)nA * sizeof(int) <= 48 * 1024)
     rmsd_rank_kernel<true><<<(unsigned)ceil_div(nA, 256), 256, (size_t)nA * sizeof(int), st>>>(key, nA, order);
   else
