@@ -444,64 +444,170 @@ gram_tiled_kernel(const float* __restrict__ A, int nA, const float* __restrict__
 // kernel's sums: first the wide references against every sample, then the
 // others against the wide samples, 128 x 128 pairs of the listed rows a tile.
 // The lists are made on the device, so the tiles are counted there and
-// persistent CTAs share them; without wide rows a launch ends at once.  The rows
-// are read where they lie: d and the alignment are the caller's.
+// persistent CTAs share them; without wide rows a launch ends at once.  Few wide
+// rows of a side (kWideThin) are taken 16 to a tile: a tile of 128 x 128 is a
+// chain of 170 us at d = 784 however many of its rows are asked for, one of 16
+// takes 92 us (one reference against 15,013 samples) or 52 (one sample against
+// 3,001 references); at 64 rows the two are equal.  The rows are read where they
+// lie: d and the alignment are the caller's.
+constexpr int kWideThin = 64;
 struct WideSide {
   const float* X;
   int64_t ld;
   const float* norm;
   const int32_t* rows;
-  int vec;  // 16-byte loads
 };
+// The product of a 16 x 128 tile, one row and eight columns to a thread: acc[j]
+// = the same sums of the rows ty x {tx*4+j, 64+tx*4+j}.  load_a is asked of the
+// first 32 threads.  A chunk of 32 products is loaded at a time, the next one
+// while it is computed: a tile of so little work waits for its loads.
+struct ThinShared {
+  float a[2][TB_K * kGramChunkTiles][16];
+  float b[2][TB_K * kGramChunkTiles][TB_N];
+};
+static_assert(sizeof(ThinShared) <= kGramChunkSmem, "in the place of the chunk sums");
+template <typename LA, typename LB>
+__device__ __forceinline__ void ffma_product_thin(const LA& load_a, const LB& load_b, int nk, ThinShared& t,
+                                                  float (&acc)[8]) {
+  const int tid = threadIdx.x, lr = tid >> 1, lk = (tid & 1) << 2, tx = tid & 15, ty = tid >> 4;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 ga[kGramChunkTiles], gb[kGramChunkTiles];
+  auto fetch = [&](int kt0) {
+#pragma unroll
+    for (int q = 0; q < kGramChunkTiles; ++q) {
+      ga[q] = tid < 32 && kt0 + q < nk ? load_a(kt0 + q) : zero;
+      gb[q] = kt0 + q < nk ? load_b(kt0 + q) : zero;
+    }
+  };
+  auto keep = [&](int buf) {
+#pragma unroll
+    for (int q = 0; q < kGramChunkTiles; ++q) {
+      const float av[4] = {ga[q].x, ga[q].y, ga[q].z, ga[q].w}, bv[4] = {gb[q].x, gb[q].y, gb[q].z, gb[q].w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (tid < 32) t.a[buf][q * TB_K + lk + e][lr] = av[e];
+        t.b[buf][q * TB_K + lk + e][lr] = bv[e];
+      }
+    }
+  };
+#pragma unroll
+  for (int j = 0; j < 8; ++j) acc[j] = 0.0f;
+  __syncthreads();  // (the last tile has been read)
+  fetch(0);
+  keep(0);
+  __syncthreads();
+  for (int kt = 0, buf = 0; kt < nk; kt += kGramChunkTiles, buf ^= 1) {
+    const bool more = kt + kGramChunkTiles < nk;
+    if (more) fetch(kt + kGramChunkTiles);
+    float part[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 8
+    for (int k = 0; k < TB_K * kGramChunkTiles; ++k) {
+      const float av = t.a[buf][k][ty];
+      const float4 bl = *reinterpret_cast<const float4*>(&t.b[buf][k][tx * 4]);
+      const float4 bh = *reinterpret_cast<const float4*>(&t.b[buf][k][64 + tx * 4]);
+      const float bv[8] = {bl.x, bl.y, bl.z, bl.w, bh.x, bh.y, bh.z, bh.w};
+#pragma unroll
+      for (int j = 0; j < 8; ++j) part[j] = fmaf(av, bv[j], part[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[j] = kt ? acc[j] + part[j] : part[j];
+    if (more) keep(buf ^ 1);
+    __syncthreads();
+  }
+}
+
+// VEC: both sides take 16-byte loads.
+template <bool VEC>
 __global__ void __launch_bounds__(256, 2)
 gram_wide_kernel(WideSide P, WideSide Q, const int* __restrict__ words, int nP, int nQ, int d, int dp, float neg_scale,
                  float* __restrict__ out, int64_t ldo, int vec_ok) {
   __shared__ __align__(16) TileShared As, Bs;
-  extern __shared__ float chunk_sum[];
+  extern __shared__ float chunk_sum[];  // of a fat tile; a ThinShared for a thin one
   const int wide_p = words[kSplitWideP], clean_p = nP - wide_p, wide_q = words[kSplitWideQ];
-  auto tiles = [](int n) { return (n + TB_M - 1) / TB_M; };
-  const int64_t n1 = (int64_t)tiles(wide_p) * tiles(nQ), n2 = (int64_t)tiles(clean_p) * tiles(wide_q);
   const int tid = threadIdx.x, lr = tid >> 1, lk = (tid & 1) << 2, tx = tid & 15, ty = tid >> 4;
+  auto load = [&](const float* p, int kt) {
+    const int c = kt * TB_K + lk;
+    if constexpr (VEC)
+      return c < d ? __ldg(reinterpret_cast<const float4*>(p + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    return make_float4(c < d ? __ldg(p + c) : 0.f, c + 1 < d ? __ldg(p + c + 1) : 0.f,
+                       c + 2 < d ? __ldg(p + c + 2) : 0.f, c + 3 < d ? __ldg(p + c + 3) : 0.f);
+  };
+  // the lists: wide references, the other references, wide samples
+  auto wide_ref = [&](int a) { return P.rows[nP - 1 - a]; };
+  auto other_ref = [&](int a) { return wide_p ? P.rows[a] : a; };
+  // (rows past a list's end repeat its last one; their outputs are dropped)
+  const bool thin1 = wide_p <= kWideThin, thin2 = wide_q <= kWideThin;
+  const int rows1 = thin1 ? 16 : TB_M, cols1 = (nQ + TB_N - 1) / TB_N;
+  const int64_t n1 = (int64_t)((wide_p + rows1 - 1) / rows1) * cols1;
+  const int cols2 = thin2 ? (clean_p + TB_N - 1) / TB_N : (wide_q + TB_N - 1) / TB_N;
+  const int64_t n2 = (int64_t)(thin2 ? (wide_q + 15) / 16 : (clean_p + TB_M - 1) / TB_M) * cols2;
   for (int64_t t = blockIdx.x; t < n1 + n2; t += gridDim.x) {
-    const bool all = t < n1;  // every sample
-    const int64_t u = all ? t : t - n1;
-    const int tb = tiles(all ? nQ : wide_q);
-    const int a0 = (int)(u / tb) * TB_M, b0 = (int)(u % tb) * TB_N;
-    const int na = all ? wide_p : clean_p, nb = all ? nQ : wide_q;
-    auto row_a = [&](int a) { return (int64_t)(all ? P.rows[nP - 1 - a] : wide_p ? P.rows[a] : a); };
-    auto row_b = [&](int b) { return (int64_t)(all ? b : Q.rows[b]); };
-    // rows past the end repeat the last one; their outputs are dropped
-    const float* const pa = P.X + row_a(min(a0 + lr, na - 1)) * P.ld;
-    const float* const pb = Q.X + row_b(min(b0 + lr, nb - 1)) * Q.ld;
-    auto load = [&](const float* p, int vec, int kt) {
-      const int c = kt * TB_K + lk;
-      if (vec) return c < d ? __ldg(reinterpret_cast<const float4*>(p + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
-      return make_float4(c < d ? __ldg(p + c) : 0.f, c + 1 < d ? __ldg(p + c + 1) : 0.f,
-                         c + 2 < d ? __ldg(p + c + 2) : 0.f, c + 3 < d ? __ldg(p + c + 3) : 0.f);
-    };
+    const bool first = t < n1;
+    const int64_t u = first ? t : t - n1;
+    if (first ? thin1 : thin2) {
+      // 16 wide rows x 128 of the other side
+      const int cols = first ? cols1 : cols2, na = first ? wide_p : wide_q, nb = first ? nQ : clean_p;
+      const int a0 = (int)(u / cols) * 16, b0 = (int)(u % cols) * TB_N;
+      auto row_a = [&](int a) { return first ? wide_ref(a) : Q.rows[a]; };
+      auto row_b = [&](int b) { return first ? b : other_ref(b); };
+      const float* const pa = (first ? P.X : Q.X) + (int64_t)row_a(min(a0 + (lr & 15), na - 1)) * (first ? P.ld : Q.ld);
+      const float* const pb = (first ? Q.X : P.X) + (int64_t)row_b(min(b0 + lr, nb - 1)) * (first ? Q.ld : P.ld);
+      float acc[8];
+      ffma_product_thin([&](int kt) { return load(pa, kt); }, [&](int kt) { return load(pb, kt); }, dp / TB_K,
+                        *reinterpret_cast<ThinShared*>(chunk_sum), acc);
+      const int a = a0 + ty;
+      if (a < na) {
+        const int64_t ra = row_a(a);
+        const float norm_a = (first ? P.norm : Q.norm)[ra];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int b = b0 + (j < 4 ? tx * 4 + j : 64 + tx * 4 + j - 4);
+          if (b < nb) {
+            const int64_t rb = row_b(b);
+            out[first ? ra * ldo + rb : rb * ldo + ra] =
+                gram_epilogue<DK_RBF>(acc[j], norm_a, (first ? Q.norm : P.norm)[rb], false, neg_scale);
+          }
+        }
+      }
+      continue;
+    }
+    // 128 wide references x 128 samples, or 128 other references x 128 wide samples
+    const int cols = first ? cols1 : cols2, na = first ? wide_p : clean_p, nb = first ? nQ : wide_q;
+    const int a0 = (int)(u / cols) * TB_M, b0 = (int)(u % cols) * TB_N;
+    auto row_a = [&](int a) { return first ? wide_ref(a) : other_ref(a); };
+    auto row_b = [&](int b) { return first ? b : Q.rows[b]; };
+    const float* const pa = P.X + (int64_t)row_a(min(a0 + lr, na - 1)) * P.ld;
+    const float* const pb = Q.X + (int64_t)row_b(min(b0 + lr, nb - 1)) * Q.ld;
     float acc[8][8];
-    ffma_product<true>([&](int kt) { return load(pa, P.vec, kt); }, [&](int kt) { return load(pb, Q.vec, kt); },
-                       dp / TB_K, As, Bs, chunk_sum, acc);
+    ffma_product<true>([&](int kt) { return load(pa, kt); }, [&](int kt) { return load(pb, kt); }, dp / TB_K, As, Bs,
+                       chunk_sum, acc);
+    int rb[8];
+    float nb8[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int b = b0 + (j < 4 ? tx * 4 + j : 64 + tx * 4 + j - 4);
+      rb[j] = b < nb ? row_b(b) : -1;
+      nb8[j] = b < nb ? Q.norm[rb[j]] : 0.0f;
+    }
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int a = a0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + i - 4);
       if (a >= na) continue;
       const int64_t ra = row_a(a);
       const float norm_a = P.norm[ra];
+      float* const o = out + ra * ldo;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const int b = b0 + h * 64 + tx * 4;
         float v[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-          v[q] = b + q < nb ? gram_epilogue<DK_RBF>(acc[i][h * 4 + q], norm_a, Q.norm[row_b(b + q)], false, neg_scale)
-                            : 0.0f;
-        if (all && vec_ok && b + 3 < nb) {
-          *reinterpret_cast<float4*>(out + ra * ldo + b) = make_float4(v[0], v[1], v[2], v[3]);
+          v[q] = gram_epilogue<DK_RBF>(acc[i][h * 4 + q], norm_a, nb8[h * 4 + q], false, neg_scale);
+        if (first && vec_ok && rb[h * 4 + 3] >= 0) {
+          *reinterpret_cast<float4*>(o + rb[h * 4]) = make_float4(v[0], v[1], v[2], v[3]);
         } else {
 #pragma unroll
           for (int q = 0; q < 4; ++q)
-            if (b + q < nb) out[ra * ldo + row_b(b + q)] = v[q];
+            if (rb[h * 4 + q] >= 0) o[rb[h * 4 + q]] = v[q];
         }
       }
     }
@@ -511,15 +617,17 @@ cudaError_t launch_gram_wide(const SplitScratch& t, const SplitSide& P, int64_t 
                              int64_t d, int dp, float neg_scale, float* out, int64_t ldo, int n_sms, cudaStream_t st) {
   if (nP <= 0 || nQ <= 0) return cudaSuccess;
   if (dp % TB_K != 0) return cudaErrorInvalidValue;
-  auto side = [&](const SplitSide& s, const SplitBufs& b) {
-    return WideSide{s.X, s.ld, s.norm ? s.norm : b.norm, b.rows, d % 4 == 0 && s.ld % 4 == 0 && aligned16(s.X)};
+  auto side = [](const SplitSide& s, const SplitBufs& b) {
+    return WideSide{s.X, s.ld, s.norm ? s.norm : b.norm, b.rows};
   };
+  const bool vec = d % 4 == 0 && P.ld % 4 == 0 && Q.ld % 4 == 0 && aligned16(P.X) && aligned16(Q.X);
+  auto* const kernel = vec ? gram_wide_kernel<true> : gram_wide_kernel<false>;
   const cudaError_t e =
-      cudaFuncSetAttribute(gram_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGramChunkSmem);
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGramChunkSmem);
   if (e != cudaSuccess) return e;
-  // at most all tiles of either part; two CTAs fit an SM
-  const int64_t most = (ceil_div(nP, TB_M) + 1) * ceil_div(nQ, TB_N);
-  gram_wide_kernel<<<(unsigned)std::min<int64_t>(most, 2 * std::max(n_sms, 1)), 256, kGramChunkSmem, st>>>(
+  // two CTAs fit an SM
+  const int64_t most = (ceil_div(nP, 16) + 1) * (ceil_div(nQ, 16) + 1);
+  kernel<<<(unsigned)std::min<int64_t>(most, 2 * std::max(n_sms, 1)), 256, kGramChunkSmem, st>>>(
       side(P, t.P), side(Q, t.Q), t.words, (int)nP, (int)nQ, (int)d, dp, neg_scale, out, ldo,
       ldo % 4 == 0 && aligned16(out));
   return cudaGetLastError();

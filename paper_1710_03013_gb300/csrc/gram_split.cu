@@ -345,8 +345,10 @@ gram_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
 // times at d = 128).
 // The slices stay at their rows' places (compacted, with the block's rows
 // through a list, a 3,001 x 15,013 x 784 call took 375 instead of 360 us), so
-// a block with wide rows pays for their tensor-core pairs as well: at most the
-// 0.27 ms beside the FFMA sums' 1.57, and nothing when a whole side is wide.
+// a block with wide rows pays for their tensor-core pairs as well, unless a whole
+// side is wide.  That call with wide rows of values like the others' (host wait
+// included): none 0.38 ms, one 0.49, 1 % 0.55, 10 % 0.86, half 1.71, 90 % 2.19,
+// all 1.81; the FFMA kernel alone 1.67.
 struct SplitSource {
   const float* X;
   int64_t ld, n, cap;

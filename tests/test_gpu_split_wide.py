@@ -73,6 +73,15 @@ def test_a_value_depends_on_its_two_rows_alone(lib):
     # the wide rows' values do not depend on the company either
     sub = _matrix(lib, A2[[3, 400] + list(range(40, 180))], B2[[700, 0]], sigma)
     assert np.array_equal(sub[:2], K2[np.ix_([3, 400], [700, 0])])
+    # nor, bit for bit, on how many of them there are (few go 16 to a tile, many 128; 64 is the line)
+    for many in (61, 62, 300):
+        A4, B4 = _widen(A2, range(4, 4 + many), g), _widen(B2, range(100, 100 + 2 * many), g)
+        B4[900:1000] = B2[900:1000]
+        K4 = _matrix(lib, A4, B4, sigma)
+        keep = [0, 700] + list(range(900, 1000))
+        assert np.array_equal(K4[np.ix_([3, 400], keep)], K2[np.ix_([3, 400], keep)])
+        clean = np.setdiff1d(np.arange(350, 500), [400])
+        assert np.array_equal(K4[np.ix_(clean, [0, 700])], K2[np.ix_(clean, [0, 700])])
     # nor on where the rows lie: unaligned rows of an odd pitch
     import torch
     flat = torch.zeros(1 + A2.size, device="cuda:0")
