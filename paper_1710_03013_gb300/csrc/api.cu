@@ -1141,15 +1141,23 @@ static RescoreArgs rescore_args(const KernelSpec& sp, const BlockBufs& b, int64_
 // when that is not to be had, the loop does without: it reads the block's own
 // FP32 values where they are there (K32; kept by row they are read 6 to 16 %
 // faster, fit included), else forms each again in every iteration.  The sums
-// are the same either way.
-static kkm_status alloc_tc_rescore(Workspace& ws, int64_t Nmax, int64_t nLmax, int C, RescoreArgs* t) {
+// are the same either way.  `later`: bytes that have to be left for others.
+static kkm_status alloc_tc_rescore(Workspace& ws, int64_t Nmax, int64_t nLmax, int C, int64_t later, RescoreArgs* t) {
   t->ldc32 = round_up(nLmax, 32);
   // one allocation, 256-byte aligned parts
   const int64_t have = round_up(Nmax * tc_rescore_blocks((int)nLmax) * 32, 64);
   const int64_t vals = round_up(Nmax * t->ldc32, 64);
   const int64_t lists = ceil_div(Nmax, 128) * tc_rescore_list_words(C, (int)nLmax);
-  uint32_t* at;
-  const kkm_status rc = ws.alloc(&at, have + vals + lists);
+  void* room = nullptr;  // held while the scratch is asked for
+  kkm_status rc = KKM_OK;
+  if (later > 0 && cudaMallocAsync(&room, (size_t)later, ws.st) != cudaSuccess) {
+    cudaGetLastError();
+    room = nullptr;
+    rc = KKM_ENOMEM;
+  }
+  uint32_t* at = nullptr;
+  if (rc == KKM_OK) rc = ws.alloc(&at, have + vals + lists);
+  if (room) cudaFreeAsync(room, ws.st);
   if (rc == KKM_ENOMEM) return ws.alloc(&t->lists, lists);
   if (rc != KKM_OK) return rc;
   t->have = at;
@@ -1605,11 +1613,6 @@ static kkm_status fit_impl(const float* X_in, int64_t N, int64_t d, int32_t C, i
   KKM_TRY(alloc_loop(ws, (int)nLmax, C, ldk, trace_cap, &lb, sp.gaussian()));
   Supports& S = lb.S;
   IterState& I = lb.I;
-  RescoreArgs tc_scratch;
-  for (const BatchGeom* g : {&geo.front(), &geo.back()})  // mini-batches come in at most two sizes
-    if (!tc_scratch.lists &&
-        loop_form(opt.iteration, sp, bm, (int)g->Ni, (int)n_landmarks(g->Ni, s), C) == kLoopTc)
-      KKM_TRY(alloc_tc_rescore(ws, Nmax, nLmax, C, &tc_scratch));
   if (from) {
     // the outer loop's state after mini-batch start - 1: medoids, counts, the
     // trace and the displacements so far
@@ -1647,6 +1650,13 @@ static kkm_status fit_impl(const float* X_in, int64_t N, int64_t d, int32_t C, i
       labels_dev = labels_out;
     }
   }
+  // (last, and only beside room for what the end of the fit allocates)
+  const int64_t later = ((int64_t)4 << 20) + (model_out ? 4 * nLmax * sp.dp + 64 * nLmax + 8 * C * (sp.dp + d) : 0);
+  RescoreArgs tc_scratch;
+  for (const BatchGeom* g : {&geo.front(), &geo.back()})  // mini-batches come in at most two sizes
+    if (!tc_scratch.lists &&
+        loop_form(opt.iteration, sp, bm, (int)g->Ni, (int)n_landmarks(g->Ni, s), C) == kLoopTc)
+      KKM_TRY(alloc_tc_rescore(ws, Nmax, nLmax, C, later, &tc_scratch));
   // Feature kernels carry the medoid rows from one mini-batch to the next
   // (the rows after the merge are rows of the mini-batch just done); MD
   // frames are prepared again from X.
@@ -2047,9 +2057,7 @@ static kkm_status assign_impl(const kkm_model* m, const float* Xnew_in, int64_t 
   SplitScratch slices;
   const SplitSide ref{mode == KKM_ASSIGN_SUPPORTS ? m->sup : m->med, sp.dp,
                       mode == KKM_ASSIGN_SUPPORTS ? m->sup_aux : m->med_aux};
-  if (split) {
-    KKM_TRY(alloc_split(ws, sp, rows_ref, std::min(chunk, M), &slices, slice_bytes));
-  } else {
+  if (!split) {
     KKM_TRY(ws.alloc(&Xc, ldm * sp.dp));
     KKM_TRY(ws.alloc(&auxc, ldm));
   }
@@ -2078,6 +2086,8 @@ static kkm_status assign_impl(const kkm_model* m, const float* Xnew_in, int64_t 
     lb.I.ghat_in = m->ghat;
     lb.I.done = bad_d;
   }
+  // (last: what is left decides whether the slices are whole)
+  if (split) KKM_TRY(alloc_split(ws, sp, rows_ref, std::min(chunk, M), &slices, slice_bytes));
   // labels and distances of rows c0 .. c0 + n - 1 from their kernel values
   auto label = [&](int64_t c0, int n) -> kkm_status {
     if (mode == KKM_ASSIGN_SUPPORTS) {
@@ -2339,7 +2349,7 @@ static kkm_status debug_step_impl(const float* Xb_in, int64_t Ni, int64_t d, con
   if (form < 0) return invalid("the iteration form asked for does not apply to this shape");
   if (form == kLoopTc) {
     RescoreArgs t;
-    KKM_TRY(alloc_tc_rescore(ws, Ni, nL, C, &t));
+    KKM_TRY(alloc_tc_rescore(ws, Ni, nL, C, 0, &t));
     use_tc_rescore(t, &R);
   }
   KKM_TRY(inner_loop(bm, b, ldk, (int)Ni, lb.S, lb.I, form, 1, kself, u, mg, fh, gh, 0, R, st));
