@@ -385,7 +385,7 @@ split_rows_kernel(SplitSource P, SplitSource Q, int d, int ks, float least, int*
   }
   top = __reduce_max_sync(kFull, top);
   if (!S.norm) {
-    norm = df_to_float(warp_sum_df(acc));
+    norm = __shfl_sync(kFull, df_to_float(warp_sum_df(acc)), 0);  // one answer for the warp
     if (lane == 0) S.norm_out[row] = norm;
   }
   // scaled maximum in [2^14, 2^15); the exponents stay within the normal range
