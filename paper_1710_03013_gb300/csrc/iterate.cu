@@ -34,6 +34,7 @@
 
 #include "device_common.cuh"
 #include "internal.h"
+#include "smem_opt_in.h"
 
 namespace kkm {
 
@@ -944,8 +945,8 @@ cudaError_t launch_assign(int64_t ldk, int Ni, const Supports& S, const IterStat
   if (smem > (size_t)kAssignMaxDynSmem) return cudaErrorInvalidValue;
   // one attribute for every launch (set once: launches from several host
   // threads never race on it)
-  const cudaError_t attr =
-      cudaFuncSetAttribute(assign_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAssignMaxDynSmem);
+  static std::atomic<uint64_t> done{0};
+  const cudaError_t attr = smem_opt_in(done, reinterpret_cast<const void*>(assign_kernel), kAssignMaxDynSmem);
   if (attr != cudaSuccess) return attr;
   const int blocks = (int)ceil_div(Ni, kAssignRows);
   // a fit's iteration launches: rows per CTA from the tuner (timing samples
@@ -1090,8 +1091,8 @@ cudaError_t launch_assign_multi(const LoopItem* items, const RoundList& L, int n
                                 cudaStream_t st) {
   if (L.n <= 0 || L.cta_off[L.n] <= 0) return cudaSuccess;
   if (nw < 1 || nw > kAssignWarps || smem > kAssignMaxDynSmem || RG < 1) return cudaErrorInvalidValue;
-  const cudaError_t attr = cudaFuncSetAttribute(assign_multi_kernel,
-                                                cudaFuncAttributeMaxDynamicSharedMemorySize, kAssignMaxDynSmem);
+  static std::atomic<uint64_t> done{0};
+  const cudaError_t attr = smem_opt_in(done, reinterpret_cast<const void*>(assign_multi_kernel), kAssignMaxDynSmem);
   if (attr != cudaSuccess) return attr;
   return launch_pdl(assign_multi_kernel, dim3((unsigned)L.cta_off[L.n]), dim3(32 * nw), (size_t)smem, st, items, L,
                     RG);
@@ -2451,8 +2452,8 @@ cudaError_t launch_kpp_fused_round(const float* X, int dp, int N0, bool linear, 
   const int nb = (int)ceil_div(N0, kKppSamples);
   const size_t smem = (size_t)dp * sizeof(float);
   if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(kpp_fused_round_kernel,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    static std::atomic<uint64_t> done{0};
+    const cudaError_t e = smem_opt_in(done, reinterpret_cast<const void*>(kpp_fused_round_kernel), 200 * 1024);
     if (e != cudaSuccess) return e;
     if (smem > 200 * 1024) return cudaErrorInvalidValue;
   }
