@@ -460,7 +460,8 @@ struct WideSide {
 // The product of a 16 x 128 tile, one row and eight columns to a thread: acc[j]
 // = the same sums of the rows ty x {tx*4+j, 64+tx*4+j}.  load_a is asked of the
 // first 32 threads.  A chunk of 32 products is loaded at a time, the next one
-// while it is computed: a tile of so little work waits for its loads.
+// while it is computed; bound by the shared-memory reads (short scoreboard and
+// MIO stalls under ncu).
 struct ThinShared {
   float a[2][TB_K * kGramChunkTiles][16];
   float b[2][TB_K * kGramChunkTiles][TB_N];
