@@ -122,3 +122,19 @@ def test_assign_of_wide_rows(lib, mode, C):
     cost = lib.kkm_cost(model, Q, mode)
     entry = 2.0 ** -21 + 8 * 2.0 ** -24 * 2 * float((X * X).sum(1).max()) / 18.0  # of a kernel value, as above
     assert abs(cost - float(dist.double().sum())) <= 3000 * 2 * entry
+
+
+def test_assign_in_several_chunks(lib):
+    """More rows than one chunk of kernel values holds (22,369 to 6,000 supports): the
+    references' slices and lists are those of the first chunk, the wide samples
+    each chunk's own."""
+    g = np.random.default_rng(4)
+    X, _ = mnist_like(6000 + 50000, 130, 10, problem=4)
+    X = _widen(X, np.nonzero(g.random(len(X)) < 0.02)[0], g)
+    S, Q = _dev(X[:6000]), _dev(X[6000:])
+    _, model = lib.kkm_fit(S, 5, 1, 1.0, "rbf", 3.0, iters=1, seed=1)
+    lab, dist = lib.kkm_assign(model, Q)
+    lab, dist = lab.cpu().numpy(), dist.cpu().numpy()
+    for a, b in ((0, 20000), (20000, 40000), (40000, 50000), (22360, 22380)):
+        la, da = lib.kkm_assign(model, Q[a:b].contiguous())
+        assert np.array_equal(la.cpu().numpy(), lab[a:b]) and np.array_equal(da.cpu().numpy(), dist[a:b])
