@@ -21,7 +21,7 @@
 // What bounds it: the epilogue's instructions, about 300 for 30 pairs (ncu: 0.6
 // issued a cycle and scheduler, tensor pipe 38 % active); with the far test
 // taken out the rest runs in 1.28 ms of the figures below.  10,000 x 10,000
-// frames of 300 atoms: 1.73 ms, 1,250 references x 25,000 samples 0.55 ms.
+// frames of 300 atoms: 1.71 ms, 1,250 references x 25,000 samples 0.55 ms.
 // Before, 2.47 and 0.81 ms: frames in four planes (x, y, z, 0), tiles of 32 x
 // 64 frames (1.6 times the operand bytes and products a pair), eight epilogue
 // warps.  Tried: eight warps here 3.0 ms, twenty 1.77, the regrouping by
@@ -91,6 +91,9 @@ struct ScreenShared {
   int abort_flag;
 };
 
+// LIMITED: waits of `polls` polls, for tests.  A limit in a register instead of a
+// constant costs 1.5 % (1.736 ms against 1.709, 10,000 x 10,000 frames of 300 atoms).
+template <bool LIMITED>
 __global__ void __launch_bounds__(SC_THREADS, 1)
 rmsd_screen_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapP, int nQ, int nP,
                    int dk, const float* __restrict__ gQ, const float* __restrict__ gP, float n_r2_far,
@@ -99,6 +102,7 @@ rmsd_screen_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* const stages = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ ScreenShared sh;
+  const uint32_t limit = LIMITED ? polls : kTcSpinLimit;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tiles_m = (nQ + SC_FQ - 1) / SC_FQ, tiles_n = (nP + SC_FP - 1) / SC_FP;
   const int64_t n_tiles = (int64_t)tiles_m * tiles_n;
@@ -136,7 +140,7 @@ rmsd_screen_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
         int tm, tn;
       screen_tile(t, tiles_m, tiles_n, tm, tn);
         for (int kb = 0; kb < nk; ++kb) {
-          if (!mbar_wait(&sh.empty[s], ph ^ 1u, &sh.abort_flag, polls)) {
+          if (!mbar_wait(&sh.empty[s], ph ^ 1u, &sh.abort_flag, limit)) {
             ok = false;
             break;
           }
@@ -167,14 +171,14 @@ rmsd_screen_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
       const uint32_t idesc = sc_idesc();
       for (int64_t t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++lt) {
         const int buf = lt & 1;
-        if (!mbar_wait(&sh.tempty[buf], ((uint32_t)(lt >> 1) & 1u) ^ 1u, &sh.abort_flag, polls)) {
+        if (!mbar_wait(&sh.tempty[buf], ((uint32_t)(lt >> 1) & 1u) ^ 1u, &sh.abort_flag, limit)) {
           ok = false;
           break;
         }
         tc_fence_after();
         const uint32_t d_tmem = tmem + (uint32_t)(buf * 256);
         for (int kb = 0; kb < nk; ++kb) {
-          if (!mbar_wait(&sh.full[s], ph, &sh.abort_flag, polls)) {
+          if (!mbar_wait(&sh.full[s], ph, &sh.abort_flag, limit)) {
             ok = false;
             break;
           }
@@ -214,7 +218,7 @@ rmsd_screen_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
       const float gy = valid ? gQ[sf] : 0.0f;
       bool ok = true;
       __syncwarp();
-      if (lane == 0) ok = mbar_wait(&sh.tfull[buf], (uint32_t)(lt >> 1) & 1u, &sh.abort_flag, polls);
+      if (lane == 0) ok = mbar_wait(&sh.tfull[buf], (uint32_t)(lt >> 1) & 1u, &sh.abort_flag, limit);
       ok = __shfl_sync(kFull, ok ? 1 : 0, 0) != 0;
       if (!ok) {
         if (lane == 0) {
@@ -287,8 +291,8 @@ cudaError_t launch_rmsd_screen(const __nv_bfloat16* P, int64_t nP, const __nv_bf
     return cudaErrorInvalidValue;
   alignas(64) CUtensorMap mq, mp;
   if (!screen_map(&mq, Q, nQ, dk, 30) || !screen_map(&mp, P, nP, dk, SC_N)) return cudaErrorInvalidValue;
-  const cudaError_t attr =
-      cudaFuncSetAttribute(rmsd_screen_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SC_SMEM);
+  auto* const kernel = polls == kTcSpinLimit ? rmsd_screen_kernel<false> : rmsd_screen_kernel<true>;
+  const cudaError_t attr = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SC_SMEM);
   if (attr != cudaSuccess) return attr;
   cudaError_t e = ldo == nQ ? cudaMemsetAsync(out, 0, (size_t)nP * nQ * 4, st)
                             : cudaMemset2DAsync(out, (size_t)ldo * 4, 0, (size_t)nQ * 4, (size_t)nP, st);
@@ -297,7 +301,7 @@ cudaError_t launch_rmsd_screen(const __nv_bfloat16* P, int64_t nP, const __nv_bf
   // n rmsd^2 at which the kernel value falls to kRmsdRefine
   const float n_r2_far = (log2f(kRmsdRefine) / neg_scale) / (1.0f / (float)n_atoms);
   const int64_t tiles = ceil_div(nQ, SC_FQ) * ceil_div(nP, SC_FP);
-  rmsd_screen_kernel<<<(unsigned)std::min<int64_t>(tiles, std::max(n_sms, 1)), SC_THREADS, SC_SMEM, st>>>(
+  kernel<<<(unsigned)std::min<int64_t>(tiles, std::max(n_sms, 1)), SC_THREADS, SC_SMEM, st>>>(
       mq, mp, (int)nQ, (int)nP, dk, gQ, gP, n_r2_far, quat, ldo, reinterpret_cast<uint32_t*>(near), pitch / 4, err,
       polls);
   return cudaGetLastError();
